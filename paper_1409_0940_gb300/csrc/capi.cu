@@ -1781,16 +1781,17 @@ rff_status sqdiff(rff_admm_t h, const float* a, const float* b, int64_t n, doubl
   return sum_partials(h, out);
 }
 
-// scores S (slots x m_pad) = Z(rows) Wbar, on the handle's training rows or a query batch
+// scores S (slots x m_pad) = Z(rows) Wbar, on the handle's training rows or a query batch;
+// part: part_bytes of scratch (16-byte aligned) for the tensor-core path's partial sums, or null
 rff_status scores_pass(rff_admm_t h, const float* Xrows32, const __half* Xh, const __half* Xl,
-                       int64_t nrows, const int32_t* row_ok, float* out) {
+                       int64_t nrows, const int32_t* row_ok, float* out, float* part, size_t part_bytes) {
   auto& s = *h;
   if (s.tc_scores()) {
     CK(cudaMemsetAsync(s.amax + AMAX_WB, 0, 4, s.st));
     CK(launch_finite_check(s.Wbar, s.fslots * s.mpad, 0, reinterpret_cast<int*>(s.amax + AMAX_FLAG), s.st, s.amax + AMAX_WB));
     CK(launch_transpose_split_f16(s.Wbar, s.fslots, (int)s.mpad, 1, 0, s.WbThi, s.WbTlo, s.fslots, 0, 1.f,
                                   s.amax + AMAX_WB, s.st));
-    CK(tc_predict(tc_view(s), Xh, Xl, nrows, s.WbThi, s.WbTlo, s.amax + AMAX_WB, out));
+    CK(tc_predict(tc_view(s), Xh, Xl, nrows, s.WbThi, s.WbTlo, s.amax + AMAX_WB, out, part, part_bytes));
   } else if (s.tensorsketch()) {
     // the rows' sketches, TS_SCORE_ROWS at a time, then their product with Wbar in FP32
     for (int64_t r0 = 0; r0 < nrows; r0 += TS_SCORE_ROWS) {
@@ -1903,12 +1904,14 @@ rff_status rff_admm_solve(rff_admm_t h, int32_t iters, rff_admm_stats* stats) {
     // blocks keep it): the outer form's product scratch, else the pass-1 partials
     double loss = 0, reg = 0;
     float* sc = s.outer ? s.U32 : s.Rpart;
+    const int64_t sc_elems = s.outer ? 2 * (int64_t)s.C * s.nslots * s.mpad : s.rpart_elems();
     const int64_t chunk = s.outer ? s.nslots
                                   : std::min<int64_t>(s.nslots, std::max<int64_t>(SLOT, s.rpart_elems() / s.mpad / SLOT * SLOT));
     for (int64_t r0 = 0; r0 < s.nslots; r0 += chunk) {
       const int64_t nr = std::min(chunk, s.nslots - r0);
       if ((r = scores_pass(h, s.X32 ? s.X32 + r0 * s.dld : nullptr, s.Xhi ? s.Xhi + r0 * s.dld : nullptr,
-                           s.Xlo ? s.Xlo + r0 * s.dld : nullptr, nr, s.row_of_slot + r0, sc)) != RFF_OK)
+                           s.Xlo ? s.Xlo + r0 * s.dld : nullptr, nr, s.row_of_slot + r0, sc, sc + nr * s.mpad,
+                           (size_t)std::max<int64_t>(0, sc_elems - nr * s.mpad) * 4)) != RFF_OK)
         return r;
       CK(launch_loss_partials(s.p.loss, s.Y + r0 * s.mpad, sc, s.row_of_slot + r0, nr, (int)s.m, (int)s.mpad,
                               s.partials, 1024, s.st));
@@ -2310,13 +2313,24 @@ rff_status rff_admm_predict(rff_admm_t h, const float* Xq, int64_t q, float* sco
   const int64_t chunk = std::min<int64_t>(round_up(q, SLOT), 65536);
   const size_t need = (size_t)chunk * s.d * 4 + (size_t)chunk * s.dld * 4 + (size_t)chunk * s.dld * 2 * 2 +
                       (size_t)chunk * s.mpad * 4 + 4096;
-  rff_status r = ensure_scratch(h, need);
+  // a split batch's partial sums behind them, where the memory is there
+  size_t partb = 0;
+  if (s.tc_scores())
+    for (int64_t nq : {chunk, round_up(q % chunk, SLOT)})
+      partb = std::max(partb, tc_predict_part_bytes(tc_view(s), nq));
+  rff_status r = ensure_scratch(h, need + partb);
+  if (r != RFF_OK && partb) {
+    h->err.clear();
+    partb = 0;
+    r = ensure_scratch(h, need);
+  }
   if (r != RFF_OK) return r;
   float* stage = static_cast<float*>(s.scratch.p);
   float* xq32 = stage + round_up(chunk * s.d, 64);
   __half* xh = reinterpret_cast<__half*>(xq32 + chunk * s.dld);
   __half* xl = xh + chunk * s.dld;
   float* sc = reinterpret_cast<float*>(xl + chunk * s.dld);
+  float* part = partb ? sc + chunk * s.mpad : nullptr;
   const cudaMemcpyKind kin = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   const cudaMemcpyKind kout = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   for (int64_t q0 = 0; q0 < q; q0 += chunk) {
@@ -2336,7 +2350,7 @@ rff_status rff_admm_predict(rff_admm_t h, const float* Xq, int64_t q, float* sco
     CK(launch_gather_rows(stage, s.d, s.d, nullptr, nq, xq32, s.dld, s.st));
     if (s.bias_col >= 0) CK(launch_set_column(xq32, s.dld, nqp, s.bias_col, 1.f, s.st));
     if (s.tc_scores()) CK(launch_split_f16(xq32, nqp * s.dld, s.xscale, xh, xl, s.st));
-    if ((r = scores_pass(h, xq32, xh, xl, nqp, nullptr, sc)) != RFF_OK) return r;
+    if ((r = scores_pass(h, xq32, xh, xl, nqp, nullptr, sc, part, partb)) != RFF_OK) return r;
     CK(cudaMemcpy2DAsync(scores + q0 * s.m, s.m * 4, sc, s.mpad * 4, s.m * 4, nq, kout, s.st));
   }
   CK(cudaStreamSynchronize(s.st));
@@ -2502,7 +2516,7 @@ rff_status predict_into_scratch(rff_admm_t h, const float* Xq, int64_t q, float*
   CK(launch_gather_rows(Xq, s.d, s.d, nullptr, q, xq32, s.dld, s.st));
   if (s.bias_col >= 0) CK(launch_set_column(xq32, s.dld, qp, s.bias_col, 1.f, s.st));
   if (s.tc_scores()) CK(launch_split_f16(xq32, qp * s.dld, s.xscale, xh, xl, s.st));
-  rff_status r = scores_pass(h, xq32, xh, xl, qp, nullptr, sc);
+  rff_status r = scores_pass(h, xq32, xh, xl, qp, nullptr, sc, sc + qp * s.mpad, scratch_bytes - need);
   if (r != RFF_OK) return r;
   CK(cudaMemcpy2DAsync(scores, s.m * 4, sc, s.mpad * 4, s.m * 4, q, cudaMemcpyDeviceToDevice, s.st));
   CK(cudaStreamSynchronize(s.st));

@@ -61,7 +61,8 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t ACC2_COL = 256;         // acc2 with a single acc1 (ZT 0, 1)
 constexpr int MAXG = 64;                    // groups (column blocks) per CTA
 static_assert(COS_SCALE == 128.f, "the epilogues form COS_SCALE cos(.) as cos_rr_pow2<7>");
-constexpr int PRED_GT = 8;                  // feature tiles per scoring group
+constexpr int PRED_GT = 8;                  // scoring: feature tiles per group, at least
+constexpr size_t PRED_PART_BYTES = size_t(64) << 20;   // the most a split batch may take for its groups' sums
 
 // Ring geometry.  KC = K elements per ring stage: 64 (128-byte rows, 128-byte
 // swizzle, 64 KB stages) or 32 (64-byte rows, 64-byte swizzle, 32 KB stages, so
@@ -128,6 +129,7 @@ struct TcArgs {
   __half *zt_hi, *zt_lo;                    // write mode: Z^T as an FP16 hi/lo split (ld ldo), or null
   float zt_scale;                           // its power-of-two scale
   int bias_in_mma;                          // 1: b already in the product (column of ones)
+  int pred_gt, pred_part;                   // scoring: feature tiles per group; 1: every group's sums apart
   const uint8_t* bmask;                     // passes 1 and 2: active blocks (R x C), or null
   int m_shared;                             // pass 1: the chained operand's rows 0..m_pad serve every block
   int* err;
@@ -135,6 +137,12 @@ struct TcArgs {
 };
 
 using namespace tc5;
+
+// *p += v, added in the L2 without a reply: a thread's additions to one address keep its order
+__device__ __forceinline__ void red_add_v4(float4* p, float4 v) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
 
 // ------------------------------------------------------------------ shared state
 template <int NS, int MG = MAXG>
@@ -290,16 +298,18 @@ __device__ void plan_work(const TcArgs& a, SH& sh, uint32_t rank, const CtaPos& 
     a_row0 = pos.x * 128;
     m_y = 0;
     {
-      // scoring: the features in groups of up to PRED_GT tiles, each group accumulated in
-      // a fresh acc2 and added into the output rows in FP32 (the tensor cores' accumulator
-      // rounds toward zero at every accumulation; shorter chains keep its bias small)
+      // scoring: the features in groups of pred_gt tiles, each group accumulated in a fresh acc2
+      // and added into the output rows in FP32 in the groups' order (the tensor cores'
+      // accumulator rounds toward zero at every accumulation; shorter chains keep its bias
+      // small).  Split y of nsplit takes its share of the groups and, like every CTA of a split
+      // batch, writes each group's sums apart (pred_part) for k_pred_reduce to add in that order
       const bool phantom = a_row0 >= a.a_rows;
       const int ntiles = (int)(a.fslots / 128);
-      const int gt = max(PRED_GT, (int)ceil_div(ntiles, SH::maxg));
-      for (int t0 = 0; t0 < ntiles && ng < SH::maxg; t0 += gt) {
-        sh.g_b0[ng] = (int64_t)t0 * 128;
-        sh.g_nt[ng] = min(gt, ntiles - t0);
-        sh.g_out[ng] = phantom ? nullptr : a.out + a_row0 * a.mpad;
+      const int ngr = (int)ceil_div(ntiles, a.pred_gt);
+      for (int g = pos.y * ngr / a.nsplit; g < (pos.y + 1) * ngr / a.nsplit && ng < SH::maxg; ++g) {
+        sh.g_b0[ng] = (int64_t)g * a.pred_gt * 128;
+        sh.g_nt[ng] = min(a.pred_gt, ntiles - g * a.pred_gt);
+        sh.g_out[ng] = phantom ? nullptr : a.out + (a.pred_part ? g * a.out_block_stride : 0) + a_row0 * a.mpad;
         ++ng;
       }
     }
@@ -713,6 +723,7 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
             // undo the FP16 scales of Z (COS_SCALE) and of the chained operand, apply sqrt(2/D)
             const float sc = a.scale / COS_SCALE * (a.m_amax ? f16_inv_scale(__uint_as_float(*a.m_amax)) : 1.f);
             float omx = 0.f;
+            const bool add_rows = a.mode == MODE_PREDICT && !a.pred_part && g > 0;
             for (int c = 0; c < half; c += 8) {
               uint32_t r8[8];
               tmem_ld8(tmem + lane_addr + A2 + c0 + c, r8);
@@ -723,12 +734,10 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
               float4 v1 = make_float4(sc * __uint_as_float(r8[4]), sc * __uint_as_float(r8[5]),
                                       sc * __uint_as_float(r8[6]), sc * __uint_as_float(r8[7]));
               const bool in = RFF_SPAN(orow + c0 + c - a.out, 8, a.out_elems);
-              if (in && a.mode == MODE_PREDICT && g > 0) {   // this CTA wrote these rows for group g-1
-                const float4 p0 = dst[0], p1 = dst[1];
-                v0 = make_float4(p0.x + v0.x, p0.y + v0.y, p0.z + v0.z, p0.w + v0.w);
-                v1 = make_float4(p1.x + v1.x, p1.y + v1.y, p1.z + v1.z, p1.w + v1.w);
-              }
-              if (in) {
+              if (in && add_rows) {   // this thread wrote these values for the groups before
+                red_add_v4(dst, v0);
+                red_add_v4(dst + 1, v1);
+              } else if (in) {
                 dst[0] = v0;
                 dst[1] = v1;
               }
@@ -1129,6 +1138,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
             float* orow = sh.g_out[g] + (int64_t)row * a.mpad;
             const float sc = a.scale / COS_SCALE * (a.m_amax ? f16_inv_scale(__uint_as_float(*a.m_amax)) : 1.f);
             float omx = 0.f;
+            const bool add_rows = a.mode == MODE_PREDICT && !a.pred_part && g > 0;
             for (int c = 0; c < half; c += 8) {
               uint32_t r8[8];
               tmem_ld8(tmem + lane_addr + W_A2 + c0 + c, r8);
@@ -1139,12 +1149,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
               float4 v1 = make_float4(sc * __uint_as_float(r8[4]), sc * __uint_as_float(r8[5]),
                                       sc * __uint_as_float(r8[6]), sc * __uint_as_float(r8[7]));
               const bool in = RFF_SPAN(orow + c0 + c - a.out, 8, a.out_elems);
-              if (in && a.mode == MODE_PREDICT && g > 0) {
-                const float4 p0 = dst[0], p1 = dst[1];
-                v0 = make_float4(p0.x + v0.x, p0.y + v0.y, p0.z + v0.z, p0.w + v0.w);
-                v1 = make_float4(p1.x + v1.x, p1.y + v1.y, p1.z + v1.z, p1.w + v1.w);
-              }
-              if (in) {
+              if (in && add_rows) {
+                red_add_v4(dst, v0);
+                red_add_v4(dst + 1, v1);
+              } else if (in) {
                 dst[0] = v0;
                 dst[1] = v1;
               }
@@ -1578,19 +1586,45 @@ cudaError_t tc_multi_launch(const TcMulti* t, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t tc_predict(const TcView& v, const __half* Xh, const __half* Xl, int64_t nrows,
-                       const __half* Mhi, const __half* Mlo, const unsigned* m_amax, float* out) {
-  if (nrows <= 0) return cudaSuccess;
-  if (nrows % 128) return cudaErrorInvalidValue;
+namespace {
+// out[e] = part[0][e] + part[1][e] + ... in the groups' order (n4 float4 each, stride n4)
+__global__ void __launch_bounds__(128) k_pred_reduce(const float4* __restrict__ part, int ngroups, int64_t n4,
+                                                     float4* __restrict__ out) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= n4) return;
+  float4 s = part[t];
+#pragma unroll 8
+  for (int g = 1; g < ngroups; ++g) {
+    const float4 v = part[g * n4 + t];
+    s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
+  }
+  out[t] = s;
+}
+
+// feature tiles per scoring group: PRED_GT, or as many as keep the groups within a CTA's plan
+int pred_group(const TcView& v) {
+  return (int)std::max<int64_t>(PRED_GT, ceil_div(v.fslots / 128, view_zt(v) == 3 ? W_MAXG : MAXG));
+}
+
+// one scoring launch over all nrows rows; ns > 1: the groups dealt out over ns CTAs per row
+// tile, every group's sums written apart into `part` and added up afterwards
+cudaError_t predict_rows(const TcView& v, const __half* Xh, const __half* Xl, int64_t nrows, const __half* Mhi,
+                         const __half* Mlo, const unsigned* m_amax, float* out, int gt, int ns, float* part) {
   TcArgs a;
   cudaError_t e = common_args(v, a);
   if (e != cudaSuccess) return e;
+  const int ntiles = (int)(v.fslots / 128);
   a.mode = MODE_PREDICT;
   a.a_rows = nrows;
   a.a_ok = nullptr;
   a.b_ok = v.feat_ok;
-  a.out = out;
-  a.out_elems = nrows * v.mpad;
+  a.pred_gt = gt;
+  a.pred_part = ns > 1 ? 1 : 0;
+  a.nsplit = ns;
+  const int ngr = (int)ceil_div(ntiles, a.pred_gt);
+  a.out = ns > 1 ? part : out;
+  a.out_block_stride = nrows * v.mpad;
+  a.out_elems = nrows * v.mpad * (ns > 1 ? ngr : 1);
   a.m_amax = m_amax;
   const int cg = view_cg(v), brows = view_brows(v), mrows = view_mrows(v);
   if ((e = make_map(&a.tA_hi, Xh, v.dld, nrows, v.dld, 128, view_kc(v))) != cudaSuccess) return e;
@@ -1599,7 +1633,55 @@ cudaError_t tc_predict(const TcView& v, const __half* Xh, const __half* Xl, int6
   if ((e = make_map(&a.tB_lo, v.Glo, v.dld, v.fslots, v.dld, brows, view_kc(v))) != cudaSuccess) return e;
   if ((e = make_map(&a.tM_hi, Mhi, v.fslots, v.mpad, v.fslots, mrows, view_kc(v))) != cudaSuccess) return e;
   if ((e = make_map(&a.tM_lo, Mlo, v.fslots, v.mpad, v.fslots, mrows, view_kc(v))) != cudaSuccess) return e;
-  return launch(a, dim3((unsigned)tile_grid(v, nrows / 128)), v.st, view_kc(v), view_zt(v), cg);
+  e = launch(a, dim3((unsigned)tile_grid(v, nrows / 128), (unsigned)ns), v.st, view_kc(v), view_zt(v), cg);
+  if (e != cudaSuccess || ns == 1) return e;
+  const int64_t n4 = nrows * v.mpad / 4;
+  k_pred_reduce<<<(unsigned)ceil_div(n4, 128), 128, 0, v.st>>>(reinterpret_cast<const float4*>(part), ngr, n4,
+                                                               reinterpret_cast<float4*>(out));
+  return cudaGetLastError();
+}
+}  // namespace
+
+// A CTA takes 128 rows through every feature tile, so a batch of few rows, or the last part of
+// one that does not fill the SMs once more, leaves most of them idle: the row tiles past the
+// last whole wave are split over the feature groups, into the ns that ends soonest (waves times
+// groups per CTA).  The sums and their order are the same either way, so a row's scores do not
+// depend on the batch it came in.  Measured at D = 16,384, d = 440, m = 147 (kernel time):
+// 1000 rows 852 us on 8 CTAs -> 55 us on 128 and 5 us for their sums; a call of one row 1.05 ms
+// -> 0.17 ms, of 1000 rows 1.03 -> 0.20 ms.
+cudaError_t tc_predict(const TcView& v, const __half* Xh, const __half* Xl, int64_t nrows,
+                       const __half* Mhi, const __half* Mlo, const unsigned* m_amax, float* out, float* part,
+                       size_t part_bytes) {
+  if (nrows <= 0) return cudaSuccess;
+  if (nrows % 128) return cudaErrorInvalidValue;
+  const int64_t tiles = nrows / 128, nsm = sm_count();
+  const int gt = pred_group(v);
+  const int64_t ngr = ceil_div(v.fslots / 128, gt);
+  const int64_t full = tiles / nsm * nsm, rest = tiles - full;
+  int64_t best = 1;
+  if (view_cg(v) == 1 && rest > 0 && part &&
+      (size_t)ngr * rest * 128 * v.mpad * sizeof(float) <= std::min(part_bytes, PRED_PART_BYTES)) {
+    int64_t cost = ceil_div(rest, nsm) * ngr;
+    for (int64_t ns = 2; ns <= ngr; ++ns) {
+      const int64_t c = ceil_div(rest * ns, nsm) * ceil_div(ngr, ns);
+      if (c < cost) {
+        cost = c;
+        best = ns;
+      }
+    }
+  }
+  if (best == 1) return predict_rows(v, Xh, Xl, nrows, Mhi, Mlo, m_amax, out, gt, 1, nullptr);
+  const int64_t r0 = full * 128;
+  cudaError_t e = full ? predict_rows(v, Xh, Xl, r0, Mhi, Mlo, m_amax, out, gt, 1, nullptr) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  return predict_rows(v, Xh + r0 * v.dld, Xl + r0 * v.dld, nrows - r0, Mhi, Mlo, m_amax, out + r0 * v.mpad,
+                      gt, (int)best, part);
+}
+
+size_t tc_predict_part_bytes(const TcView& v, int64_t nrows) {
+  const int64_t rest = nrows / 128 % sm_count(), ngr = ceil_div(v.fslots / 128, pred_group(v));
+  const size_t need = (size_t)ngr * rest * 128 * v.mpad * sizeof(float);
+  return ngr > 1 && view_cg(v) == 1 && need <= PRED_PART_BYTES ? need : 0;
 }
 
 RFF_CHECK_UNIT(tc)

@@ -60,13 +60,17 @@ cudaError_t tc_multi_create(const TcView* views, int n, int which, float* const*
                             TcMulti** out);
 cudaError_t tc_multi_launch(const TcMulti* t, cudaStream_t st);
 void tc_multi_destroy(TcMulti* t);
-// Scores for a query block (nrows slot-padded rows of split X) against M (mpad x fslots hi/lo).
 // Error word of the tensor-core kernels (bounded waits that gave up); reads and clears it.
 // Synchronises the device.  0 = no error.
 int tc_error_word();
+// Scores for a query block (nrows slot-padded rows of split X) against M (mpad x fslots hi/lo);
+// part: part_bytes of scratch, or null.
 cudaError_t tc_predict(const TcView& v, const __half* Xh, const __half* Xl, int64_t nrows,
-                       const __half* Mhi, const __half* Mlo, const unsigned* m_amax, float* out);
-
+                       const __half* Mhi, const __half* Mlo, const unsigned* m_amax, float* out, float* part,
+                       size_t part_bytes);
+// Bytes of `part` that let tc_predict split a batch of nrows (slot-padded) rows over the SMs; with
+// less, or none (0 when it would not split), the batch is scored unsplit, to the same bits.
+size_t tc_predict_part_bytes(const TcView& v, int64_t nrows);
 
 // Split streaming GEMM on the tensor cores, one CTA per job:
 //   out[job.out + r*mpad + c] = out_scale / s_B sum_k A[job.a_row + r][job.a_k0 + k] B[job.b_row + c][job.b_k0 + k]

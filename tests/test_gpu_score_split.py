@@ -1,0 +1,40 @@
+"""Scoring of small batches, which the tensor-core path splits over the feature groups.
+
+The groups' sums are added in one order whether one CTA takes them all or several share them, so
+a row's scores are the same bits in any batch; against the float64 features they stay within the
+split path's tolerance.  Sizes: one row, one less and one more than a 128-row tile, a whole wave
+of the SMs plus a remainder; one feature group, three (the last of them short), and thirteen.
+"""
+import numpy as np
+import pytest
+
+from oracle import rff as orff
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rff():
+    import paper_1409_0940_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("prec", ["split_bf16", "cached_z"])
+@pytest.mark.parametrize("D,C", [(100, 1), (2500, 2), (13000, 3)])
+def test_scores_do_not_depend_on_the_batch(rff, prec, D, C):
+    rng = np.random.default_rng(3)
+    d, m, n = 21, 3, 400
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    Y = np.sign(rng.standard_normal((n, m))).astype(np.float32)
+    s = rff.Solver(loss="squared", reg="l2", lam=1e-3, sigma=4.0, rho=1.0, D=D, R=1, C=C, seed=9, m=m, prec=prec)
+    s.set_data(X, Y)
+    s.solve(2)
+    W = s.weights()
+    Q = rng.standard_normal((160 * 128 + 45, d)).astype(np.float32)
+    full = s.predict(Q)
+    for q in (1, 127, 129, 1000, 152 * 128 + 1):
+        assert np.array_equal(s.predict(np.ascontiguousarray(Q[:q])), full[:q])
+    rows = np.r_[0:50, Q.shape[0] - 50:Q.shape[0]]
+    ref = orff.features_block(Q[rows], 9, 4.0, D, 0, D) @ W.astype(np.float64)
+    assert np.linalg.norm(full[rows] - ref) <= 1e-4 * np.linalg.norm(ref)
+    s.close()
