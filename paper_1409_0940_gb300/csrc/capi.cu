@@ -1904,7 +1904,9 @@ rff_status rff_admm_solve(rff_admm_t h, int32_t iters, rff_admm_stats* stats) {
     // blocks keep it): the outer form's product scratch, else the pass-1 partials
     double loss = 0, reg = 0;
     float* sc = s.outer ? s.U32 : s.Rpart;
-    const int64_t sc_elems = s.outer ? 2 * (int64_t)s.C * s.nslots * s.mpad : s.rpart_elems();
+    // (only the first half of U32, which every iteration writes whole: the second, y, keeps zeros in
+    // its padding rows that pass 1 relies on)
+    const int64_t sc_elems = s.outer ? (int64_t)s.C * s.nslots * s.mpad : s.rpart_elems();
     const int64_t chunk = s.outer ? s.nslots
                                   : std::min<int64_t>(s.nslots, std::max<int64_t>(SLOT, s.rpart_elems() / s.mpad / SLOT * SLOT));
     for (int64_t r0 = 0; r0 < s.nslots; r0 += chunk) {
