@@ -433,6 +433,7 @@ void compute_geometry(rff_admm_s& s, int64_t n, int64_t d) {
 // hi/lo pair and 128 x 256 tiles of Z^T Z over 512-row pieces of K, GRAM_GROUP pieces per
 // launch, their partial tiles summed into H in FP64.
 constexpr int GRAM_KCH = 512, GRAM_GROUP = 16;
+constexpr size_t OUTER_ZT_BYTES = size_t(256) << 20;   // outer form: the most Z^T formed at once
 
 int64_t tc_gram_tiles(int64_t smax, std::vector<int2>* out = nullptr) {
   const int64_t spad = round_up(smax, 256);
@@ -462,7 +463,7 @@ size_t setup_bytes(const rff_admm_s& s, int64_t batch) {
   int64_t smax = 0;
   for (int j = 0; j < s.C; ++j) smax = std::max(smax, s.col_size[j]);
   const int64_t chunk_rows = std::min<int64_t>(32768, round_up(*std::max_element(s.row_size.begin(), s.row_size.end()), SLOT));
-  const size_t t = (size_t)batch * smax * smax * 8 * 2 + (size_t)chunk_rows * smax * 4 +
+  const size_t t = (size_t)batch * smax * smax * 8 * 2 + (size_t)chunk_rows * round_up(smax, SLOT) * 4 +
                    factor_scratch_bytes((int)batch, (int)smax) + (size_t)batch * 4 + 4096 +
                    (tc_gram(s) ? tc_gram_bytes(chunk_rows, smax) : 0);
   // the cached-Z precision forms Z in the same scratch first, in row chunks of ~256 MB
@@ -1180,15 +1181,23 @@ rff_status setup_factors(rff_admm_t h) {
   CK(cudaMemGetInfo(&fr, &tot));
   const size_t per_block = (size_t)fmax * fmax * 8 * 2;
   const int64_t chunk_rows = std::min<int64_t>(32768, round_up(nmax, SLOT));
-  // outer form: Z_ij in chunks of feature columns, each transposed for the Gram kernel
-  const int64_t chunk_feat = std::min<int64_t>(2048, round_up(smax, SLOT));
-  const size_t zbytes = (s.outer ? (size_t)nmax * chunk_feat * 4 * 2 : (size_t)chunk_rows * smax * 4) +
-                        (tc_gram(s) ? tc_gram_bytes(chunk_rows, smax) : 0);
   size_t budget = (size_t)(fr * 0.6);
   if (s.mem_limit) {
     const size_t ws = working_set_bytes(s);
     budget = std::min(budget, s.mem_limit > ws ? s.mem_limit - ws : (size_t)0);
   }
+  // outer form: Z^T in chunks of features, over as many row blocks at once as OUTER_ZT_BYTES (or an
+  // eighth of the memory left) holds: a chunk of one block of 625 rows gives the 152 SMs 5 tiles
+  // of work for the regeneration and 30 for the Gram (512 launches of each, 243 ms, on the
+  // 20k x 32,768 workload at 32 x 8; in 16 launches of each, 30 ms)
+  const int64_t chunk_feat = std::min<int64_t>(2048, round_up(smax, SLOT));
+  const int64_t smax_pad = round_up(smax, SLOT);
+  const int64_t zt_blocks = std::max<int64_t>(
+      1, std::min<int64_t>(s.R, (int64_t)(std::min<size_t>(OUTER_ZT_BYTES, budget / 8) /
+                                          ((size_t)round_up(nmax, SLOT) * chunk_feat * 4))));
+  const size_t zbytes = (s.outer ? (size_t)zt_blocks * round_up(nmax, SLOT) * chunk_feat * 4
+                                 : (size_t)chunk_rows * smax_pad * 4) +
+                        (tc_gram(s) ? tc_gram_bytes(chunk_rows, smax) : 0);
   budget = budget > zbytes + (256u << 20) ? budget - zbytes - (256u << 20) : 0;
   int64_t batch = std::max<int64_t>(1, std::min<int64_t>(nblocks, (int64_t)(budget / std::max<size_t>(per_block + factor_scratch_bytes(1, (int)fmax), 1))));
   size_t need = (size_t)batch * per_block + zbytes + factor_scratch_bytes((int)batch, (int)fmax) + (size_t)batch * 4 + 4096;
@@ -1203,10 +1212,9 @@ rff_status setup_factors(rff_admm_t h) {
   double* H64 = reinterpret_cast<double*>(base);
   double* Q64 = H64 + batch * fmax * fmax;
   float* Zc = reinterpret_cast<float*>(Q64 + batch * fmax * fmax);
-  float* Zt = Zc + (s.outer ? nmax * chunk_feat : 0);   // transposed chunk (outer form)
   // tensor-core Gram buffers after the row chunk, on a 256-byte boundary (tc_gram_bytes keeps 1 KB of slack)
   char* gbase = reinterpret_cast<char*>(
-      round_up((uintptr_t)(reinterpret_cast<char*>(Zc) + (size_t)chunk_rows * smax * 4), (uintptr_t)256));
+      round_up((uintptr_t)(reinterpret_cast<char*>(Zc) + (size_t)chunk_rows * smax_pad * 4), (uintptr_t)256));
   int32_t* info = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(Zc) + zbytes);
   void* fscr = reinterpret_cast<char*>(info) + round_up(batch * 4, 256);
 
@@ -1216,6 +1224,7 @@ rff_status setup_factors(rff_admm_t h) {
     const int64_t nb = std::min(batch, nblocks - b0);
     std::vector<MatJob> jobs;
     CK(cudaMemsetAsync(info, 0, nb * 4, s.st));
+    CK(cudaMemsetAsync(H64, 0, (size_t)nb * fmax * fmax * 8, s.st));
     for (int64_t bb = 0; bb < nb; ++bb) {
       const int64_t blk = b0 + bb;
       const int i = (int)(blk / s.C), j = (int)(blk % s.C);
@@ -1223,25 +1232,12 @@ rff_status setup_factors(rff_admm_t h) {
       const int64_t fd = s.outer ? ni : sj;
       double* Hb = H64 + bb * fmax * fmax;
       double* Qb = Q64 + bb * fmax * fmax;
-      CK(cudaMemsetAsync(Hb, 0, fd * fd * 8, s.st));
-      // outer form: H = I + Z Z^T accumulated over feature chunks (the rows of Z^T)
-      for (int64_t f0 = 0; s.outer && f0 < sj; f0 += chunk_feat) {
-        const int64_t nf = std::min(chunk_feat, sj - f0);
-        if (s.split_path()) {
-          CK(tc_write_z(tc_view(s), s.row_slot[i], ni, s.col_slot[j] + f0, nf, Zc, nf));
-        } else {
-          ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)s.dld, s.bias, scale, s.row_of_slot, s.feat_of_slot,
-                   s.row_slot[i], ni, s.col_slot[j] + f0, nf, Zc, nf, s.p.feature_map};
-          CK(launch_write_z_simt(za, s.st));
-        }
-        CK(launch_transpose_f32(Zc, ni, nf, Zt, ni, s.st));
-        CK(launch_gram_f32_to_f64(Zt, ni, nf, ni, Hb, ni, s.st));
-      }
+      jobs.push_back(MatJob{Hb, fd, (int)fd, Qb, fd, info + bb});
       for (int64_t r = 0; !s.outer && r < s.row_size[i]; r += chunk_rows) {
         const int64_t nr = std::min(chunk_rows, s.row_size[i] - r);
         if (s.split_path() && getenv("RFF_DIAG_SIMT_GRAM")) {
-          CK(tc_write_z(tc_view(s), s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, sj));
-          CK(launch_gram_f32_to_f64(Zc, sj, nr, sj, Hb, sj, s.st));
+          CK(tc_write_z(tc_view(s), s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, smax_pad));
+          CK(launch_gram_f32_to_f64(Zc, smax_pad, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
           continue;
         }
         if (tc_gram(s)) {   // Z^T's split written by the regeneration itself, or the stored one
@@ -1253,25 +1249,43 @@ rff_status setup_factors(rff_admm_t h) {
         }
         // FP32 precision: Z on the SIMT pipes, its Gram from FP32 products with float-float sums
         ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)s.dld, s.bias, scale, s.row_of_slot, s.feat_of_slot,
-                 s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, sj, s.p.feature_map};
+                 s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, smax_pad, s.p.feature_map, 0};
         CK(launch_write_z_simt(za, s.st));
-        CK(launch_gram_f32_to_f64(Zc, sj, nr, sj, Hb, sj, s.st));
+        CK(launch_gram_f32_to_f64(Zc, smax_pad, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
       }
-      CK(launch_add_identity_and_mirror(Hb, fd, fd, s.st));
-      CK(cudaMemsetAsync(Qb, 0, fd * fd * 8, s.st));
-      CK(launch_set_diag(Qb, fd, fd, 1.0, s.st));
-      jobs.push_back(MatJob{Hb, fd, (int)fd, Qb, fd, info + bb});
     }
+    // outer form: H = I + Z Z^T accumulated over feature chunks (the rows of Z^T); the batch's row
+    // blocks of column block j, zt_blocks of them at a time
+    for (int j = 0; s.outer && j < s.C; ++j) {
+      const int64_t i_lo = ceil_div(std::max<int64_t>(0, b0 - j), s.C), i_end = ceil_div(b0 + nb - j, s.C);
+      for (int64_t i0 = i_lo; i0 < i_end; i0 += zt_blocks) {
+        const int64_t i1 = std::min(i0 + zt_blocks, i_end), w0 = s.row_slot[i0];
+        const int64_t wn = s.row_slot[i1 - 1] + round_up(s.row_size[i1 - 1], SLOT) - w0;
+        for (int64_t f0 = 0; f0 < s.col_size[j]; f0 += chunk_feat) {
+          const int64_t nf = std::min(chunk_feat, s.col_size[j] - f0);
+          if (s.split_path()) {
+            CK(tc_write_z(tc_view(s), w0, wn, s.col_slot[j] + f0, nf, Zc, wn, 1));
+          } else {
+            ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)s.dld, s.bias, scale, s.row_of_slot, s.feat_of_slot,
+                     w0, wn, s.col_slot[j] + f0, nf, Zc, wn, s.p.feature_map, 1};
+            CK(launch_write_z_simt(za, s.st));
+          }
+          CK(launch_gram_f32_to_f64(Zc, wn, nf, s.d_row_slot + i0, s.d_row_size + i0, nmax, (int)(i1 - i0),
+                                    H64 + (i0 * s.C + j - b0) * fmax * fmax, (int64_t)s.C * fmax * fmax, s.st));
+        }
+      }
+    }
+    CK(launch_factor_init(jobs, s.st));
     // Q is stored to 24 bits (FP32, or three BF16 pieces): updates that keep 40 bits of every
     // operand leave it within cond(H) 2^-40 (about 2e-9 at cond 2.3e3), far inside that
     CK(factor_and_invert_f64(jobs, true, fscr, s.st, true, 40));
-    for (int64_t bb = 0; bb < nb; ++bb) {
-      const int64_t blk = b0 + bb;
-      const int64_t fd = s.outer ? s.row_size[blk / s.C] : s.col_size[blk % s.C];
-      if (s.split_path() && !s.outer)
-        CK(launch_split3_q(Q64 + bb * fmax * fmax, (int)fd, s.ldq, s.qrow[blk], s.Q1, s.Q2, s.Q3, s.st));
-      else
-        CK(launch_convert_f64_f32(Q64 + bb * fmax * fmax, s.Q32 + s.foff[blk], fd * fd, s.st));
+    if (s.split_path() && !s.outer) {
+      for (int64_t bb = 0; bb < nb; ++bb)
+        CK(launch_split3_q(Q64 + bb * fmax * fmax, jobs[bb].s, s.ldq, s.qrow[b0 + bb], s.Q1, s.Q2, s.Q3, s.st));
+    } else {
+      std::vector<float*> dst(nb);
+      for (int64_t bb = 0; bb < nb; ++bb) dst[bb] = s.Q32 + s.foff[b0 + bb];
+      CK(launch_convert_factors(jobs, dst.data(), s.st));
     }
     std::vector<int32_t> hinfo(nb);
     CK(cudaMemcpyAsync(hinfo.data(), info, nb * 4, cudaMemcpyDeviceToHost, s.st));

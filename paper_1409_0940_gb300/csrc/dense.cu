@@ -302,10 +302,15 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
 // 2^-44 relative per entry.
 constexpr int GR_M = 128, GR_N = 64, GR_K = 32;
 
-__global__ void __launch_bounds__(256) k_gram_tile(const float* __restrict__ Z, int64_t ldz, int64_t n, int64_t s,
-                                                   double* __restrict__ H, int64_t ldh) {
+__global__ void __launch_bounds__(256) k_gram_tile(const float* __restrict__ Zall, int64_t ldz, int64_t n,
+                                                   const int64_t* __restrict__ slot,
+                                                   const int64_t* __restrict__ size, int64_t s_one,
+                                                   double* __restrict__ Hall, int64_t h_stride) {
   const int64_t a0 = (int64_t)blockIdx.x * GR_M, b0 = (int64_t)blockIdx.y * GR_N;
-  if (b0 > a0 + GR_M - 1) return;   // wholly above the diagonal: the mirror fills it
+  const int64_t s = size ? size[blockIdx.z] : s_one, ldh = s;
+  const float* Z = Zall + (slot ? slot[blockIdx.z] - slot[0] : 0);
+  double* H = Hall + blockIdx.z * h_stride;
+  if (a0 >= s || b0 > a0 + GR_M - 1) return;   // past this matrix, or wholly above the diagonal
   __shared__ __align__(16) float As[2][GR_K][GR_M];
   __shared__ __align__(16) float Bs[2][GR_K][GR_N];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -460,14 +465,6 @@ __global__ void k_zero_strict_upper(double* A, int64_t s) {
   if (t % s > t / s) A[t] = 0.0;
 }
 
-__global__ void k_add_identity_and_mirror(double* H, int64_t ldh, int64_t s) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= s * s) return;
-  const int64_t r = t / s, c = t % s;
-  if (c > r) H[r * ldh + c] = H[c * ldh + r];
-  else if (c == r) H[r * ldh + c] += 1.0;
-}
-
 }  // namespace
 
 cudaError_t launch_gemm_f32_nn(const GemmDesc* descs_dev, int nbatch, int maxM, int maxN, float alpha, float beta,
@@ -512,11 +509,11 @@ cudaError_t launch_to_pairs(const GemmDesc* descs_dev, int nbatch, int maxM, int
   return cudaGetLastError();
 }
 
-cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, int64_t s, double* H, int64_t ldh,
-                                   cudaStream_t st) {
-  if (n <= 0 || s <= 0) return cudaSuccess;
-  dim3 grid((unsigned)ceil_div(s, GR_M), (unsigned)ceil_div(s, GR_N));
-  k_gram_tile<<<grid, 256, 0, st>>>(Z, ldz, n, s, H, ldh);
+cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, const int64_t* slot, const int64_t* size,
+                                   int64_t s_max, int nb, double* H, int64_t h_stride, cudaStream_t st) {
+  if (n <= 0 || s_max <= 0 || nb <= 0) return cudaSuccess;
+  dim3 grid((unsigned)ceil_div(s_max, GR_M), (unsigned)ceil_div(s_max, GR_N), (unsigned)nb);
+  k_gram_tile<<<grid, 256, 0, st>>>(Z, ldz, n, slot, size, s_max, H, h_stride);
   return cudaGetLastError();
 }
 
@@ -524,12 +521,6 @@ cudaError_t launch_zero_strict_upper(double* A, int64_t s, int nbatch, cudaStrea
   for (int b = 0; b < nbatch; ++b) {
     k_zero_strict_upper<<<(unsigned)ceil_div(s * s, 256), 256, 0, st>>>(A + (size_t)b * s * s, s);
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_add_identity_and_mirror(double* H, int64_t ldh, int64_t s, cudaStream_t st) {
-  if (s <= 0) return cudaSuccess;
-  k_add_identity_and_mirror<<<(unsigned)ceil_div(s * s, 256), 256, 0, st>>>(H, ldh, s);
   return cudaGetLastError();
 }
 
@@ -546,18 +537,104 @@ cudaError_t launch_potrf_diag(const DiagJob* jobs_dev, int njobs, int kcol, cuda
 //   L Y = I:       Y_k = L_kk^-1 B_k;  B_i -= L_ik Y_k   (i > k)
 //   L^T Q = Y:     Q_k = L_kk^-T Y_k;  Y_i -= L_ki^T Q_k (i < k)
 // Descriptors live in `dev_scratch` (>= factor_scratch_bytes bytes).
-// Q[r][c] = Q[c][r] for c > r (the upper triangle from the lower)
-__global__ void k_mirror_lower(double* __restrict__ Q, int64_t ld, int64_t s) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= s * s) return;
-  const int64_t r = t / s, c = t % s;
-  if (c > r) Q[r * ld + c] = Q[c * ld + r];
+// Kernels over the matrices of a batch take up to MAT_BATCH jobs by value (one launch instead of
+// one per matrix: 256 blocks of order 625 took 1280 launches of ~3 us for what these do in 24).
+constexpr int MAT_BATCH = 64;
+struct MatBatch {
+  double* A[MAT_BATCH];   // the matrix, or the source
+  void* D[MAT_BATCH];     // the second matrix, or the destination
+  int64_t ld[MAT_BATCH];
+  int s[MAT_BATCH];
+};
+
+template <typename Fill, typename Launch>
+static cudaError_t over_batches(const std::vector<MatJob>& jobs, Fill&& fill, Launch&& launch) {
+  for (size_t b0 = 0; b0 < jobs.size(); b0 += MAT_BATCH) {
+    const int nb = (int)std::min<size_t>(MAT_BATCH, jobs.size() - b0);
+    MatBatch mb;
+    int smax = 0;
+    for (int b = 0; b < nb; ++b) {
+      fill(mb, b, b0 + b);
+      smax = std::max(smax, mb.s[b]);
+    }
+    if (smax <= 0) continue;
+    launch(mb, nb, smax);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-cudaError_t launch_mirror_lower(double* Q, int64_t ld, int64_t s, cudaStream_t st) {
-  if (s <= 1) return cudaSuccess;
-  k_mirror_lower<<<(unsigned)ceil_div(s * s, 256), 256, 0, st>>>(Q, ld, s);
-  return cudaGetLastError();
+// 32 x 32 tiles of the strict lower triangle and the diagonal, through shared memory so that both
+// the reads and the writes run along rows
+__global__ void __launch_bounds__(256) k_mirror_lower(const __grid_constant__ MatBatch mb) {
+  const int s = mb.s[blockIdx.z], r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+  if (r0 >= s || c0 > r0) return;
+  double* Q = mb.A[blockIdx.z];
+  const int64_t ld = mb.ld[blockIdx.z];
+  __shared__ double t[32][33];
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  for (int y = ty; y < 32; y += 8)
+    if (r0 + y < s && c0 + tx < s) t[y][tx] = Q[(int64_t)(r0 + y) * ld + c0 + tx];
+  __syncthreads();
+  for (int y = ty; y < 32; y += 8)   // element (c0 + y, r0 + tx) from (r0 + tx, c0 + y)
+    if (c0 + y < s && r0 + tx < s && r0 + tx > c0 + y) Q[(int64_t)(c0 + y) * ld + r0 + tx] = t[tx][y];
+}
+
+cudaError_t launch_mirror_lower(const std::vector<MatJob>& jobs, cudaStream_t st) {
+  return over_batches(
+      jobs,
+      [&](MatBatch& mb, int b, size_t k) {
+        mb.A[b] = jobs[k].Q;
+        mb.D[b] = nullptr;
+        mb.ld[b] = jobs[k].ldq;
+        mb.s[b] = jobs[k].Q ? jobs[k].s : 0;
+      },
+      [&](const MatBatch& mb, int nb, int smax) {
+        const unsigned g = (unsigned)ceil_div(smax, 32);
+        k_mirror_lower<<<dim3(g, g, (unsigned)nb), 256, 0, st>>>(mb);
+      });
+}
+
+__global__ void k_factor_init(const __grid_constant__ MatBatch mb) {
+  const int64_t s = mb.s[blockIdx.y], t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= s * s) return;
+  const int64_t r = t / s, c = t % s;
+  static_cast<double*>(mb.D[blockIdx.y])[t] = r == c ? 1.0 : 0.0;
+  if (r == c) mb.A[blockIdx.y][r * mb.ld[blockIdx.y] + r] += 1.0;
+}
+
+cudaError_t launch_factor_init(const std::vector<MatJob>& jobs, cudaStream_t st) {
+  return over_batches(
+      jobs,
+      [&](MatBatch& mb, int b, size_t k) {
+        mb.A[b] = jobs[k].A;
+        mb.D[b] = jobs[k].Q;   // ldq = s
+        mb.ld[b] = jobs[k].ld;
+        mb.s[b] = jobs[k].s;
+      },
+      [&](const MatBatch& mb, int nb, int smax) {
+        k_factor_init<<<dim3((unsigned)ceil_div((int64_t)smax * smax, 256), (unsigned)nb), 256, 0, st>>>(mb);
+      });
+}
+
+__global__ void k_convert_factors(const __grid_constant__ MatBatch mb) {
+  const int64_t s = mb.s[blockIdx.y], t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t < s * s) static_cast<float*>(mb.D[blockIdx.y])[t] = (float)mb.A[blockIdx.y][t];
+}
+
+cudaError_t launch_convert_factors(const std::vector<MatJob>& jobs, float* const* dst, cudaStream_t st) {
+  return over_batches(
+      jobs,
+      [&](MatBatch& mb, int b, size_t k) {
+        mb.A[b] = jobs[k].Q;
+        mb.D[b] = dst[k];
+        mb.ld[b] = jobs[k].ldq;
+        mb.s[b] = jobs[k].s;
+      },
+      [&](const MatBatch& mb, int nb, int smax) {
+        k_convert_factors<<<dim3((unsigned)ceil_div((int64_t)smax * smax, 256), (unsigned)nb), 256, 0, st>>>(mb);
+      });
 }
 
 // descriptor phases of the blocked factorisation: 0 panel, 1 trailing update, 2-3 forward
@@ -719,9 +796,7 @@ cudaError_t factor_and_invert_f64(const std::vector<MatJob>& jobs, bool invert, 
       if ((e = upd(5, k, c0, c0, 1, 0, 0)) != cudaSuccess) return e;
     }
   }
-  for (const auto& J : jobs)
-    if ((e = launch_mirror_lower(J.Q, J.ldq, J.s, st)) != cudaSuccess) return e;
-  return cudaSuccess;
+  return launch_mirror_lower(jobs, st);
 }
 
 }  // namespace rff

@@ -598,23 +598,6 @@ __global__ void k_outer_update(float* __restrict__ Op, const float* __restrict__
   Op[t] += U[e] + y[t];
 }
 
-// dst[c][r] = src[r][c] (src rows x cols, dst ld dld)
-__global__ void k_transpose_f32(const float* __restrict__ src, int64_t rows, int64_t cols, float* __restrict__ dst,
-                                int64_t dld) {
-  __shared__ float tile[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32, c0 = (int64_t)blockIdx.y * 32;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int rr = ty; rr < 32; rr += 8) {
-    const int64_t r = r0 + rr, c = c0 + tx;
-    tile[rr][tx] = (r < rows && c < cols) ? src[r * cols + c] : 0.f;
-  }
-  __syncthreads();
-  for (int cc = ty; cc < 32; cc += 8) {
-    const int64_t c = c0 + cc, r = r0 + tx;
-    if (c < cols && r < rows) dst[c * dld + r] = tile[tx][cc];
-  }
-}
-
 // Double-float arithmetic on the FP32 pipes (this part's FP64 pipe runs at 1/64 of the FP32
 // rate): Knuth's TwoSum and Dekker's Fast2Sum, every operation rounded on its own.
 struct FF {
@@ -801,11 +784,6 @@ __global__ void __launch_bounds__(256) k_reg_sum(int reg, const float* __restric
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
-__global__ void k_f64_to_f32(const double* __restrict__ s, float* __restrict__ d, int64_t n) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e < n) d[e] = (float)s[e];
-}
-
 // flag |= 1 for a NaN/Inf entry; with pm1, flag |= 2 for an entry outside {-1, +1}
 // flag |= 1 for NaN/Inf, 2 for a value other than +-1 (pm1); maxbits = max |x| of the
 // finite values as float bits (unsigned order equals float order for x >= 0)
@@ -826,11 +804,6 @@ __global__ void k_finite(const float* __restrict__ x, int64_t n, int pm1, int* _
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0 && mx > 0.f) atomicMax(maxbits, __float_as_uint(mx));
   }
-}
-
-__global__ void k_set_diag(double* __restrict__ A, int64_t ld, int64_t s, double v) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < s) A[t * ld + t] = v;
 }
 
 inline unsigned nblk(int64_t n, int bs = 256) { return (unsigned)ceil_div(n, bs); }
@@ -961,14 +934,6 @@ cudaError_t launch_outer_update(float* Op, const float* U, const float* y, int64
   return cudaGetLastError();
 }
 
-cudaError_t launch_transpose_f32(const float* src, int64_t rows, int64_t cols, float* dst, int64_t dld,
-                                 cudaStream_t st) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  dim3 grid((unsigned)ceil_div(rows, 32), (unsigned)ceil_div(cols, 32));
-  k_transpose_f32<<<grid, 256, 0, st>>>(src, rows, cols, dst, dld);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_avg_dual(const float* W, const float* What, int R, int64_t nfe, float* Wbar, float* mu,
                             float* muij, cudaStream_t st) {
   k_avg_dual<<<nblk(nfe), 256, 0, st>>>(W, What, R, nfe, Wbar, mu, muij);
@@ -1009,12 +974,6 @@ cudaError_t launch_loss_partials(int loss, const float* Y, const float* S, const
 cudaError_t launch_reg_partials(int reg, const float* W, int64_t n, double* partials, int nblocks, cudaStream_t st,
                                 const float* w, int ncol) {
   k_reg_sum<<<nblocks, 256, 0, st>>>(reg, W, n, w, ncol > 0 ? ncol : 1, partials);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_convert_f64_f32(const double* src, float* dst, int64_t n, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  k_f64_to_f32<<<nblk(n), 256, 0, st>>>(src, dst, n);
   return cudaGetLastError();
 }
 
@@ -1105,12 +1064,6 @@ __global__ void k_argmax_rows(const float* __restrict__ S, int64_t q, int m, int
 cudaError_t launch_argmax_rows(const float* scores, int64_t q, int m, int64_t ld, int32_t* labels, cudaStream_t st) {
   if (q <= 0) return cudaSuccess;
   k_argmax_rows<<<nblk(q * 32), 256, 0, st>>>(scores, q, m, ld, labels);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_set_diag(double* A, int64_t ld, int64_t s, double v, cudaStream_t st) {
-  if (s <= 0) return cudaSuccess;
-  k_set_diag<<<nblk(s), 256, 0, st>>>(A, ld, s, v);
   return cudaGetLastError();
 }
 

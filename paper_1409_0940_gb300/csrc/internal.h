@@ -92,6 +92,7 @@ struct ZArgs {
   float* out;
   int64_t ldo;
   int map;                  // as PassArgs::map
+  int trans;                // 1: out holds Z^T (nf x nr)
 };
 
 // philox.cu
@@ -152,9 +153,13 @@ cudaError_t launch_gemm_df_pairs(const GemmDesc* descs_dev, int nbatch, int maxM
                                  double alpha, double beta, int lower_only, cudaStream_t st);
 // D (float pairs, ld ldd) = A (FP64, ld lda), M x N per descriptor
 cudaError_t launch_to_pairs(const GemmDesc* descs_dev, int nbatch, int maxM, int maxN, cudaStream_t st);
-// Gram: D(f64) = beta*D + Z^T Z over rows, Z float32 (n x s, ld), FP32 products, FP64 accumulation
-cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, int64_t s, double* H, int64_t ldh,
-                                   cudaStream_t st);
+// Gram: H_b (FP64, s_b x s_b, ld s_b; 128 x 128 tiles on or below the diagonal) += A_b^T A_b for the
+// nb matrices A_b = Z[0..n) x [slot[b] - slot[0], + size[b]) (FP32, row-major, ld ldz), H_b h_stride
+// apart; slot and size on the device (slots are multiples of 128), s_max the largest size; or
+// one matrix with slot = size = null, s = s_max.  FP32 products, float-float sums.  ldz % 4 == 0
+// and Z holds round_up(s, 128) columns per matrix (those past s_b are read, not used)
+cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, const int64_t* slot, const int64_t* size,
+                                   int64_t s_max, int nb, double* H, int64_t h_stride, cudaStream_t st);
 struct DiagJob {   // one matrix of a batched factorisation
   double* A;       // matrix base (s x s, leading dimension ld)
   int64_t ld;
@@ -163,7 +168,6 @@ struct DiagJob {   // one matrix of a batched factorisation
   int32_t* info;   // first failing column + 1, or untouched
 };
 cudaError_t launch_potrf_diag(const DiagJob* jobs_dev, int njobs, int kcol, cudaStream_t st);
-cudaError_t launch_add_identity_and_mirror(double* H, int64_t ldh, int64_t s, cudaStream_t st);
 cudaError_t launch_zero_strict_upper(double* A, int64_t s, int nbatch, cudaStream_t st);
 struct MatJob {    // host description of one matrix to factor (and invert)
   double* A;       // in: SPD matrix; out: lower Cholesky factor
@@ -173,13 +177,18 @@ struct MatJob {    // host description of one matrix to factor (and invert)
   int64_t ldq;
   int32_t* info;   // device int32, zero on entry
 };
+// H += I on the diagonal and Q = I for every job (A = H)
+cudaError_t launch_factor_init(const std::vector<MatJob>& jobs, cudaStream_t st);
+// dst[b] (FP32, s x s) = jobs[b].Q (ld s)
+cudaError_t launch_convert_factors(const std::vector<MatJob>& jobs, float* const* dst, cudaStream_t st);
 size_t factor_scratch_bytes(int njobs, int smax);
 // blocked Cholesky (and inverse); double_float selects the double-float GEMM for the block
 // updates under RFF_FACTOR=df (the 64 x 64 diagonal factorisations stay FP64); oz_bits: the
 // leading bits of every update operand the tensor-core updates keep (48 or 40)
 cudaError_t factor_and_invert_f64(const std::vector<MatJob>& jobs, bool invert, void* dev_scratch, cudaStream_t st,
                                   bool double_float = false, int oz_bits = 48);
-cudaError_t launch_mirror_lower(double* Q, int64_t ld, int64_t s, cudaStream_t st);
+// Q[r][c] = Q[c][r] for c > r, every job with a Q
+cudaError_t launch_mirror_lower(const std::vector<MatJob>& jobs, cudaStream_t st);
 
 // ozaki.cu: the same factorisation with the block updates on the tensor cores (error-free
 // slices of the FP64 operands); factor_and_invert_f64 calls it unless RFF_FACTOR=df
@@ -253,9 +262,6 @@ cudaError_t launch_outer_residual(float* u, const float* Op, const float* U, int
 //   O'_ij += U_i + y_ij for the active blocks (bmask per row block i, column block j; null: all)
 cudaError_t launch_outer_update(float* Op, const float* U, const float* y, int64_t nslots, int mpad, int R, int C,
                                 const int64_t* d_row_slot, const uint8_t* bmask, cudaStream_t st);
-// dst[c][r] = src[r][c]
-cudaError_t launch_transpose_f32(const float* src, int64_t rows, int64_t cols, float* dst, int64_t dld,
-                                 cudaStream_t st);
 cudaError_t launch_avg_dual(const float* W, const float* What, int R, int64_t nfe, float* Wbar, float* mu,
                             float* muij, cudaStream_t st);
 // hi/lo FP16 split of src^T scaled by f16_scale(*amax) (amax non-null) or by scale
@@ -271,11 +277,9 @@ cudaError_t launch_loss_partials(int loss, const float* Y, const float* S, const
                                  int m, int mpad, double* partials, int nblocks, cudaStream_t st);
 cudaError_t launch_reg_partials(int reg, const float* W, int64_t n, double* partials, int nblocks, cudaStream_t st,
                                 const float* w = nullptr, int ncol = 1);
-cudaError_t launch_convert_f64_f32(const double* src, float* dst, int64_t n, cudaStream_t st);
 // flag |= 1 for NaN/Inf; pm1 = 1: |= 2 for a value other than +-1; pm1 = 2: |= 4 for a negative value
 cudaError_t launch_finite_check(const float* x, int64_t n, int pm1, int* flag, cudaStream_t st,
                                 unsigned* maxbits = nullptr);
-cudaError_t launch_set_diag(double* A, int64_t ld, int64_t s, double v, cudaStream_t st);
 // H (FP64, ld ldh) += the sum over nchunk partial tiles (FP32, 128 x 256 each, chunk-major)
 // of the 128 x 256 tiles listed in tiles (first row, first column); entries at or below the
 // diagonal of the s x s matrix only; the chunks (at most 8) are added in order in FP64

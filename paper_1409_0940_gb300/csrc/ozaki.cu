@@ -709,9 +709,7 @@ cudaError_t factor_and_invert_sliced(const std::vector<MatJob>& jobs, bool inver
     if ((e = run(OZ_BA, k, 64, ncol, 0, 0, 0)) != cudaSuccess) return e;
     if ((e = run(OZ_BB, k, c0, c0, 1, 1, 1)) != cudaSuccess) return e;
   }
-  for (const auto& J : jobs)
-    if (J.Q && (e = launch_mirror_lower(J.Q, J.ldq, J.s, st)) != cudaSuccess) return e;
-  return cudaSuccess;
+  return launch_mirror_lower(jobs, st);
 }
 
 }  // namespace

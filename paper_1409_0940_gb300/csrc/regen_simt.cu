@@ -293,6 +293,19 @@ __global__ void __launch_bounds__(NT, 1) k_write_z_simt(ZArgs p) {
   }
 }
 
+// the same into Z^T (nf x nr, leading dimension ldo)
+__global__ void __launch_bounds__(NT, 1) k_write_zt_simt(ZArgs p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SimtSmem& sm = *reinterpret_cast<SimtSmem*>(smem_raw);
+  const int64_t a0 = p.r0 + (int64_t)blockIdx.x * BM, b0 = p.f0 + (int64_t)blockIdx.y * BN;
+  tile_z(sm, p.X, p.ldx, a0, p.Gt, p.ldg, b0, p.K, p.bias, false, p.scale, p.row_ok, p.feat_ok, p.map);
+  for (int t = threadIdx.x; t < BM * BN; t += NT) {
+    const int r = t % BM, c = t / BM;
+    const int64_t gr = a0 - p.r0 + r, gc = b0 - p.f0 + c;
+    if (gr < p.nr && gc < p.nf) p.out[gc * p.ldo + gr] = sm.ZsT[c][r];
+  }
+}
+
 template <int MQ>
 cudaError_t launch_pass_mq(int which, const PassArgs& p, dim3 grid, cudaStream_t st) {
   const size_t smem = sizeof(SimtSmem) + (size_t)BN * p.mpad * sizeof(float);
@@ -336,9 +349,14 @@ cudaError_t launch_write_z_simt(const ZArgs& p, cudaStream_t st) {
   if (p.nr <= 0 || p.nf <= 0) return cudaSuccess;
   if (p.K % BK) return cudaErrorInvalidValue;
   const size_t smem = sizeof(SimtSmem);
-  cudaFuncSetAttribute(k_write_z_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   dim3 grid((unsigned)ceil_div(p.nr, BM), (unsigned)ceil_div(p.nf, BN));
-  k_write_z_simt<<<grid, NT, smem, st>>>(p);
+  if (p.trans) {
+    cudaFuncSetAttribute(k_write_zt_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_write_zt_simt<<<grid, NT, smem, st>>>(p);
+  } else {
+    cudaFuncSetAttribute(k_write_z_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_write_z_simt<<<grid, NT, smem, st>>>(p);
+  }
   return cudaGetLastError();
 }
 

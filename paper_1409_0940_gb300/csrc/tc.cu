@@ -130,6 +130,7 @@ struct TcArgs {
   float zt_scale;                           // its power-of-two scale
   int bias_in_mma;                          // 1: b already in the product (column of ones)
   int pred_gt, pred_part;                   // scoring: feature tiles per group; 1: every group's sums apart
+  int wz_trans;                             // write mode: out holds Z^T (ld ldo) instead of Z
   const uint8_t* bmask;                     // passes 1 and 2: active blocks (R x C), or null
   int m_shared;                             // pass 1: the chained operand's rows 0..m_pad serve every block
   int* err;
@@ -346,12 +347,14 @@ __device__ void plan_work(const TcArgs& a, SH& sh, uint32_t rank, const CtaPos& 
                             : a.out + ((int64_t)split * a.R + i) * a.out_block_stride + a_row0 * a.mpad;
       ng = 1;
     }
-  } else {  // materialisation window
+  } else {  // materialisation window: split y of nsplit takes its share of the feature tiles
+    const int ntiles = (int)ceil_div(a.wz_nf, 128);
+    const int t0 = pos.y * ntiles / a.nsplit, t1 = (pos.y + 1) * ntiles / a.nsplit;
     a_row0 = a.wz_r0 + pos.x * 128;
-    sh.g_b0[0] = a.wz_f0;
-    sh.g_nt[0] = (int)ceil_div(a.wz_nf, 128);
+    sh.g_b0[0] = a.wz_f0 + (int64_t)t0 * 128;
+    sh.g_nt[0] = t1 - t0;
     sh.g_out[0] = nullptr;
-    ng = 1;
+    ng = t1 > t0 ? 1 : 0;
   }
   if (a.mode != MODE_PASS2)
     for (int g = 0; g < ng; ++g) {
@@ -656,10 +659,12 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
               }
             }
           } else if (r < a.wz_nr) {
+            // FP32 Z^T (each store of a warp fills 32 consecutive elements of a row) or Z
+            const int64_t rs = a.wz_trans ? 1 : a.ldo, fs = a.wz_trans ? a.ldo : 1;
 #pragma unroll
             for (int c = 0; c < 64; ++c) {
               const int64_t f = bslot + colbase + c - a.wz_f0;
-              if (f < a.wz_nf && RFF_IN(r * a.ldo + f, a.out_elems)) a.out[r * a.ldo + f] = a.scale * z[c];
+              if (f < a.wz_nf && RFF_IN(r * rs + f * fs, a.out_elems)) a.out[r * rs + f * fs] = a.scale * z[c];
             }
           }
           continue;
@@ -1372,9 +1377,19 @@ int tc_error_word() {
 }
 
 namespace {
-cudaError_t write_z(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float* out, __half* zt_hi,
-                    __half* zt_lo, float zt_scale, int64_t ldo) {
+// One write-mode launch.  A CTA takes 128 rows through its share of the window's feature tiles:
+// the tiles are split into as many shares as end soonest (waves of CTAs times tiles per CTA,
+// half a tile for a CTA's start).  A window of few row tiles would otherwise leave most SMs
+// idle (625 rows x 2048 features, d = 784: 300 us on 5 CTAs).  Nothing is chained, so acc1 is
+// double-buffered (ZT = 2) and shared memory holds three ring stages.
+cudaError_t write_z(const TcView& view, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float* out, int trans,
+                    __half* zt_hi, __half* zt_lo, float zt_scale, int64_t ldo) {
   if (nr <= 0 || nf <= 0) return cudaSuccess;
+  TcView v = view;
+  v.kc = 64;
+  v.zt = 2;
+  v.cg = 1;
+  v.mpad = 16;   // no chained product: any m_pad may take this geometry
   TcArgs a;
   cudaError_t e = common_args(v, a);
   if (e != cudaSuccess) return e;
@@ -1382,29 +1397,40 @@ cudaError_t write_z(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t
   a.a_ok = v.row_ok;
   a.b_ok = v.feat_ok;
   a.wz_r0 = r0; a.wz_nr = nr; a.wz_f0 = f0; a.wz_nf = nf; a.ldo = ldo;
+  a.wz_trans = trans;
   a.out = out;
   a.zt_hi = zt_hi;
   a.zt_lo = zt_lo;
   a.zt_scale = zt_scale;
-  a.out_elems = zt_hi ? (nf - 1) * ldo + nr : (nr - 1) * ldo + nf;
+  a.out_elems = zt_hi || trans ? (nf - 1) * ldo + nr : (nr - 1) * ldo + nf;
   if ((e = make_map(&a.tA_hi, v.Xhi, v.dld, v.nslots, v.dld, 128, view_kc(v))) != cudaSuccess) return e;
   if ((e = make_map(&a.tA_lo, v.Xlo, v.dld, v.nslots, v.dld, 128, view_kc(v))) != cudaSuccess) return e;
-  const int brows = view_brows(v);
-  if ((e = make_map(&a.tB_hi, v.Ghi, v.dld, v.fslots, v.dld, brows, view_kc(v))) != cudaSuccess) return e;
-  if ((e = make_map(&a.tB_lo, v.Glo, v.dld, v.fslots, v.dld, brows, view_kc(v))) != cudaSuccess) return e;
+  if ((e = make_map(&a.tB_hi, v.Ghi, v.dld, v.fslots, v.dld, 128, view_kc(v))) != cudaSuccess) return e;
+  if ((e = make_map(&a.tB_lo, v.Glo, v.dld, v.fslots, v.dld, 128, view_kc(v))) != cudaSuccess) return e;
   a.tM_hi = a.tB_hi;
   a.tM_lo = a.tB_lo;
-  return launch(a, dim3((unsigned)tile_grid(v, ceil_div(nr, 128))), v.st, view_kc(v), view_zt(v), view_cg(v));
+  const int64_t rt = ceil_div(nr, 128), nt = ceil_div(nf, 128);
+  int64_t best = 1, cost = INT64_MAX;
+  for (int64_t ny = 1; ny <= std::min<int64_t>(nt, 1024); ++ny) {
+    const int64_t c = ceil_div(rt * ny, sm_count()) * (2 * ceil_div(nt, ny) + 1);
+    if (c < cost) {
+      cost = c;
+      best = ny;
+    }
+  }
+  a.nsplit = (int)best;
+  return launch(a, dim3((unsigned)rt, (unsigned)best), v.st, view_kc(v), view_zt(v), view_cg(v));
 }
 }  // namespace
 
-cudaError_t tc_write_z(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float* out, int64_t ldo) {
-  return write_z(v, r0, nr, f0, nf, out, nullptr, nullptr, 0.f, ldo);
+cudaError_t tc_write_z(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float* out, int64_t ldo,
+                       int trans) {
+  return write_z(v, r0, nr, f0, nf, out, trans, nullptr, nullptr, 0.f, ldo);
 }
 
 cudaError_t tc_write_zt_split(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float scale,
                               __half* hi, __half* lo, int64_t ldt) {
-  return write_z(v, r0, nr, f0, nf, nullptr, hi, lo, scale, ldt);
+  return write_z(v, r0, nr, f0, nf, nullptr, 0, hi, lo, scale, ldt);
 }
 
 namespace {

@@ -35,8 +35,9 @@ struct TcView {
   cudaStream_t st;
 };
 
-// Z for row slots [r0, r0+nr) x feature slots [f0, f0+nf) into out (ld ldo), float32.
-cudaError_t tc_write_z(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float* out, int64_t ldo);
+// Z for row slots [r0, r0+nr) x feature slots [f0, f0+nf) into out (ld ldo), float32; trans: Z^T.
+cudaError_t tc_write_z(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float* out, int64_t ldo,
+                       int trans = 0);
 // The same window as Z^T split into FP16 hi/lo of scale * Z: hi[f][r], lo[f][r] (ld ldt) for
 // f < nf, r < nr; the elements outside the window are left as they are.
 cudaError_t tc_write_zt_split(const TcView& v, int64_t r0, int64_t nr, int64_t f0, int64_t nf, float scale,
