@@ -400,7 +400,7 @@ void compute_geometry(rff_admm_s& s, int64_t n, int64_t d) {
     int nsm = 148, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tile = s.split_path() ? 128 : 64;   // pass-1 row step of a split
+    const int64_t tile = 128;                          // pass-1 row step of a split
     const int64_t ftiles = s.fslots / 128;             // pass-1 CTAs per row block and split
     int64_t min_rows = n;
     for (int i = 0; i < s.R; ++i) min_rows = std::min(min_rows, s.row_size[i]);
@@ -928,7 +928,7 @@ rff_status materialise_z(rff_admm_t h) {
       ta.pad = 1;
       CK(launch_tensorsketch(ta, s.C, ts_block_max(s), s.st));
     } else {
-      ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)s.dld, s.bias, s.zmap_scale(), s.row_of_slot,
+      ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)round_up(s.d, 4), s.bias, s.zmap_scale(), s.row_of_slot,
                s.feat_of_slot, r0, nr, 0, s.fslots, zc, s.fslots, s.p.feature_map};
       CK(launch_write_z_simt(za, s.st));
     }
@@ -1248,7 +1248,7 @@ rff_status setup_factors(rff_admm_t h) {
           continue;
         }
         // FP32 precision: Z on the SIMT pipes, its Gram from FP32 products with float-float sums
-        ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)s.dld, s.bias, scale, s.row_of_slot, s.feat_of_slot,
+        ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)round_up(s.d, 4), s.bias, scale, s.row_of_slot, s.feat_of_slot,
                  s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, smax_pad, s.p.feature_map, 0};
         CK(launch_write_z_simt(za, s.st));
         CK(launch_gram_f32_to_f64(Zc, smax_pad, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
@@ -1266,7 +1266,7 @@ rff_status setup_factors(rff_admm_t h) {
           if (s.split_path()) {
             CK(tc_write_z(tc_view(s), w0, wn, s.col_slot[j] + f0, nf, Zc, wn, 1));
           } else {
-            ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)s.dld, s.bias, scale, s.row_of_slot, s.feat_of_slot,
+            ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)round_up(s.d, 4), s.bias, scale, s.row_of_slot, s.feat_of_slot,
                      w0, wn, s.col_slot[j] + f0, nf, Zc, wn, s.p.feature_map, 1};
             CK(launch_write_z_simt(za, s.st));
           }
@@ -1347,7 +1347,7 @@ PassArgs base_pass_args(const rff_admm_s& s) {
   a.ldx = s.dld;
   a.Gt = s.Gt32;
   a.ldg = s.dld;
-  a.K = (int)s.dld;
+  a.K = (int)round_up(s.d, 4);
   a.bias = s.bias;
   a.scale = s.zmap_scale();
   a.map = s.p.feature_map;
@@ -2657,7 +2657,7 @@ rff_status features_impl(const float* X, int64_t n, int64_t d, uint64_t seed, do
   const float scale = (float)(map ? 1.0 / std::sqrt((double)D) : std::sqrt(2.0 / (double)D));
   if (e == cudaSuccess && !negative) {
     if (prec == RFF_PREC_FP32) {
-      ZArgs za{X32, dld, G32, dld, (int)dld, bias, scale, rok, fok, 0, n, 0, nf, Z, nf, map};
+      ZArgs za{X32, dld, G32, dld, (int)round_up(d, 4), bias, scale, rok, fok, 0, n, 0, nf, Z, nf, map};
       e = launch_write_z_simt(za, st);
     } else {
       if (bcol >= 0) e = launch_set_column(X32, dld, np, bcol, 1.f, st);

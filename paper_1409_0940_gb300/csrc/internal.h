@@ -54,7 +54,7 @@ struct PassArgs {
   int64_t ldx;
   const float* Gt;       // feature rows (slots) x K, float32         (SIMT)
   int64_t ldg;
-  int K;                 // padded input dimension (multiple of 64)
+  int K;                 // input dimension, rounded up to a multiple of 4 (the rows hold round_up(K, 32) values)
   const float* bias;     // b per feature slot
   float scale;           // sqrt(2/D)
   const int32_t* row_ok; // row_of_slot table (-1 = padding), or null = all valid
