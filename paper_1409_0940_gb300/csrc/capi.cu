@@ -367,7 +367,7 @@ void compute_geometry(rff_admm_s& s, int64_t n, int64_t d) {
   for (int i = 0; i < s.R; ++i)
     for (int j = 0; j < s.C; ++j) {
       const int64_t fd = s.outer ? s.row_size[i] : s.col_size[j];
-      s.foff[(size_t)i * s.C + j + 1] = s.foff[(size_t)i * s.C + j] + fd * fd;
+      s.foff[(size_t)i * s.C + j + 1] = s.foff[(size_t)i * s.C + j] + fd * round_up(fd, 4);
     }
   s.qrow.assign((size_t)s.R * s.C, 0);
   s.q_rows = 0;
@@ -1189,7 +1189,7 @@ rff_status setup_factors(rff_admm_t h) {
   // outer form: Z^T in chunks of features, over as many row blocks at once as OUTER_ZT_BYTES (or an
   // eighth of the memory left) holds: a chunk of one block of 625 rows gives the 152 SMs 5 tiles
   // of work for the regeneration and 30 for the Gram (512 launches of each, 243 ms, on the
-  // 20k x 32,768 workload at 32 x 8; in 16 launches of each, 30 ms)
+  // 20k x 32,768 workload at 32 x 8; in 16 launches of each, 19 ms)
   const int64_t chunk_feat = std::min<int64_t>(2048, round_up(smax, SLOT));
   const int64_t smax_pad = round_up(smax, SLOT);
   const int64_t zt_blocks = std::max<int64_t>(
@@ -1306,7 +1306,7 @@ rff_status setup_factors(rff_admm_t h) {
         // O'_ij = (I + Z_ij Z_ij^T)^-1 u_ij, rows of block i in column block j
         const int64_t ni = s.row_size[i], roff = ((int64_t)j * s.nslots + s.row_slot[i]) * s.mpad;
         float* yb = s.U32 + (int64_t)s.C * s.nslots * s.mpad;   // y_ij = -P_ij e_ij (alpha = -1)
-        g[blk] = GemmDesc{s.Q32 + s.foff[blk], s.U32 + roff, nullptr, yb + roff, (int)ni, (int)s.mpad, (int)ni, ni,
+        g[blk] = GemmDesc{s.Q32 + s.foff[blk], s.U32 + roff, nullptr, yb + roff, (int)ni, (int)s.mpad, (int)ni, round_up(ni, 4),
                           s.mpad, 0, s.mpad};
       } else if (s.split_path()) {
         // one job per 128-row tile of Q_ij: rows of W'_ij, all m_pad columns, K = s_j
@@ -1323,8 +1323,8 @@ rff_status setup_factors(rff_admm_t h) {
         }
       } else {
         float* Qb = s.Q32 + s.foff[blk];   // W'_ij += Q_ij rhs_ij (the incremental projection)
-        g[blk] = GemmDesc{Qb, s.rhs + off, s.What + off, s.What + off, (int)sj, (int)s.mpad, (int)sj, sj, s.mpad,
-                          s.mpad, s.mpad};
+        g[blk] = GemmDesc{Qb, s.rhs + off, s.What + off, s.What + off, (int)sj, (int)s.mpad, (int)sj, round_up(sj, 4),
+                          s.mpad, s.mpad, s.mpad};
       }
     }
   if (s.split_path() && !s.outer) {
@@ -1541,7 +1541,7 @@ rff_status iterate_outer(rff_admm_t h, int k) {
   }
   // e_ij = V_ij - u_ij (in place), y_ij = -P_ij e_ij
   CK(launch_outer_residual(s.U32, s.Op, s.V32, s.nslots, (int)s.mpad, s.C, s.st));
-  CK(launch_gemm_f32_nn(s.gdesc, s.R * s.C, (int)nmax, (int)s.mpad, -1.f, 0.f, s.st, s.act()));
+  CK(launch_gemm_f32_nn(s.gdesc, s.R * s.C, (int)nmax, (int)nmax, (int)s.mpad, -1.f, 0.f, s.st, s.act()));
   // W'_ij = c_ij - Z_ij^T y_ij (operand per block)
   PassArgs a = base_pass_args(s);
   a.bmask = s.act();
@@ -1640,7 +1640,7 @@ rff_status phase_project(rff_admm_t h, int k) {
                                   s.mpad * s.fslots, 1.f, s.amax + AMAX_W, s.st));
   } else {
     CK(launch_rhs(s.Wbar, s.muij, s.Rpart, s.nsplit, s.R, nfe, s.rhs, s.st, nullptr, 0, s.What));
-    CK(launch_gemm_f32_nn(s.gdesc, (int)nblocks, (int)smax, (int)s.mpad, 1.f, 1.f, s.st, s.act()));
+    CK(launch_gemm_f32_nn(s.gdesc, (int)nblocks, (int)smax, (int)smax, (int)s.mpad, 1.f, 1.f, s.st, s.act()));
   }
   if ((r = mark(h, k, 3)) != RFF_OK) return r;
   if (s.split_path()) CK(cudaMemsetAsync(s.amax + AMAX_OP, 0, 4, s.st));   // max |O'| for the exchange

@@ -4,6 +4,7 @@
 // per-iteration products with Q_ij and H_ij.
 #include "common.cuh"
 #include "internal.h"
+#include "simt.cuh"
 
 #include <algorithm>
 #include <cstdlib>
@@ -84,75 +85,195 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmDesc* __restrict__ descs
 }
 
 // ------------------------------------------------------------------ FP32 NN GEMM
-// The per-iteration products x = Q r and r = b - H x: A (M x K) and B (K x N)
-// row-major with K-contiguous A rows, N-contiguous B rows; vector loads when the
-// tile is interior.  Tile 64 x 64, BK = 32.  descs null: the one product given by value.
-__global__ void __launch_bounds__(256) k_gemm_f32_nn(const GemmDesc* __restrict__ descs, const GemmDesc one,
-                                                     float alpha, float beta, const uint8_t* __restrict__ bmask) {
-  if (bmask && !bmask[blockIdx.z]) return;
-  const GemmDesc g = descs ? descs[blockIdx.z] : one;
-  const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 64;
-  if (m0 >= g.M || n0 >= g.N) return;
+// The per-iteration products with the cached factors, W' += Q r and y = -P e, and the scores of
+// sketched rows: D = alpha A B + beta C, A (M x K) row-major with 16-byte aligned rows, B (K x N)
+// with N = 16 MQ = ldb columns.  One CTA per 128 rows and all N columns, so A is read once; 8 x MQ
+// outputs per thread (rows ty + 16 i, columns tx + 16 q); 32 K elements per stage of a four-stage
+// ring of asynchronous copies.
+//
+// FP32 products are summed 32 at a time, each chunk's sum folded into a float-float accumulator
+// (TwoSum): the error of a K-term dot product is that of one 32-term FP32 sum instead of a K-term
+// one (K = s_j = 4096 for the cached projection).  For N > 64 the float-float accumulators wait
+// in tensor memory.
+//
+// cl = GEMM_CL: the K chunks of a product are shared by a cluster of GEMM_CL CTAs, whose
+// float-float sums are added in order through distributed shared memory.
+// Measured against 64 x 64 tiles without a pipeline: four 4096 x 4096 by 160, 1.92 -> 0.71 ms (30
+// TFLOP/s); 256 of 625 x 625 by 16, 856 -> 180 us (2.2 TB/s of factors); and, split over clusters,
+// 512 x 512 by 16, 68 -> 5.6 us, 2048 x 8192 by 16, 1265 -> 61 us.
+constexpr int GEMM_NS = 4, GEMM_CL = 8, GEMM_M = 128, GEMM_K = 32, GEMM_LDK = simt::row_stride(GEMM_K);
+constexpr int GEMM_CL_MAX_N = 144;   // the float-float sums of 128 rows fit the ring's memory
+__host__ __device__ constexpr int gemm_stage(int n) { return GEMM_M * GEMM_LDK + GEMM_K * n; }   // floats
+__host__ __device__ constexpr size_t gemm_smem(int n) { return (size_t)GEMM_NS * gemm_stage(n) * 4; }
+static_assert((size_t)2 * GEMM_M * GEMM_CL_MAX_N * 4 <= gemm_smem(GEMM_CL_MAX_N), "");
+static_assert(gemm_smem(256) <= 232448 - 256, "the ring fits a CTA's shared memory at N = 256");
+// tensor-memory columns of the parked accumulators (16 MQ words a thread, two threads a lane)
+__host__ __device__ constexpr uint32_t gemm_tmem_cols(int mq) { return mq <= 8 ? 256u : 512u; }
+
+template <int MQ>
+__global__ void __launch_bounds__(256) k_gemm_f32_nn(const GemmDesc* __restrict__ descs,
+                                                     const __grid_constant__ GemmDesc one, float alpha, float beta,
+                                                     const uint8_t* __restrict__ bmask, int cl) {
+  using namespace simt;
+  constexpr int N = 16 * MQ, STG = gemm_stage(N);
+  constexpr bool PARK = MQ > 4;
+  if (bmask && !bmask[blockIdx.y]) return;
+  const GemmDesc g = descs ? descs[blockIdx.y] : one;
+  const int rank = cl > 1 ? (int)tc5::cluster_rank() : 0;
+  const int m0 = (int)(blockIdx.x / cl) * GEMM_M;
+  if (m0 >= g.M) return;   // (a cluster's CTAs share m0)
+  extern __shared__ __align__(16) float gm_smem[];
+  __shared__ uint32_t tmem_word;
+  const int tid = threadIdx.x, tx = thread_tx(), ty = thread_ty();
+  if (PARK && tid < 32) tc5::tmem_alloc<1>(tc5::smem_u32(&tmem_word), gemm_tmem_cols(MQ));
   const float* __restrict__ A = static_cast<const float*>(g.A);
   const float* __restrict__ B = static_cast<const float*>(g.B);
-  __shared__ __align__(16) float As[32][64 + 4];
-  __shared__ __align__(16) float Bs[32][64 + 4];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  // FP32 products summed 32 at a time (acc), each chunk's sum folded into a float-float
-  // accumulator (hi, lo) by TwoSum: the error of a K-term dot product is that of one
-  // 32-term FP32 sum instead of a K-term one (K = s_j = 4096 for the cached projection)
-  float hi[4][4] = {}, lo[4][4] = {};
-  for (int k0 = 0; k0 < g.K; k0 += 32) {
-    float acc[4][4] = {};
-    // A tile: 64 rows x 32 k
-    for (int t = tid; t < 64 * 32; t += 256) {
-      const int kk = t % 32, mm = t / 32;
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < g.M && gk < g.K) ? A[(int64_t)gm * g.lda + gk] : 0.f;
-    }
-    // B tile: 32 k x 64 n
-    for (int t = tid; t < 64 * 32; t += 256) {
-      const int nn = t % 64, kb = t / 64;
-      const int gn = n0 + nn, gk = k0 + kb;
-      Bs[kb][nn] = (gn < g.N && gk < g.K) ? B[(int64_t)gk * g.ldb + gn] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-      const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
+  const int nch = (g.K + GEMM_K - 1) / GEMM_K;
+  const int c0 = (int)((int64_t)rank * nch / cl), c1 = (int)((int64_t)(rank + 1) * nch / cl);
+  auto issue = [&](int c) {
+    if (c < c1) {
+      float* As = gm_smem + ((c - c0) % GEMM_NS) * STG;
+      float* Bs = As + GEMM_M * GEMM_LDK;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // TwoSum (Knuth); separately rounded operations, not contracted
-        const float sum = __fadd_rn(hi[i][j], acc[i][j]);
-        const float bb = __fsub_rn(sum, hi[i][j]);
-        lo[i][j] += __fadd_rn(__fsub_rn(hi[i][j], __fsub_rn(sum, bb)), __fsub_rn(acc[i][j], bb));
-        hi[i][j] = sum;
+      for (int q = 0; q < 4; ++q) {
+        const int e = tid + 256 * q, r = e / 8, k = c * GEMM_K + 4 * (e % 8);
+        const int bytes = m0 + r < g.M ? max(0, min(16, 4 * (g.K - k))) : 0;
+        cp_async16_fill(As + r * GEMM_LDK + 4 * (e % 8), bytes ? A + (int64_t)(m0 + r) * g.lda + k : A, bytes);
       }
+      for (int e = tid; e < GEMM_K * N / 4; e += 256) {
+        const int k = c * GEMM_K + e / (N / 4);
+        const int bytes = k < g.K ? 16 : 0;
+        cp_async16_fill(Bs + 4 * e, bytes ? B + (int64_t)k * N + 4 * (e % (N / 4)) : B, bytes);
+      }
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int c = 0; c < GEMM_NS - 1; ++c) issue(c0 + c);
+  uint32_t park = 0;
+  float hi[PARK ? 1 : MQ][8], lo[PARK ? 1 : MQ][8];
+#pragma unroll
+  for (int q = 0; q < (PARK ? 1 : MQ); ++q)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) hi[q][i] = lo[q][i] = 0.f;
+  if (PARK) {
+    tc5::fence_before();
+    __syncthreads();
+    tc5::fence_after();
+    park = park_base(tmem_word, gemm_tmem_cols(MQ));
+    for (int q = 0; q < 2 * MQ; ++q) park8(park + 8 * q, hi[0]);
+    tc5::tmem_wait_st();
   }
+  for (int c = c0; c < c1; ++c) {
+    cp_wait<GEMM_NS - 2>();
+    __syncthreads();   // chunk c has landed; everyone is done with chunk c - 1
+    issue(c + GEMM_NS - 1);
+    const float* ap = gm_smem + ((c - c0) % GEMM_NS) * STG + ty * GEMM_LDK;
+    const float* bp = gm_smem + ((c - c0) % GEMM_NS) * STG + GEMM_M * GEMM_LDK + tx;
+    float acc[MQ][8];
+#pragma unroll
+    for (int q = 0; q < MQ; ++q)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[q][i] = 0.f;
+#pragma unroll 2
+    for (int k4 = 0; k4 < GEMM_K / 4; ++k4) {
+      float a[8][4];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(ap + 16 * i * GEMM_LDK + 4 * k4);
+        a[i][0] = v.x; a[i][1] = v.y; a[i][2] = v.z; a[i][3] = v.w;
+      }
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+        for (int q = 0; q < MQ; ++q) {
+          const float b = bp[(4 * k4 + kk) * N + 16 * q];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) acc[q][i] = fmaf(a[i][kk], b, acc[q][i]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < MQ; ++q) {
+      if (PARK) {
+        float h[8], l[8];
+        unpark8(park + 8 * q, h);
+        unpark8(park + 8 * (MQ + q), l);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) two_sum_into(h[i], l[i], acc[q][i]);
+        park8(park + 8 * q, h);
+        park8(park + 8 * (MQ + q), l);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) two_sum_into(hi[PARK ? 0 : q][i], lo[PARK ? 0 : q][i], acc[q][i]);
+      }
+    }
+    if (PARK) tc5::tmem_wait_st();
+  }
+  cp_wait<0>();   // (only empty groups are left)
   const float* __restrict__ Cm = static_cast<const float*>(g.Cm);
   float* __restrict__ D = static_cast<float*>(g.D);
+  if (cl == 1) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty * 4 + i;
-    if (gm >= g.M) continue;
+    for (int q = 0; q < MQ; ++q) {
+      float h[8], l[8];
+      if (PARK) {
+        unpark8(park + 8 * q, h);
+        unpark8(park + 8 * (MQ + q), l);
+      }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx * 4 + j;
-      if (gn >= g.N) continue;
-      float v = alpha * (hi[i][j] + lo[i][j]);
-      if (beta != 0.f) v = fmaf(beta, Cm[(int64_t)gm * g.ldc + gn], v);
-      D[(int64_t)gm * g.ldd + gn] = v;
+      for (int i = 0; i < 8; ++i) {
+        const int gm = m0 + ty + 16 * i;
+        if (gm >= g.M) continue;
+        float v = alpha * (PARK ? h[i] + l[i] : hi[PARK ? 0 : q][i] + lo[PARK ? 0 : q][i]);
+        if (beta != 0.f) v = fmaf(beta, Cm[(int64_t)gm * g.ldc + tx + 16 * q], v);
+        D[(int64_t)gm * g.ldd + tx + 16 * q] = v;
+      }
     }
+  } else {
+    __syncthreads();   // everyone is done reading the ring
+#pragma unroll
+    for (int q = 0; q < MQ; ++q) {
+      float h[8], l[8];
+      if (PARK) {
+        unpark8(park + 8 * q, h);
+        unpark8(park + 8 * (MQ + q), l);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        gm_smem[(ty + 16 * i) * N + tx + 16 * q] = PARK ? h[i] : hi[PARK ? 0 : q][i];
+        gm_smem[(GEMM_M + ty + 16 * i) * N + tx + 16 * q] = PARK ? l[i] : lo[PARK ? 0 : q][i];
+      }
+    }
+    tc5::cluster_sync_all();
+    constexpr int SHARE = GEMM_M * N / GEMM_CL;
+    const uint32_t base = tc5::smem_u32(gm_smem);
+    for (int e = rank * SHARE + tid; e < (rank + 1) * SHARE; e += 256) {
+      float h[GEMM_CL], l[GEMM_CL];
+#pragma unroll
+      for (int r = 0; r < GEMM_CL; ++r) {
+        h[r] = ld_cluster(base + 4 * e, r);
+        l[r] = ld_cluster(base + 4 * (GEMM_M * N + e), r);
+      }
+      float th = h[0], tl = l[0];
+#pragma unroll
+      for (int r = 1; r < GEMM_CL; ++r) {
+        two_sum_into(th, tl, h[r]);
+        tl = __fadd_rn(tl, l[r]);
+      }
+      const int gm = m0 + e / N, col = e % N;
+      if (gm < g.M) {
+        float v = alpha * (th + tl);
+        if (beta != 0.f) v = fmaf(beta, Cm[(int64_t)gm * g.ldc + col], v);
+        D[(int64_t)gm * g.ldd + col] = v;
+      }
+    }
+    tc5::cluster_sync_all();   // nobody leaves while others read its shared memory
+  }
+  if (PARK) {
+    tc5::fence_before();
+    __syncthreads();
+    tc5::fence_after();
+    if (tid < 32) tc5::tmem_dealloc<1>(tmem_word, gemm_tmem_cols(MQ));
   }
 }
 
@@ -284,109 +405,120 @@ __global__ void k_to_pairs(const GemmDesc* __restrict__ descs) {
   static_cast<float2*>(g.D)[r * g.ldd + c] = make_float2(h, __double2float_rn(v - (double)h));
 }
 
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float bb = s - hi;
-  const float e = (hi - (s - bb)) + (x - bb);
-  hi = s;
-  lo += e;
-}
+// Gram accumulation H (FP64) += Z^T Z over the n rows of Z (row-major, ld ldz): one CTA per
+// 128 x 128 tile of H on or below the diagonal, 8 x 8 outputs per thread (rows ty*4 + {0..3} and
+// 64 + ty*4 + {0..3}, columns the same of tx), 32 rows of both operands per stage of a
+// four-stage ring of asynchronous copies.  Bound: the FP32 pipe (64 multiply-adds for four
+// 16-byte shared-memory loads).  Products and 64-row partial sums in FP32 (round to nearest,
+// unbiased), folded into a float-float accumulator (TwoSum) after every 64 rows, added to H in
+// FP64 at the end: about 2^-44 relative per entry.  The 128 words of the float-float accumulator
+// wait in tensor memory between folds.  Against 128 x 64 tiles of 8 x 4 outputs with the
+// accumulator in registers (238 of them, one CTA of eight warps): the 256 blocks of
+// 625 rows x 4096 features of a 32 x 8 grid 86 ms in 512 launches -> 15.3 ms in 16 (34 TFLOP/s).
+constexpr int GR_T = 128, GR_K = 32, GR_NS = 4;
+constexpr size_t GR_SMEM = (size_t)GR_NS * 2 * GR_K * GR_T * 4;
 
-// Gram accumulation H (FP64) += Z^T Z over the n rows of Z (n x s, row-major, ld ldz): one CTA
-// per 128 x 64 tile of H that reaches the lower triangle, 8 x 4 outputs per thread (rows
-// ty*4 + {0..3} and 64 + ty*4 + {0..3}, columns tx*4 + {0..3}: a warp's shared-memory reads are
-// broadcasts or consecutive), rows staged 32 at a time through double-buffered shared memory
-// (one stage's arithmetic covers the next stage's global loads).
-// Products and 64-row partial sums in FP32 (round to nearest, unbiased), folded into a
-// float-float accumulator (TwoSum) after every chunk, added to H in FP64 at the end: about
-// 2^-44 relative per entry.
-constexpr int GR_M = 128, GR_N = 64, GR_K = 32;
-
-__global__ void __launch_bounds__(256) k_gram_tile(const float* __restrict__ Zall, int64_t ldz, int64_t n,
-                                                   const int64_t* __restrict__ slot,
-                                                   const int64_t* __restrict__ size, int64_t s_one,
-                                                   double* __restrict__ Hall, int64_t h_stride) {
-  const int64_t a0 = (int64_t)blockIdx.x * GR_M, b0 = (int64_t)blockIdx.y * GR_N;
-  const int64_t s = size ? size[blockIdx.z] : s_one, ldh = s;
-  const float* Z = Zall + (slot ? slot[blockIdx.z] - slot[0] : 0);
-  double* H = Hall + blockIdx.z * h_stride;
-  if (a0 >= s || b0 > a0 + GR_M - 1) return;   // past this matrix, or wholly above the diagonal
-  __shared__ __align__(16) float As[2][GR_K][GR_M];
-  __shared__ __align__(16) float Bs[2][GR_K][GR_N];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  float acc[8][4], hi[8][4], lo[8][4];
+__global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ Zall, int64_t ldz, int64_t n,
+                                                      const int64_t* __restrict__ slot,
+                                                      const int64_t* __restrict__ size, int64_t s_one,
+                                                      double* __restrict__ Hall, int64_t h_stride) {
+  using namespace simt;
+  // tile (ta, tb), tb <= ta, of the lower triangle
+  int ta = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while (ta * (ta + 1) / 2 > (int)blockIdx.x) --ta;
+  while ((ta + 1) * (ta + 2) / 2 <= (int)blockIdx.x) ++ta;
+  const int64_t a0 = (int64_t)ta * GR_T, b0 = ((int64_t)blockIdx.x - (int64_t)ta * (ta + 1) / 2) * GR_T;
+  const int64_t s = size ? size[blockIdx.y] : s_one;
+  if (a0 >= s) return;   // past this matrix
+  const float* Z = Zall + (slot ? slot[blockIdx.y] - slot[0] : 0);
+  double* H = Hall + blockIdx.y * h_stride;
+  extern __shared__ __align__(16) float gr_smem[];
+  __shared__ uint32_t tmem_word;
+  const int tid = threadIdx.x, tx = thread_tx(), ty = thread_ty();
+  if (tid < 32) tc5::tmem_alloc<1>(tc5::smem_u32(&tmem_word), 512);
+  const int64_t nst = ceil_div(n, GR_K);
+  auto issue = [&](int64_t st) {
+    if (st < nst) {
+      float* As = gr_smem + (st % GR_NS) * (2 * GR_K * GR_T);
+      float* Bs = As + GR_K * GR_T;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int e = tid + 256 * q, r = e / 32, c = 4 * (e % 32);
+        const int64_t gr = st * GR_K + r;
+        const float* row = Z + (gr < n ? gr : n - 1) * ldz;   // rows past n: zeros
+        const int bytes = gr < n ? 16 : 0;
+        cp_async16_fill(As + r * GR_T + c, row + a0 + c, bytes);
+        cp_async16_fill(Bs + r * GR_T + c, row + b0 + c, bytes);
+      }
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int st = 0; st < GR_NS - 1; ++st) issue(st);
+  tc5::fence_before();
+  __syncthreads();
+  tc5::fence_after();
+  const uint32_t park = park_base(tmem_word, 512);
+  float acc[8][8];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = hi[i][j] = lo[i][j] = 0.f;
-  float ra[16], rb[8];   // the next stage in registers: A element tid + 256 q, B element tid + 256 q
-  auto fetch = [&](int64_t r0) {
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int e = tid + 256 * q, r = e / GR_M, c = e % GR_M;
-      ra[q] = (r0 + r < n && a0 + c < s) ? __ldg(Z + (r0 + r) * ldz + a0 + c) : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int e = tid + 256 * q, r = e / GR_N, c = e % GR_N;
-      rb[q] = (r0 + r < n && b0 + c < s) ? __ldg(Z + (r0 + r) * ldz + b0 + c) : 0.f;
-    }
-  };
-  auto stash = [&](int buf) {
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int e = tid + 256 * q;
-      As[buf][e / GR_M][e % GR_M] = ra[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int e = tid + 256 * q;
-      Bs[buf][e / GR_N][e % GR_N] = rb[q];
-    }
-  };
-  fetch(0);
-  stash(0);
-  __syncthreads();
-  int buf = 0, stage = 0;
-  for (int64_t r0 = 0; r0 < n; r0 += GR_K, ++stage) {
-    const bool more = r0 + GR_K < n;
-    if (more) fetch(r0 + GR_K);
-#pragma unroll
+  for (int i = 0; i < 16; ++i) park8(park + 8 * i, acc[0]);
+  tc5::tmem_wait_st();
+  for (int64_t st = 0; st < nst; ++st) {
+    cp_wait<GR_NS - 2>();
+    __syncthreads();   // stage st has landed; everyone is done with stage st - 1
+    issue(st + GR_NS - 1);
+    const float* As = gr_smem + (st % GR_NS) * (2 * GR_K * GR_T);
+    const float* Bs = As + GR_K * GR_T;
+#pragma unroll 4
     for (int k = 0; k < GR_K; ++k) {
-      const float4 a_lo = *reinterpret_cast<const float4*>(&As[buf][k][ty * 4]);
-      const float4 a_hi = *reinterpret_cast<const float4*>(&As[buf][k][64 + ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-      const float a[8] = {a_lo.x, a_lo.y, a_lo.z, a_lo.w, a_hi.x, a_hi.y, a_hi.z, a_hi.w};
-      const float b[4] = {bv.x, bv.y, bv.z, bv.w};
+      const float4 al = *reinterpret_cast<const float4*>(As + k * GR_T + ty * 4);
+      const float4 ah = *reinterpret_cast<const float4*>(As + k * GR_T + 64 + ty * 4);
+      const float4 bl = *reinterpret_cast<const float4*>(Bs + k * GR_T + tx * 4);
+      const float4 bh = *reinterpret_cast<const float4*>(Bs + k * GR_T + 64 + tx * 4);
+      const float a[8] = {al.x, al.y, al.z, al.w, ah.x, ah.y, ah.z, ah.w};
+      const float b[8] = {bl.x, bl.y, bl.z, bl.w, bh.x, bh.y, bh.z, bh.w};
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
-    if ((stage & 1) || !more) {   // every 64 rows: fold the partial sums into hi + lo
+    if ((st & 1) || st + 1 == nst) {   // every 64 rows: fold the partial sums into hi + lo
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 8; ++i) {
+        float hi[8], lo[8];
+        unpark8(park + 16 * i, hi);
+        unpark8(park + 16 * i + 8, lo);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          two_sum_acc(hi[i][j], lo[i][j], acc[i][j]);
+        for (int j = 0; j < 8; ++j) {
+          two_sum_into(hi[j], lo[j], acc[i][j]);
           acc[i][j] = 0.f;
         }
-    }
-    if (more) {   // nobody reads buf ^ 1 in this stage: the sync below ends the stage that did
-      stash(buf ^ 1);
-      __syncthreads();
-      buf ^= 1;
+        park8(park + 16 * i, hi);
+        park8(park + 16 * i + 8, lo);
+      }
+      tc5::tmem_wait_st();
     }
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
+    float hi[8], lo[8];
+    unpark8(park + 16 * i, hi);
+    unpark8(park + 16 * i + 8, lo);
     const int64_t gm = a0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t gn = b0 + tx * 4 + j;
-      if (gm < s && gn < s) H[gm * ldh + gn] += (double)hi[i][j] + (double)lo[i][j];
+    for (int j = 0; j < 8; ++j) {
+      const int64_t gn = b0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
+      if (gm < s && gn < s) H[gm * s + gn] += (double)hi[j] + (double)lo[j];
     }
   }
+  tc5::fence_before();
+  __syncthreads();
+  tc5::fence_after();
+  if (tid < 32) tc5::tmem_dealloc<1>(tmem_word, 512);
 }
 
 // ------------------------------------------------------------------ diagonal potrf
@@ -467,19 +599,72 @@ __global__ void k_zero_strict_upper(double* A, int64_t s) {
 
 }  // namespace
 
-cudaError_t launch_gemm_f32_nn(const GemmDesc* descs_dev, int nbatch, int maxM, int maxN, float alpha, float beta,
-                               cudaStream_t st, const uint8_t* bmask) {
-  if (nbatch <= 0 || maxM <= 0 || maxN <= 0) return cudaSuccess;
-  dim3 grid((unsigned)ceil_div(maxM, 64), (unsigned)ceil_div(maxN, 64), (unsigned)nbatch);
-  k_gemm_f32_nn<<<grid, 256, 0, st>>>(descs_dev, GemmDesc{}, alpha, beta, bmask);
-  return cudaGetLastError();
+namespace {
+int dense_sms() {
+  static int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      v = 0;
+    cudaGetLastError();
+    return v > 0 ? v : 148;
+  }();
+  return n;
+}
+
+template <int MQ>
+cudaError_t launch_gemm_mq(const GemmDesc* descs, const GemmDesc& one, int nbatch, int maxM, int maxK, float alpha,
+                           float beta, const uint8_t* bmask, cudaStream_t st) {
+  constexpr size_t smem = gemm_smem(16 * MQ);
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_f32_nn<MQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // One CTA per 128 rows, or a cluster sharing its K chunks where that ends sooner: waves times
+  // chunks per CTA, four chunks for filling the ring and, in a cluster, the exchange (clusters of
+  // eight leave about an eighth of the SMs unused)
+  const int64_t ctas = ceil_div(maxM, GEMM_M) * nbatch, nch = ceil_div(maxK, GEMM_K), nsm = dense_sms();
+  const int64_t whole = ceil_div(ctas, nsm) * (nch + 2);
+  const int64_t shared = ceil_div(ctas * GEMM_CL, nsm * 7 / 8) * (ceil_div(nch, GEMM_CL) + 4);
+  const int cl = 16 * MQ <= GEMM_CL_MAX_N && shared < whole ? GEMM_CL : 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(ceil_div(maxM, GEMM_M) * cl), (unsigned)nbatch);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_gemm_f32_nn<MQ>, descs, one, alpha, beta, bmask, cl);
+}
+
+cudaError_t launch_gemm(const GemmDesc* descs, const GemmDesc& one, int nbatch, int maxM, int maxK, int N, float alpha,
+                        float beta, const uint8_t* bmask, cudaStream_t st) {
+  if (nbatch <= 0 || maxM <= 0) return cudaSuccess;
+  if (N % 16) return cudaErrorInvalidValue;
+  switch (N / 16) {
+#define RFF_MQ(q) \
+  case q:         \
+    return launch_gemm_mq<q>(descs, one, nbatch, maxM, maxK, alpha, beta, bmask, st);
+    RFF_MQ(1) RFF_MQ(2) RFF_MQ(3) RFF_MQ(4) RFF_MQ(5) RFF_MQ(6) RFF_MQ(7) RFF_MQ(8)
+    RFF_MQ(9) RFF_MQ(10) RFF_MQ(11) RFF_MQ(12) RFF_MQ(13) RFF_MQ(14) RFF_MQ(15) RFF_MQ(16)
+#undef RFF_MQ
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+}  // namespace
+
+cudaError_t launch_gemm_f32_nn(const GemmDesc* descs_dev, int nbatch, int maxM, int maxK, int N, float alpha,
+                               float beta, cudaStream_t st, const uint8_t* bmask) {
+  return launch_gemm(descs_dev, GemmDesc{}, nbatch, maxM, maxK, N, alpha, beta, bmask, st);
 }
 
 cudaError_t launch_gemm_f32_nn_one(const GemmDesc& g, float alpha, float beta, cudaStream_t st) {
-  if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid((unsigned)ceil_div(g.M, 64), (unsigned)ceil_div(g.N, 64), 1);
-  k_gemm_f32_nn<<<grid, 256, 0, st>>>(nullptr, g, alpha, beta, nullptr);
-  return cudaGetLastError();
+  if (g.lda % 4 || g.ldb != g.N || (reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.B)) % 16)
+    return cudaErrorInvalidValue;
+  return launch_gemm(nullptr, g, 1, g.M, g.K, g.N, alpha, beta, nullptr, st);
 }
 
 cudaError_t launch_gemm_f64(const GemmDesc* descs_dev, int nbatch, int maxM, int maxN, int transA, int transB,
@@ -512,8 +697,11 @@ cudaError_t launch_to_pairs(const GemmDesc* descs_dev, int nbatch, int maxM, int
 cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, const int64_t* slot, const int64_t* size,
                                    int64_t s_max, int nb, double* H, int64_t h_stride, cudaStream_t st) {
   if (n <= 0 || s_max <= 0 || nb <= 0) return cudaSuccess;
-  dim3 grid((unsigned)ceil_div(s_max, GR_M), (unsigned)ceil_div(s_max, GR_N), (unsigned)nb);
-  k_gram_tile<<<grid, 256, 0, st>>>(Z, ldz, n, slot, size, s_max, H, h_stride);
+  const int64_t nt = ceil_div(s_max, GR_T);
+  const cudaError_t e = cudaFuncSetAttribute(k_gram_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GR_SMEM);
+  if (e != cudaSuccess) return e;
+  k_gram_tile<<<dim3((unsigned)(nt * (nt + 1) / 2), (unsigned)nb), 256, GR_SMEM, st>>>(Z, ldz, n, slot, size, s_max, H,
+                                                                                       h_stride);
   return cudaGetLastError();
 }
 
@@ -620,7 +808,7 @@ cudaError_t launch_factor_init(const std::vector<MatJob>& jobs, cudaStream_t st)
 
 __global__ void k_convert_factors(const __grid_constant__ MatBatch mb) {
   const int64_t s = mb.s[blockIdx.y], t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < s * s) static_cast<float*>(mb.D[blockIdx.y])[t] = (float)mb.A[blockIdx.y][t];
+  if (t < s * s) static_cast<float*>(mb.D[blockIdx.y])[t / s * round_up(s, 4) + t % s] = (float)mb.A[blockIdx.y][t];
 }
 
 cudaError_t launch_convert_factors(const std::vector<MatJob>& jobs, float* const* dst, cudaStream_t st) {

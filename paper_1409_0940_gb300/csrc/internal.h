@@ -139,10 +139,11 @@ struct GemmDesc {          // D = alpha * op(A) op(B) + beta * Cm, row-major
   int M, N, K;
   int64_t lda, ldb, ldc, ldd;
 };
-// f32 iteration GEMM, NN only, desc array on the device; bmask: descriptor b runs only if
-// bmask[b] != 0 (null: all run)
-cudaError_t launch_gemm_f32_nn(const GemmDesc* descs_dev, int nbatch, int maxM, int maxN, float alpha, float beta,
-                               cudaStream_t st, const uint8_t* bmask = nullptr);
+// f32 iteration GEMM, NN only, desc array on the device: every product has N columns (a multiple
+// of 16, at most 256) and ldb = N, A's rows and B are 16-byte aligned, M <= maxM and K <= maxK;
+// bmask: descriptor b runs only if bmask[b] != 0 (null: all run)
+cudaError_t launch_gemm_f32_nn(const GemmDesc* descs_dev, int nbatch, int maxM, int maxK, int N, float alpha,
+                               float beta, cudaStream_t st, const uint8_t* bmask = nullptr);
 // the same for one product whose descriptor is passed by value (no device copy of it)
 cudaError_t launch_gemm_f32_nn_one(const GemmDesc& g, float alpha, float beta, cudaStream_t st);
 // f64 with runtime transposes; double_float: FP64 in and out, double-float arithmetic inside
@@ -179,7 +180,7 @@ struct MatJob {    // host description of one matrix to factor (and invert)
 };
 // H += I on the diagonal and Q = I for every job (A = H)
 cudaError_t launch_factor_init(const std::vector<MatJob>& jobs, cudaStream_t st);
-// dst[b] (FP32, s x s) = jobs[b].Q (ld s)
+// dst[b] (FP32, s x s, ld round_up(s, 4)) = jobs[b].Q (ld s)
 cudaError_t launch_convert_factors(const std::vector<MatJob>& jobs, float* const* dst, cudaStream_t st);
 size_t factor_scratch_bytes(int njobs, int smax);
 // blocked Cholesky (and inverse); double_float selects the double-float GEMM for the block
