@@ -48,6 +48,7 @@ __host__ __device__ constexpr int m_rows(int mq) { return mq <= 6 ? 128 : mq <= 
 static_assert(m_rows(6) * 96 <= STAGE && m_rows(13) * 208 <= STAGE && m_rows(16) * 256 <= STAGE,
               "the rows of M fit a stage");
 constexpr int PARTS = 8;                          // parts of a run of tiles (see pass 2)
+enum { CHAIN, ADD, FF };                          // how the sums of a run are formed (see chain_tile)
 // phases and validity (slot table entries) of a tile pair's B rows, two pairs deep: read from global
 // memory where T becomes Z, their latency was 7 % of the kernel
 struct Meta {
@@ -99,6 +100,7 @@ __device__ __forceinline__ Walk make_walk(int64_t nt, int parts, int p0, int p1)
 // pair of tiles) by tile: nk panel stages and then, with a chain, 128 / MR stages of M per tile.
 struct Feed {
   Walk w;
+  int last;      // rows of the last tile that are read (64 or 128)
   int64_t b0;    // B row of tile 0
   int r;         // step within the tile
   int slot, pair;
@@ -111,7 +113,8 @@ __device__ __forceinline__ void feed_step(Feed& f, const Operands& o, int nk, fl
     float* st = ring + f.slot * STAGE;
     const int tid = threadIdx.x, wd = f.w.width();
     const int64_t b = f.b0 + f.w.t * BN;
-    if (f.r == 0 && tid < wd * BN) {
+    const int rows = wd * BN - (f.w.t + wd == f.w.nt ? BN - f.last : 0);   // B rows of this tile pair
+    if (f.r == 0 && tid < rows) {
       if (o.b_bias) cp_async4(&meta[f.pair].bias[tid], o.b_bias + b + tid);
       if (o.b_ok) cp_async4(&meta[f.pair].ok[tid], o.b_ok + b + tid);
     }
@@ -124,15 +127,12 @@ __device__ __forceinline__ void feed_step(Feed& f, const Operands& o, int nk, fl
 #pragma unroll
       for (int q = 0; q < BM / ROWS; ++q) cp_async16(dst + q * ROWS * LDK, a + q * ROWS * o.lda);
 #pragma unroll
-      for (int q = 0; q < BN / ROWS; ++q) cp_async16(dst + (BM + q * ROWS) * LDK, bp + q * ROWS * o.ldb);
-      if (wd == 2) {
-#pragma unroll
-        for (int q = BN / ROWS; q < 2 * BN / ROWS; ++q)
-          cp_async16(dst + (BM + q * ROWS) * LDK, bp + q * ROWS * o.ldb);
-      }
+      for (int q = 0; q < 2 * BN / ROWS; ++q)
+        if (q * ROWS < rows) cp_async16(dst + (BM + q * ROWS) * LDK, bp + q * ROWS * o.ldb);
     } else {
       const float* src = o.M + (b + (int64_t)(f.r - nk) * MR) * o.mpad;
-      for (int t = tid; t < MR * o.mpad / 4; t += NT) cp_async16(st + 4 * t, src + 4 * t);
+      const int n4 = min(MR, rows - (f.r - nk) * MR) * o.mpad / 4;
+      for (int t = tid; t < n4; t += NT) cp_async16(st + 4 * t, src + 4 * t);
     }
     if (++f.r == nk + (MR ? wd * (BN / (MR ? MR : 1)) : 0)) {
       f.r = 0;
@@ -252,8 +252,8 @@ struct Body {
   uint32_t park;
 
   // tiles of 128 B rows, tile 0 at row b0, walked by w
-  __device__ __forceinline__ Body(float* smem, const Operands& op, int64_t b0, const Walk& w)
-      : ring(smem), ZsT(smem + NS * STAGE), meta(reinterpret_cast<Meta*>(ZsT + BN * ZLD)), o(op), f{w, b0, 0, 0, 0},
+  __device__ __forceinline__ Body(float* smem, const Operands& op, int64_t b0, const Walk& w, int last_rows = BN)
+      : ring(smem), ZsT(smem + NS * STAGE), meta(reinterpret_cast<Meta*>(ZsT + BN * ZLD)), o(op), f{w, last_rows, b0, 0, 0, 0},
         nk((op.K + BK - 1) / BK), slot(0), pair(0), tx(thread_tx()), ty(thread_ty()), park(0) {
 #pragma unroll
     for (int s = 0; s < NS - 1; ++s) feed_step<MR>(f, o, nk, ring, meta);
@@ -280,7 +280,7 @@ struct Body {
     }
   }
   // The tile or two at w: T, then half by half Z and its products with M (chain_tile)
-  template <int MQ, bool FF>
+  template <int MQ, int MODE>
   __device__ __forceinline__ void run(const Walk& w, const RowSide& rs, float scale, int map) {
     float acc[16][8];
     const int wd = w.width();
@@ -288,28 +288,32 @@ struct Body {
     else form_t<8>(acc);
     // (every thread is past the chain of the previous tile: nk >= 1 barriers ago)
     store_z<0>(ZsT, acc, tx, ty, meta[pair], o.b_ok, rs, scale, map);
-    chain_tile<MQ, FF>();
+    chain_tile<MQ, MODE>(w.t + 1 == w.nt ? f.last : BN);
     if (wd == 2) {
       __syncthreads();   // everyone is done with the first half's Z
       store_z<1>(ZsT, acc, tx, ty, meta[pair], o.b_ok, rs, scale, map);
-      chain_tile<MQ, FF>();
+      chain_tile<MQ, MODE>(w.t + 2 == w.nt ? f.last : BN);
     }
     pair ^= 1;
   }
-  // The products of the Z tile (the first barrier in here makes it whole) with M, every 64 rows'
-  // sums added to the parked ones: words 0.. and, for FF (float-float, TwoSum), their low parts at
-  // 8 MQ..; short chains also keep the FP32 sums' rounding small
-  template <int MQ, bool FF>
-  __device__ __forceinline__ void chain_tile() {
-    // 64 rows at a time: half a stage, a stage, or several
-    const float* st = nullptr;
+  // The products of the Z tile's first `rows` rows (64 or 128; the first barrier in here makes it
+  // whole) with M, 64 rows at a time, into the sums parked at words 0..
+  //   CHAIN: one chain of multiply-adds per sum, through all tiles;
+  //   ADD:   every 64 rows' sums are added to them;
+  //   FF:    the same in float-float (TwoSum), the low parts at 8 MQ..
+  template <int MQ, int MODE>
+  __device__ __forceinline__ void chain_tile(int rows) {
+    const float* st = nullptr;   // half a stage, a stage, or several per 64 rows
 #pragma unroll 1
-    for (int n0 = 0; n0 < BN; n0 += 64) {
+    for (int n0 = 0; n0 < rows; n0 += 64) {
       f32x2 acc2[MQ][4];
 #pragma unroll
-      for (int q = 0; q < MQ; ++q)
+      for (int q = 0; q < MQ; ++q) {
+        float h[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (MODE == CHAIN) unpark8(park + 8 * q, h);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc2[q][i] = 0ull;
+        for (int i = 0; i < 4; ++i) acc2[q][i] = pair2(h[2 * i], h[2 * i + 1]);
+      }
       if (MR >= 64) {
         if (n0 % MR == 0) st = next();
         chain_fma<MQ, 64>(ZsT + n0 * ZLD, st + n0 % MR * o.mpad, o.mpad, tx, ty, acc2);
@@ -325,8 +329,12 @@ struct Body {
         float h[8], v[8];
 #pragma unroll
         for (int i = 0; i < 4; ++i) unpair2(acc2[q][i], v[2 * i], v[2 * i + 1]);
+        if (MODE == CHAIN) {
+          park8(park + 8 * q, v);
+          continue;
+        }
         unpark8(park + 8 * q, h);
-        if (FF) {
+        if (MODE == FF) {
           float l[8];
           unpark8(park + 8 * (MQ + q), l);
 #pragma unroll
@@ -392,7 +400,7 @@ __global__ void __launch_bounds__(NT, 1) k_pass2_simt(const __grid_constant__ Pa
   b.park_zeros((COMP ? 4 : 2) * MQ);
   while (!w.done()) {
     const int part = w.p;
-    b.template run<MQ, COMP>(w, rs, p.scale, p.map);
+    b.template run<MQ, COMP ? FF : ADD>(w, rs, p.scale, p.map);
     w.step();
     if (cl > 1 || w.p == part) continue;
     // the part's sum into the totals, and back to zero
@@ -487,7 +495,8 @@ __global__ void __launch_bounds__(NT, 1) k_pass2_simt(const __grid_constant__ Pa
 }
 
 // Pass 1: one CTA per (128 feature slots, row block i, row split); runs over the
-// data rows of its split in 128-row steps.  Writes R-partials (features x m_pad).
+// data rows of its split (whole runs of 64 rows) in 128-row tiles, one chain of multiply-adds per
+// sum.  Writes R-partials (features x m_pad).
 template <int MQ>
 __global__ void __launch_bounds__(NT, 1) k_pass1_simt(const __grid_constant__ PassArgs p) {
   extern __shared__ __align__(16) float smem[];
@@ -499,26 +508,26 @@ __global__ void __launch_bounds__(NT, 1) k_pass1_simt(const __grid_constant__ Pa
   while (j + 1 < p.C && p.col_slot[j + 1] <= a0) ++j;
   if (a0 - p.col_slot[j] >= p.col_size[j]) return;
   if (p.bmask && !p.bmask[i * p.C + j]) return;   // inactive block: its partials are not read
-  const int64_t r0 = p.row_slot[i], nsteps = ceil_div(p.row_size[i], BN);
+  const int64_t nsteps = ceil_div(p.row_size[i], 64);
   const int64_t t0 = split * nsteps / p.nsplit, t1 = (split + 1) * nsteps / p.nsplit;
+  const int64_t r0 = p.row_slot[i] + t0 * 64, tiles = ceil_div(t1 - t0, 2);
   const int64_t o = ((int64_t)split * p.R + i) * p.out_block_stride;
-  if (!RFF_SPAN(a0, BM, p.g_rows) || !RFF_SPAN(r0 + t0 * BN, (t1 - t0) * BN, p.x_rows) ||
-      !RFF_SPAN(j * p.m_block_stride + (r0 + t0 * BN) * p.mpad, (t1 - t0) * BN * p.mpad, p.m_elems) ||
+  if (!RFF_SPAN(a0, BM, p.g_rows) || !RFF_SPAN(r0, (t1 - t0) * 64, p.x_rows) ||
+      !RFF_SPAN(j * p.m_block_stride + r0 * p.mpad, (t1 - t0) * 64 * p.mpad, p.m_elems) ||
       !RFF_SPAN(o + a0 * p.mpad, BM * p.mpad, p.out_elems))
     return;
   if (threadIdx.x < 32) tc5::tmem_alloc<1>(tc5::smem_u32(&tmem_word), 512);
-  Walk w = make_walk(t1 - t0, 1, 0, 1);
+  Walk w = make_walk(tiles, 1, 0, 1);
   Body<m_rows(MQ)> b(smem, Operands{p.Gt + a0 * p.ldg, p.X, p.M + j * p.m_block_stride, nullptr, p.row_ok, p.ldg, p.ldx,
                                     p.K, p.mpad},
-                     r0 + t0 * BN, w);
+                     r0, w, (t1 - t0) % 2 ? 64 : BN);
   const RowSide rs = row_side(p.feat_ok, p.bias, a0);
   tc5::fence_before();
   __syncthreads();
   tc5::fence_after();
   b.park = park_base(tmem_word, 512);
   b.park_zeros(MQ);
-  for (; !w.done(); w.step())
-    b.template run<MQ, false>(w, rs, p.scale, p.map);
+  for (; !w.done(); w.step()) b.template run<MQ, CHAIN>(w, rs, p.scale, p.map);
   cp_wait<0>();   // (only empty groups are left)
   float* out = p.out + o + a0 * p.mpad;
 #pragma unroll
