@@ -526,67 +526,102 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
 // (bs = min(64, s - kcol)) in shared memory, write L back (upper part zeroed) and
 // the inverse of L into inv (64 x 64, zero padded).  info = column+1 of the first
 // non-positive pivot (the pivot is replaced by 1 so the factorisation finishes).
-// Step c of the right-looking factorisation also takes step c of the forward substitution
-// L X = I (X = L^-1, built in place of the identity: row c scaled by 1 / L_cc, then
-// X_rq -= L_rc X_cq for r > c, q <= c), so the inverse needs no sweep of its own.  The
-// trailing update walks only the pairs (r, q), c < q <= r, in an order where step c's pairs
-// are a prefix of one table (pair (r, q) at r'(r'+1)/2 + q', r' = 63 - q, q' = 63 - r): no lane
-// of a warp idles on this part's narrow FP64 pipe.  Every element sees the same operations in
-// the same order as the column-by-column forms of both sweeps.
+//
+// The factorisation runs as L D L^T with unit lower L: step c needs the reciprocal of pivot d_c
+// only, and one multiplication per element of the column, t_r = A_rc / d_c, before the updates
+//   A_rq -= t_r A_qc   (c < q <= r)      and, the forward substitution L X = I in place of the
+//   X_rq -= t_r X_cq   (r > c, q <= c)   identity, so that the inverse needs no sweep of its own;
+// the square roots of all pivots are taken together at the end (L_rc sqrt(d_c), X_rq / sqrt(d_r)).
+// X_rq takes the place of A_rq in M once column q has been eliminated, so that step c updates the
+// elements (r, q), q <= r, of every row r > c by the same rule, with u_q = A_qc for q > c and X_cq
+// for q <= c: a prefix of one table of the lower triangle's elements, last row first, in which
+// no lane of a warp idles.  Warp 0 updates the next pivot first and inverts it while the other
+// warps run the updates: on this part's 1/64-rate FP64 pipe a square root and a division in front
+// of every step's updates, by one thread, took as long as the updates.
+// Bound: that pipe (2 multiply-adds per clock and SM: 89k of them, 23 us).  measured 61 us
+// per 64 columns, 92 us with square root, division and column scaling in front of every step.
 __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ jobs, int kcol) {
+  __shared__ double M[64][65];
+  __shared__ double L[64][65];  // eliminated columns: A_rc at step c
+  __shared__ double col[64];    // t of the current step
+  __shared__ double u[64];
+  __shared__ double piv[64];    // the pivots d_c, then their square roots
+  __shared__ double rinv[64];   // 1 / d_c, then 1 / sqrt(d_c)
+  __shared__ uint16_t elem[64 * 65 / 2];   // (r << 8) | q, r = 63 first
+  __shared__ int bad;
+  const int tid = threadIdx.x;
+  for (int t = tid; t < 64 * 64; t += 256) {
+    const int r = t / 64, c = t % 64;
+    if (c <= r) elem[64 * 65 / 2 - (r + 1) * (r + 2) / 2 + c] = (uint16_t)((r << 8) | c);
+  }
+  if (tid == 0) bad = 0;
   const DiagJob jb = jobs[blockIdx.x];
   if (kcol >= jb.s) return;
   const int bs = min(64, jb.s - kcol);
-  __shared__ double L[64][65];
-  __shared__ double Li[64][65];
-  __shared__ double rinv[64];   // reciprocals of the pivots (one FP64 division each: this part's
-                                // FP64 division is a long sequence on its 1/64-rate pipe)
-  __shared__ uint16_t pairs[63 * 64 / 2];   // (r' << 8) | q', 0 <= q' <= r' < 63
-  __shared__ int bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) bad = 0;
+  // pivot c: positive, or recorded and replaced by 1
+  auto pivot = [&](int c, double d) {
+    if (!(d > 0.0)) {
+      if (bad == 0) bad = kcol + c + 1;
+      d = 1.0;
+    }
+    piv[c] = d;
+    // 1 / d by Newton's iteration from the FP32 reciprocal (within an ulp or two), shorter than a
+    // division: everything waits for it
+    const float f = (float)d;
+    double r;
+    if (f > 1e-30f && f < 1e30f) {
+      r = (double)(1.f / f);
+      r = fma(r, fma(-d, r, 1.0), r);
+      r = fma(r, fma(-d, r, 1.0), r);
+    } else {
+      r = 1.0 / d;
+    }
+    rinv[c] = r;
+  };
   for (int t = tid; t < 64 * 64; t += 256) {
     const int r = t / 64, c = t % 64;
-    L[r][c] = (r < bs && c < bs) ? jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] : (r == c ? 1.0 : 0.0);
-    Li[r][c] = r == c ? 1.0 : 0.0;
-    if (r < 63 && c <= r) pairs[r * (r + 1) / 2 + c] = (uint16_t)((r << 8) | c);
+    M[r][c] = (r < bs && c < bs) ? jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] : (r == c ? 1.0 : 0.0);
   }
   __syncthreads();
+  if (tid == 0) pivot(0, M[0][0]);
+  __syncthreads();
   for (int c = 0; c < bs; ++c) {
-    if (tid == 0) {
-      double d = L[c][c];
-      if (!(d > 0.0)) {
-        if (bad == 0) bad = kcol + c + 1;
-        d = 1.0;
-      }
-      L[c][c] = sqrt(d);
-      rinv[c] = 1.0 / L[c][c];
-    }
-    __syncthreads();
-    const double ri = rinv[c];
     if (tid < 64) {
-      if (c + 1 + tid < 64) L[c + 1 + tid][c] *= ri;
-    } else if (tid < 128) {
-      if (tid - 64 <= c) Li[c][tid - 64] *= ri;
+      double v;
+      if (tid > c) {
+        v = M[tid][c];
+        col[tid] = v * rinv[c];
+        L[tid][c] = v;
+        M[tid][c] = 0.0;   // X_rc starts from the identity's zero
+      } else {
+        v = tid == c ? 1.0 : M[c][tid];
+      }
+      u[tid] = tid == c ? 1.0 : v;
     }
     __syncthreads();
-    const int w = 63 - c, cw = c + 1;
-    for (int p = tid; p < w * (w + 1) / 2; p += 256) {
-      const uint32_t v = pairs[p];
-      const int r = 63 - (int)(v & 0xffu), q = 63 - (int)(v >> 8);
-      L[r][q] -= L[r][c] * L[q][c];
-    }
-    for (int t = tid; t < w * cw; t += 256) {
-      const int r = c + 1 + t / cw, q = t % cw;
-      Li[r][q] -= L[r][c] * Li[c][q];
+    if (tid == 0 && c + 1 < bs) pivot(c + 1, M[c + 1][c + 1] - col[c + 1] * u[c + 1]);
+    if (tid >= 32) {
+      const int len = 64 * 65 / 2 - (c + 1) * (c + 2) / 2 - 1;   // (the last element is the next pivot)
+#pragma unroll 2
+      for (int p = tid - 32; p < len; p += 224) {
+        const uint32_t v = elem[p];
+        const int r = (int)(v >> 8), q = (int)(v & 0xffu);
+        M[r][q] -= col[r] * u[q];
+      }
     }
     __syncthreads();
   }
+  if (tid < bs) {
+    const double s = sqrt(piv[tid]);
+    piv[tid] = s;
+    rinv[tid] = 1.0 / s;
+  }
+  __syncthreads();
   for (int t = tid; t < 64 * 64; t += 256) {
     const int r = t / 64, c = t % 64;
     const bool in = r < bs && c < bs;
-    if (in) jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] = (c <= r) ? L[r][c] : 0.0;
-    jb.inv[t] = in ? Li[r][c] : 0.0;
+    if (in) jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] = c < r ? L[r][c] * rinv[c] : c == r ? piv[r] : 0.0;
+    jb.inv[t] = in && c <= r ? (c < r ? M[r][c] : 1.0) * rinv[r] : 0.0;
   }
   if (tid == 0 && bad && jb.info && *jb.info == 0) *jb.info = bad;
 }
