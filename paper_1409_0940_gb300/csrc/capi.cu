@@ -1278,7 +1278,8 @@ rff_status setup_factors(rff_admm_t h) {
     CK(launch_factor_init(jobs, s.st));
     // Q is stored to 24 bits (FP32, or three BF16 pieces): updates that keep 40 bits of every
     // operand leave it within cond(H) 2^-40 (about 2e-9 at cond 2.3e3), far inside that
-    CK(factor_and_invert_f64(jobs, true, fscr, s.st, true, 40));
+    // (a memory limit leaves no room for the buffers of the overlap)
+    CK(factor_and_invert_f64(jobs, true, fscr, s.st, true, 40, s.mem_limit == 0));
     if (s.split_path() && !s.outer) {
       for (int64_t bb = 0; bb < nb; ++bb)
         CK(launch_split3_q(Q64 + bb * fmax * fmax, jobs[bb].s, s.ldq, s.qrow[b0 + bb], s.Q1, s.Q2, s.Q3, s.st));

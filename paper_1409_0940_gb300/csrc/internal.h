@@ -185,9 +185,11 @@ cudaError_t launch_convert_factors(const std::vector<MatJob>& jobs, float* const
 size_t factor_scratch_bytes(int njobs, int smax);
 // blocked Cholesky (and inverse); double_float selects the double-float GEMM for the block
 // updates under RFF_FACTOR=df (the 64 x 64 diagonal factorisations stay FP64); oz_bits: the
-// leading bits of every update operand the tensor-core updates keep (48 or 40)
+// leading bits of every update operand the tensor-core updates keep (48 or 40); overlap: the
+// factorisation and the forward sweep of the inverse may run side by side, on a stream and
+// buffers of the call's own (results are the same; without the memory they run in turn)
 cudaError_t factor_and_invert_f64(const std::vector<MatJob>& jobs, bool invert, void* dev_scratch, cudaStream_t st,
-                                  bool double_float = false, int oz_bits = 48);
+                                  bool double_float = false, int oz_bits = 48, bool overlap = false);
 // Q[r][c] = Q[c][r] for c > r, every job with a Q
 cudaError_t launch_mirror_lower(const std::vector<MatJob>& jobs, cudaStream_t st);
 
@@ -195,7 +197,7 @@ cudaError_t launch_mirror_lower(const std::vector<MatJob>& jobs, cudaStream_t st
 // slices of the FP64 operands); factor_and_invert_f64 calls it unless RFF_FACTOR=df
 size_t oz_factor_scratch_bytes(int njobs, int smax);
 cudaError_t factor_and_invert_oz(const std::vector<MatJob>& jobs, bool invert, void* dev_scratch, cudaStream_t st,
-                                 int bits);
+                                 int bits, bool overlap);
 
 // elementwise.cu
 // dst[p][c] = src[map[p] * lds + c] (c < w), zero for c >= w or map[p] < 0; map null = identity
