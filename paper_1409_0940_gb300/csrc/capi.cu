@@ -433,6 +433,7 @@ void compute_geometry(rff_admm_s& s, int64_t n, int64_t d) {
 // hi/lo pair and 128 x 256 tiles of Z^T Z over 512-row pieces of K, GRAM_GROUP pieces per
 // launch, their partial tiles summed into H in FP64.
 constexpr int GRAM_KCH = 512, GRAM_GROUP = 16;
+constexpr size_t TS_WHOLE_BYTES = size_t(1) << 30;     // TensorSketch: the most FP32 Z formed at once
 constexpr size_t OUTER_ZT_BYTES = size_t(256) << 20;   // outer form: the most Z^T formed at once
 
 int64_t tc_gram_tiles(int64_t smax, std::vector<int2>* out = nullptr) {
@@ -910,17 +911,19 @@ TsArgs ts_args(const rff_admm_s& s, const float* X, int64_t ldx, const int32_t* 
 
 int64_t ts_block_max(const rff_admm_s& s) { return *std::max_element(s.col_size.begin(), s.col_size.end()); }
 
-rff_status materialise_z(rff_admm_t h) {
+// whole: FP32 Z of every row slot (ld fslots), already formed at the start of the scratch, or null
+rff_status materialise_z(rff_admm_t h, const float* whole = nullptr) {
   NvtxRange range("rff set-up: materialise Z");
   auto& s = *h;
-  const int64_t chunk = materialise_chunk(s);
+  const int64_t chunk = whole ? s.nslots : materialise_chunk(s);
   rff_status rs = ensure_scratch(h, (size_t)chunk * s.fslots * 4);
   if (rs != RFF_OK) return rs;
   float* zc = static_cast<float*>(s.scratch.p);
   s.zscale = pow2_scale(s.zmap_scale());   // |Z| <= sqrt(2/D) (cos) or 1/sqrt(D) (exp(-T))
   for (int64_t r0 = 0; r0 < s.nslots; r0 += chunk) {
     const int64_t nr = std::min(chunk, s.nslots - r0);
-    if (s.tensorsketch()) {
+    if (whole) {
+    } else if (s.tensorsketch()) {
       TsArgs ta = ts_args(s, s.X32, s.dld, s.row_of_slot, r0, nr);
       ta.out = zc;
       ta.ldo = s.fslots;
@@ -1156,18 +1159,39 @@ rff_status setup_factors(rff_admm_t h) {
     rff_status r = generate_features(h);
     if (r != RFF_OK) return r;
   }
+  // The sketches have no a-priori bound: a pass over the training rows measures max |z|, the
+  // scale of Z's FP16 split (and of the Gram's).  Where an FP32 Z of all rows is no larger than
+  // TS_WHOLE_BYTES and an eighth of the free memory, that pass also forms it (a sketch costs far
+  // more than writing it out), else Z is sketched again in row chunks.
+  const size_t ts_bytes = (size_t)s.nslots * s.fslots * 4;
+  bool ts_whole = false;
   if (s.tensorsketch()) {
-    // the sketches have no a-priori bound: one pass over the training rows measures max |z|,
-    // the scale of Z's FP16 split (and of the Gram's)
+    size_t free_b = 0, total_b = 0;
+    CK(cudaMemGetInfo(&free_b, &total_b));
+    ts_whole = !s.mem_limit && ts_bytes <= std::min(TS_WHOLE_BYTES, free_b / 8);
+    if (ts_whole && ensure_scratch(h, ts_bytes) != RFF_OK) {
+      h->err.clear();
+      ts_whole = false;
+    }
     unsigned* bits = reinterpret_cast<unsigned*>(s.flag + 3);
     CK(cudaMemsetAsync(bits, 0, 4, s.st));
     TsArgs ta = ts_args(s, s.X32, s.dld, s.row_of_slot, 0, s.nslots);
     ta.amax = bits;
+    if (ts_whole) {
+      ta.out = static_cast<float*>(s.scratch.p);
+      ta.ldo = s.fslots;
+      ta.out_elems = s.nslots * s.fslots;
+      ta.pad = 1;
+    }
     CK(launch_tensorsketch(ta, s.C, ts_block_max(s), s.st));
     unsigned hb = 0;
     CK(cudaMemcpyAsync(&hb, bits, 4, cudaMemcpyDeviceToHost, s.st));
     CK(cudaStreamSynchronize(s.st));
     memcpy(&s.ts_zmax, &hb, 4);
+    if (ts_whole) {
+      rff_status zr = materialise_z(h, static_cast<float*>(s.scratch.p));
+      if (zr != RFF_OK) return zr;
+    }
   }
   const float scale = s.zmap_scale();
   // Gram matrices H_ij = I + Z_ij^T Z_ij (eq. (cache)), or I + Z_ij Z_ij^T in the outer
@@ -1201,10 +1225,10 @@ rff_status setup_factors(rff_admm_t h) {
   budget = budget > zbytes + (256u << 20) ? budget - zbytes - (256u << 20) : 0;
   int64_t batch = std::max<int64_t>(1, std::min<int64_t>(nblocks, (int64_t)(budget / std::max<size_t>(per_block + factor_scratch_bytes(1, (int)fmax), 1))));
   size_t need = (size_t)batch * per_block + zbytes + factor_scratch_bytes((int)batch, (int)fmax) + (size_t)batch * 4 + 4096;
-  if (s.cached_z()) need = std::max(need, (size_t)materialise_chunk(s) * s.fslots * 4);
+  if (s.cached_z() && !ts_whole) need = std::max(need, (size_t)materialise_chunk(s) * s.fslots * 4);
   rff_status rs = ensure_scratch(h, need);
   if (rs != RFF_OK) return rs;
-  if (s.cached_z()) {   // Z and Z^T's splits first: the Gram below reads the stored Z^T
+  if (s.cached_z() && !ts_whole) {   // Z and Z^T's splits first: the Gram below reads the stored Z^T
     rff_status zr = materialise_z(h);
     if (zr != RFF_OK) return zr;
   }
