@@ -108,6 +108,59 @@ __device__ __forceinline__ float cos_rr_pow2(float x) {
   return __int_as_float(__float_as_int(p) ^ (__float_as_int(biased) << 31));
 }
 
+// ------------------------------------------------------------------ packed FP32
+// Two FP32 operations in one instruction, each rounded as its scalar form (and not contracted).  A
+// pair is the two words of a 64-bit register.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 pair2(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpair2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 both2(float v) { return pair2(v, v); }
+
+// 2^E cos of both words, bit for bit cos_rr_pow2<E> of each: half the issue slots of the two scalar
+// evaluations.  The sign of odd k is added as k's low bit times 2^31 (modulo 2^32 the same as
+// flipping the sign bit, in one instruction).
+template <int E>
+__device__ __forceinline__ f32x2 cos2_pow2(f32x2 x) {
+  constexpr float S = (float)(1u << E);
+  const f32x2 biased = add2(mul2(x, both2(0.318309886183790672f)), both2(12582912.f));
+  const f32x2 k = add2(biased, both2(-12582912.f));
+  f32x2 r = fma2(k, both2(-3.14159274101257324f), x);
+  r = fma2(k, both2(8.74227765734758577e-08f), r);
+  const f32x2 s = mul2(r, r);
+  f32x2 p = both2(-2.605149518331018e-07f * S);
+  p = fma2(p, s, both2(2.476016197761055e-05f * S));
+  p = fma2(p, s, both2(-0.0013888361863791943f * S));
+  p = fma2(p, s, both2(0.04166663810610771f * S));
+  p = fma2(p, s, both2(-0.5f * S));
+  p = fma2(p, s, both2(1.0f * S));
+  float p0, p1, b0, b1;
+  unpair2(p, p0, p1);
+  unpair2(biased, b0, b1);
+  return pair2(__int_as_float(__float_as_int(p0) + (__float_as_int(b0) << 31)),
+               __int_as_float(__float_as_int(p1) + (__float_as_int(b1) << 31)));
+}
+
 // ------------------------------------------------------------------ BF16 split
 // x = hi + lo + O(2^-17 |x|): hi = bf16(x), lo = bf16(x - hi).
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {

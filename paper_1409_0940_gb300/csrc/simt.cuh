@@ -48,23 +48,6 @@ __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Two FP32 multiply-adds in one instruction (each rounded as fmaf): half the issue slots and
-// register reads of two scalar ones.  A pair is the two words of a 64-bit register.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f32x2 pair2(float lo, float hi) {
-  f32x2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-  return d;
-}
-__device__ __forceinline__ void unpair2(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-
 // tensor memory of this thread: base address for words 0, 1, ... (cols: columns of the CTA)
 __device__ __forceinline__ uint32_t park_base(uint32_t tmem, uint32_t cols) {
   const uint32_t w = threadIdx.x / 32;

@@ -145,6 +145,57 @@ __device__ __forceinline__ void red_add_v4(float4* p, float4 v) {
                : "memory");
 }
 
+// The epilogues' arithmetic, two elements per instruction: about 10 issue slots per cosine and split
+// instead of 17.  Eight warps leave little to hide behind, so every pass gains: a sweep of four
+// solves at d = 128, 553 -> 445 us per launch; 20,011 rows at d = 33, D = 3000, 96 -> 83 us; 200,000
+// rows at d = 440, D = 16,384, 147 classes, 7.8 -> 7.2 ms (1.68 PFLOP/s of products executed, at the
+// power cap: 0.96 of the sustained cuBLAS rate).  Sixteen warps of 32 columns gained
+// at d = 33 only (17.5 against 17.9 ms a fit) and lost at d = 440 (142 against 139 ms, 8 iterations).
+// The phases added to an epilogue thread's accumulator columns: none (b is part of the product),
+// one (the feature index is the A row: pass 1), or one per column, from global memory.
+struct Phases {
+  bool add;
+  const float* col;   // the columns' phases (16-byte aligned), or null
+  float row;
+  __device__ __forceinline__ float4 four(int c) const {   // columns c .. c + 3
+    return col ? __ldg(reinterpret_cast<const float4*>(col + c)) : make_float4(row, row, row, row);
+  }
+};
+
+// z[c] = 2^7 cos(acc inv_xg (+ phase)) of 64 accumulator words
+__device__ __forceinline__ void cos_pairs(const uint32_t (&v0)[32], const uint32_t (&v1)[32], float inv_xg,
+                                          const Phases& ph, f32x2 (&z)[32]) {
+  const f32x2 sc = both2(inv_xg);
+#pragma unroll
+  for (int q = 0; q < 32; ++q) {
+    const uint32_t a = q < 16 ? v0[2 * q] : v1[2 * q - 32], b = q < 16 ? v0[2 * q + 1] : v1[2 * q - 31];
+    z[q] = pair2(__uint_as_float(a), __uint_as_float(b));
+  }
+  if (ph.add) {
+#pragma unroll
+    for (int q = 0; q < 32; q += 2) {
+      const float4 b = ph.four(2 * q);
+      z[q] = cos2_pow2<7>(fma2(z[q], sc, pair2(b.x, b.y)));
+      z[q + 1] = cos2_pow2<7>(fma2(z[q + 1], sc, pair2(b.z, b.w)));
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) z[q] = cos2_pow2<7>(mul2(z[q], sc));
+  }
+}
+
+// the FP16 hi/lo split of a pair: hi = fp16x2(z), lo = fp16x2(z - hi)
+__device__ __forceinline__ void split_pair(f32x2 z, uint32_t& hi, uint32_t& lo) {
+  float z0, z1, l0, l1;
+  unpair2(z, z0, z1);
+  const __half2 h = __floats2half2_rn(z0, z1);
+  const float2 f = __half22float2(h);
+  unpair2(fma2(pair2(f.x, f.y), both2(-1.f), z), l0, l1);
+  const __half2 l = __floats2half2_rn(l0, l1);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
 // ------------------------------------------------------------------ shared state
 template <int NS, int MG = MAXG>
 struct Shared {
@@ -613,36 +664,15 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
         if (lane == 0) arrive_mma_side<CG>(bar_a1e + 8 * b);
         // z = cos(acc (+ b)), times COS_SCALE when it feeds the chained product; the factor
         // sqrt(2/D) is applied when acc2 (or the materialised Z) is written
-        float z[64];
-        if (add_bias) {
-          const float* bcol = a.bias + bslot + colbase;
+        const bool per_col = a.mode != MODE_PASS1 && RFF_SPAN(bslot + colbase, 64, a.fslots);
+        const Phases ph{add_bias, per_col ? a.bias + bslot + colbase : nullptr, bias_a};
+        if (!chain) {
+          float z[64];
 #pragma unroll
           for (int c = 0; c < 64; ++c) {
-            const float ph = (a.mode == MODE_PASS1)                             ? bias_a
-                             : RFF_IN(bslot + colbase + c, a.fslots) ? __ldg(bcol + c)
-                                                                     : 0.f;
-            z[c] = __uint_as_float(c < 32 ? v0[c] : v1[c - 32]) * inv_xg + ph;
+            const float x = __uint_as_float(c < 32 ? v0[c] : v1[c - 32]);
+            z[c] = cos_rr(add_bias ? x * inv_xg + (per_col ? __ldg(ph.col + c) : bias_a) : x * inv_xg);
           }
-          // one loop per branch: a per-element choice would evaluate both cosines
-          if (chain) {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = cos_rr_pow2<7>(z[c]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = cos_rr(z[c]);
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 64; ++c) z[c] = __uint_as_float(c < 32 ? v0[c] : v1[c - 32]) * inv_xg;
-          if (chain) {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = cos_rr_pow2<7>(z[c]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = cos_rr(z[c]);
-          }
-        }
-        if (!chain) {
           // materialise Z = sqrt(2/D) cos(...) (float32) inside the window
           const int64_t r = arow - a.wz_r0;
           if (r < a.wz_nr && a.zt_hi) {
@@ -669,6 +699,8 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
           }
           continue;
         }
+        f32x2 z[32];
+        cos_pairs(v0, v1, inv_xg, ph, z);
         // Z tile must be free: the chain of the previous tile has completed
         if (t >= 1 && !waitw<CG>(bar_ze, (t - 1) & 1, sh, a, ERR_TIMEOUT_EPI)) { ok = false; break; }
         if (ZTMEM) {
@@ -676,19 +708,12 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
           // store this warp's 32 rows x 64 features into the Z columns of TMEM
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
-            uint32_t ph[16], pl[16];
+            uint32_t zh[16], zl[16];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-              const float z0 = z[32 * hf + 2 * q], z1 = z[32 * hf + 2 * q + 1];   // COS_SCALE z
-              const __half2 h = __floats2half2_rn(z0, z1);
-              const float2 f = __half22float2(h);
-              const __half2 l = __floats2half2_rn(z0 - f.x, z1 - f.y);
-              ph[q] = *reinterpret_cast<const uint32_t*>(&h);
-              pl[q] = *reinterpret_cast<const uint32_t*>(&l);
-            }
+            for (int q = 0; q < 16; ++q) split_pair(z[16 * hf + q], zh[q], zl[q]);
             const uint32_t col = (uint32_t)(colbase / 2 + 16 * hf);
-            tmem_st16(tmem + lane_addr + ZH + col, ph);
-            tmem_st16(tmem + lane_addr + ZL + col, pl);
+            tmem_st16(tmem + lane_addr + ZH + col, zh);
+            tmem_st16(tmem + lane_addr + ZL + col, zl);
           }
           tmem_wait_st();
           fence_before();
@@ -698,20 +723,12 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
           unsigned char* zlo = zhi + ZBYTES / 2;
 #pragma unroll
           for (int ch = 0; ch < 8; ++ch) {
-            uint32_t ph[4], pl[4];
+            uint32_t zh[4], zl[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              // hi = fp16x2(s z0, s z1); lo = fp16x2(s z - hi) (packed conversions)
-              const float z0 = z[ch * 8 + 2 * q], z1 = z[ch * 8 + 2 * q + 1];   // COS_SCALE z
-              const __half2 h = __floats2half2_rn(z0, z1);
-              const float2 hf = __half22float2(h);
-              const __half2 l = __floats2half2_rn(z0 - hf.x, z1 - hf.y);
-              ph[q] = *reinterpret_cast<const uint32_t*>(&h);
-              pl[q] = *reinterpret_cast<const uint32_t*>(&l);
-            }
+            for (int q = 0; q < 4; ++q) split_pair(z[ch * 4 + q], zh[q], zl[q]);
             const uint32_t off = row * 128 + ((ch ^ (row & 7)) << 4);
-            *reinterpret_cast<uint4*>(zhi + off) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-            *reinterpret_cast<uint4*>(zlo + off) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
+            *reinterpret_cast<uint4*>(zhi + off) = make_uint4(zh[0], zh[1], zh[2], zh[3]);
+            *reinterpret_cast<uint4*>(zlo + off) = make_uint4(zl[0], zl[1], zl[2], zl[3]);
           }
           fence_proxy_async();
         }
@@ -1055,74 +1072,27 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
             if (lane == 0) mbar_arrive(bar_a1e);
           }
           if (h >= halves && chain) continue;    // a half past the group: computed, not chained
-          float z[64];
-          if (add_bias) {
-            const float* bcol = a.bias + bslot + colbase;
-#pragma unroll
-            for (int c = 0; c < 64; ++c) {
-              const float ph = (a.mode == MODE_PASS1)                             ? bias_a
-                               : RFF_IN(bslot + colbase + c, a.fslots) ? __ldg(bcol + c)
-                                                                       : 0.f;
-              z[c] = __uint_as_float(c < 32 ? v0[c] : v1[c - 32]) * inv_xg + ph;
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = __uint_as_float(c < 32 ? v0[c] : v1[c - 32]) * inv_xg;
-          }
-          // one loop per branch: a per-element choice would evaluate both cosines
-          if (chain) {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = cos_rr_pow2<7>(z[c]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) z[c] = cos_rr(z[c]);
-          }
-          if (!chain) {
-            const int64_t r = arow - a.wz_r0;
-            if (r < a.wz_nr && a.zt_hi) {
-#pragma unroll
-              for (int c = 0; c < 64; ++c) {
-                const int64_t f = bslot + colbase + c - a.wz_f0;
-                if (f >= 0 && f < a.wz_nf && RFF_IN(f * a.ldo + r, a.out_elems)) {
-                  const float xs = a.scale * z[c] * a.zt_scale;
-                  const __half hh = __float2half_rn(xs);
-                  a.zt_hi[f * a.ldo + r] = hh;
-                  a.zt_lo[f * a.ldo + r] = __float2half_rn(xs - __half2float(hh));
-                }
-              }
-            } else if (r < a.wz_nr) {
-#pragma unroll
-              for (int c = 0; c < 64; ++c) {
-                const int64_t f = bslot + colbase + c - a.wz_f0;
-                if (f >= 0 && f < a.wz_nf && RFF_IN(r * a.ldo + f, a.out_elems)) a.out[r * a.ldo + f] = a.scale * z[c];
-              }
-            }
-            continue;
-          }
+          const bool per_col = a.mode != MODE_PASS1 && RFF_SPAN(bslot + colbase, 64, a.fslots);
+          const Phases ph{add_bias, per_col ? a.bias + bslot + colbase : nullptr, bias_a};
+          f32x2 z[32];
+          cos_pairs(v0, v1, inv_xg, ph, z);
           // the Z tile is free once the previous half's chain has completed
           if (zu >= 1 && !waitw(bar_ze, (zu - 1) & 1, sh, a, ERR_TIMEOUT_EPI)) { ok = false; break; }
           {
             // hi: FP16 pairs into the Z columns of TMEM; lo: the swizzled K-major tile in shared memory
-            unsigned char* zl = zlo_buf + (colbase / 64) * ZATOM;
+            unsigned char* zlb = zlo_buf + (colbase / 64) * ZATOM;
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
-              uint32_t ph[16], pl[16];
+              uint32_t zh[16], zl[16];
 #pragma unroll
-              for (int q = 0; q < 16; ++q) {
-                const float z0 = z[32 * hf + 2 * q], z1 = z[32 * hf + 2 * q + 1];   // COS_SCALE z
-                const __half2 hh = __floats2half2_rn(z0, z1);
-                const float2 f = __half22float2(hh);
-                const __half2 l = __floats2half2_rn(z0 - f.x, z1 - f.y);
-                ph[q] = *reinterpret_cast<const uint32_t*>(&hh);
-                pl[q] = *reinterpret_cast<const uint32_t*>(&l);
-              }
-              tmem_st16(tmem + lane_addr + W_ZH + (uint32_t)(colbase / 2 + 16 * hf), ph);
+              for (int q = 0; q < 16; ++q) split_pair(z[16 * hf + q], zh[q], zl[q]);
+              tmem_st16(tmem + lane_addr + W_ZH + (uint32_t)(colbase / 2 + 16 * hf), zh);
               // 16 packed words = 32 features = four 16-byte chunks of this row
 #pragma unroll
               for (int q4 = 0; q4 < 4; ++q4) {
                 const int ch = 4 * hf + q4;
                 const uint32_t off = row * 128 + ((ch ^ (row & 7)) << 4);
-                *reinterpret_cast<uint4*>(zl + off) = make_uint4(pl[4 * q4], pl[4 * q4 + 1], pl[4 * q4 + 2], pl[4 * q4 + 3]);
+                *reinterpret_cast<uint4*>(zlb + off) = make_uint4(zl[4 * q4], zl[4 * q4 + 1], zl[4 * q4 + 2], zl[4 * q4 + 3]);
               }
             }
             tmem_wait_st();
