@@ -108,6 +108,7 @@ constexpr int ERR_TIMEOUT_PRODUCER = 1, ERR_TIMEOUT_MMA = 2, ERR_TIMEOUT_EPI = 4
 struct TcArgs {
   CUtensorMap tA_hi, tA_lo, tB_hi, tB_lo, tM_hi, tM_lo;   // B and M boxes: 128/CG and m_pad/CG rows
   int mode, nk, mpad, R, C, nsplit;
+  int mchunks;                              // chained-operand chunks per ring stage (see chain_chunks)
   int64_t a_rows;                           // scoring: valid query rows (CTA pairs discard the rest)
   const float* bias;
   const int32_t* a_ok;
@@ -473,6 +474,7 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
   fence_after();
   const uint32_t tmem = sh.tmem_base;
   const int nk = a.nk;
+  const int mchunks = a.mchunks;
   const int mrows = a.mpad / CG;                          // chain-operand rows this CTA holds
   const uint32_t mbytes = (uint32_t)mrows * RG::ROWB;     // one chain operand chunk (hi or lo)
 
@@ -500,13 +502,15 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
         return s;
       };
       auto load_chain = [&](int64_t bslot) -> bool {
-        for (int c = 0; c < RG::CHUNKS; ++c) {
-          const int s = acquire(2 * mbytes);
+        for (int c = 0; c < RG::CHUNKS; c += mchunks) {
+          const int s = acquire(mchunks * 2 * mbytes);
           if (s < 0) return false;
-          const uint32_t dst = smem_u32(stages + s * STAGE_BYTES);
           const int my = prev_my + (int)rank * mrows;
-          load(dst, &a.tM_hi, (int)(bslot + KC * c), my, s);
-          load(dst + mbytes, &a.tM_lo, (int)(bslot + KC * c), my, s);
+          for (int u = 0; u < mchunks; ++u) {
+            const uint32_t dst = smem_u32(stages + s * STAGE_BYTES) + u * 2 * mbytes;
+            load(dst, &a.tM_hi, (int)(bslot + KC * (c + u)), my, s);
+            load(dst + mbytes, &a.tM_lo, (int)(bslot + KC * (c + u)), my, s);
+          }
         }
         return true;
       };
@@ -555,10 +559,12 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
         fence_after();
         const uint32_t zhi = smem_u32(zbuf), zlo = zhi + ZBYTES / 2;
         for (int c = 0; c < RG::CHUNKS; ++c) {
-          const int s = it % NSTAGE;
-          if (!wait1<CG>(bar_full + 8 * s, (it / NSTAGE) & 1, sh, a, ERR_TIMEOUT_MMA)) return false;
-          fence_after();
-          const uint32_t mhi = smem_u32(stages + s * STAGE_BYTES), mlo = mhi + mbytes;
+          const int s = it % NSTAGE, u = c & (mchunks - 1);   // chunk u of its stage
+          if (u == 0) {
+            if (!wait1<CG>(bar_full + 8 * s, (it / NSTAGE) & 1, sh, a, ERR_TIMEOUT_MMA)) return false;
+            fence_after();
+          }
+          const uint32_t mhi = smem_u32(stages + s * STAGE_BYTES) + u * 2 * mbytes, mlo = mhi + mbytes;
 #pragma unroll
           for (int kk = 0; kk < RG::KSTEPS; ++kk) {
             const int zk = c * RG::KSTEPS + kk;                 // K step within the 128-wide Z tile
@@ -579,8 +585,10 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
               mma_ss<CG>(tmem + A2, dzl, dmh, id2, 1u);
             }
           }
-          commit_both<CG>(bar_empty + 8 * s);
-          ++it;
+          if (u == mchunks - 1) {
+            commit_both<CG>(bar_empty + 8 * s);
+            ++it;
+          }
         }
         commit_both<CG>(bar_ze);
         if (last) commit_both<CG>(bar_a2f);
@@ -865,7 +873,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
   unsigned char* stages = base + RG::ZLO;
   Shared<NSTAGE, W_MAXG>& sh = *reinterpret_cast<Shared<NSTAGE, W_MAXG>*>(stages + NSTAGE * STAGE_BYTES);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const bool chain = a.mode != MODE_WRITEZ;
 
   if (threadIdx.x == 0)
     plan_work<1>(a, sh, 0, CtaPos{(int64_t)blockIdx.x, (int64_t)gridDim.x, (int)blockIdx.y, (int)blockIdx.z});
@@ -900,6 +907,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
   const uint32_t tmem = sh.tmem_base;
   const int nk = a.nk;
   const uint32_t mbytes = (uint32_t)a.mpad * RG::ROWB;    // one chain operand chunk (hi or lo)
+  const int mchunks = a.mchunks;
 
   if (warp == 0) {
     // ================= TMA producer =================
@@ -920,13 +928,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
       };
       auto load_chain = [&]() -> bool {
         for (int h = 0; h < prev_halves; ++h)
-          for (int c = 0; c < RG::CHUNKS; ++c) {
-            const int s = acquire(2 * mbytes);
+          for (int c = 0; c < RG::CHUNKS; c += mchunks) {
+            const int s = acquire(mchunks * 2 * mbytes);
             if (s < 0) return false;
-            const uint32_t dst = smem_u32(stages + s * STAGE_BYTES);
-            const int x = (int)(prev_b + 128 * h + KC * c);
-            tma_load_2d(dst, &a.tM_hi, x, prev_my, bar_full + 8 * s);
-            tma_load_2d(dst + mbytes, &a.tM_lo, x, prev_my, bar_full + 8 * s);
+            for (int u = 0; u < mchunks; ++u) {
+              const uint32_t dst = smem_u32(stages + s * STAGE_BYTES) + u * 2 * mbytes;
+              const int x = (int)(prev_b + 128 * h + KC * (c + u));
+              tma_load_2d(dst, &a.tM_hi, x, prev_my, bar_full + 8 * s);
+              tma_load_2d(dst + mbytes, &a.tM_lo, x, prev_my, bar_full + 8 * s);
+            }
           }
         return true;
       };
@@ -944,13 +954,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
             tma_load_2d(dst + 2 * TILE_BYTES, &a.tB_hi, kc * KC, (int)bslot, fb);
             tma_load_2d(dst + 2 * TILE_BYTES + BTILE_BYTES, &a.tB_lo, kc * KC, (int)bslot, fb);
           }
-          if (ok && chain && prev_b >= 0) ok = load_chain();
+          if (ok && prev_b >= 0) ok = load_chain();
           prev_b = bslot;
           prev_my = sh.g_my[g];
           prev_halves = (lt + 1 < ntg) ? 2 : 1;
         }
       }
-      if (ok && chain && prev_b >= 0) ok = load_chain();
+      if (ok && prev_b >= 0) ok = load_chain();
       for (uint32_t u = (it > NSTAGE ? it - NSTAGE : 0); u < it; ++u) {
         const int s = u % NSTAGE;
         if (!mbar_try(bar_full + 8 * s, (u / NSTAGE) & 1)) {
@@ -977,10 +987,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
           fence_after();
           const uint32_t zlo = smem_u32(zlo_buf);
           for (int c = 0; c < RG::CHUNKS; ++c) {
-            const int s = it % NSTAGE;
-            if (!wait1(bar_full + 8 * s, (it / NSTAGE) & 1, sh, a, ERR_TIMEOUT_MMA)) return false;
-            fence_after();
-            const uint32_t mhi = smem_u32(stages + s * STAGE_BYTES), mlo = mhi + mbytes;
+            const int s = it % NSTAGE, u = c & (mchunks - 1);   // chunk u of its stage
+            if (u == 0) {
+              if (!wait1(bar_full + 8 * s, (it / NSTAGE) & 1, sh, a, ERR_TIMEOUT_MMA)) return false;
+              fence_after();
+            }
+            const uint32_t mhi = smem_u32(stages + s * STAGE_BYTES) + u * 2 * mbytes, mlo = mhi + mbytes;
 #pragma unroll
             for (int kk = 0; kk < RG::KSTEPS; ++kk) {
               const int zk = c * RG::KSTEPS + kk;
@@ -993,8 +1005,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
               mma_bf16_ts(tmem + W_A2, azh, dml, id2, 1u);
               mma_bf16(tmem + W_A2, sw128_desc(zlo + zo), dmh, id2, 1u);
             }
-            mma_commit(bar_empty + 8 * s);
-            ++it;
+            if (u == mchunks - 1) {
+              mma_commit(bar_empty + 8 * s);
+              ++it;
+            }
           }
           mma_commit(bar_ze);
           if (last && h == halves - 1) mma_commit(bar_a2f);
@@ -1028,14 +1042,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
           }
           if (!ok) break;
           mma_commit(bar_a1f);
-          if (chain && pg >= 0) ok = do_chain(pg, pfirst, plast, phalves);
+          if (pg >= 0) ok = do_chain(pg, pfirst, plast, phalves);
           pg = g;
           pfirst = lt == 0;
           plast = lt + 2 >= ntg;
           phalves = (lt + 1 < ntg) ? 2 : 1;
         }
       }
-      if (ok && chain && pg >= 0) ok = do_chain(pg, pfirst, plast, phalves);
+      if (ok && pg >= 0) ok = do_chain(pg, pfirst, plast, phalves);
       mma_commit(bar_done);
       wait1(bar_done, 0, sh, a, ERR_TIMEOUT_MMA);
     }
@@ -1071,7 +1085,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_a1e);
           }
-          if (h >= halves && chain) continue;    // a half past the group: computed, not chained
+          if (h >= halves) continue;    // a half past the group: computed, not chained
           const bool per_col = a.mode != MODE_PASS1 && RFF_SPAN(bslot + colbase, 64, a.fslots);
           const Phases ph{add_bias, per_col ? a.bias + bslot + colbase : nullptr, bias_a};
           f32x2 z[32];
@@ -1104,7 +1118,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
           ++zu;
         }
         if (!ok) break;
-        if (chain && lt + 2 >= ntg) {
+        if (lt + 2 >= ntg) {
           if (!waitw(bar_a2f, g & 1, sh, a, ERR_TIMEOUT_EPI)) { ok = false; break; }
           fence_after();
           if (sh.g_out[g]) {
@@ -1298,10 +1312,24 @@ int view_mrows(const TcView& v) { return (int)v.mpad / view_cg(v); }
 // grid x extent of a launch over `units` 128-row A tiles: a CTA pair takes two
 int64_t tile_grid(const TcView& v, int64_t units) { return view_cg(v) == 2 ? 2 * ceil_div(units, 2) : units; }
 
+// Chunks of the chained operand (KC of a tile's 128 K elements, m_pad rows, hi and lo) that share a
+// ring stage: all of a tile's where they fit.  A stage's cycle is bound by its copy's round trip,
+// however few bytes that brings, and a tile takes only one stage per KC input dimensions besides:
+// with a chunk to a stage the chain took two of the four stages of a tile at d = 128 and two of three at d = 33 (there 50
+// iterations and their set-up 18.2 -> 17.9 ms; nothing lost elsewhere).
+int chain_chunks(int kc, int zt, int cg, int64_t mpad) {
+  const int64_t stage = zt == 3 ? (128 + 256) * kc * 4 : cg == 2 ? (128 + 64) * kc * 4 : 256 * kc * 4;
+  const int64_t chunk = mpad / cg * kc * 4;
+  int n = 128 / kc;
+  while (n > 1 && n * chunk > stage) n /= 2;
+  return n;
+}
+
 cudaError_t common_args(const TcView& v, TcArgs& a) {
   memset(&a, 0, sizeof(a));
   a.nk = (int)(v.dld / view_kc(v));
   a.mpad = (int)v.mpad;
+  a.mchunks = chain_chunks(view_kc(v), view_zt(v), view_cg(v), v.mpad);
   a.R = v.R;
   a.C = v.C;
   a.nsplit = v.nsplit;
