@@ -1,0 +1,89 @@
+"""Edges of the FP32 tiles, the set-up's batches and the splits of work over CTAs.
+
+Where work is split (feature parts over a cluster's CTAs, K chunks of a factor product, the
+factorisation beside the forward sweep, row blocks of the outer form) the sums keep their order or
+their float-float accuracy: results are the same bits where the order is the same, and within the
+FP32 path's tolerance of the float64 oracle everywhere.
+"""
+import numpy as np
+import pytest
+
+from oracle import admm, rff as orff
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rff():
+    import paper_1409_0940_gb300 as m
+    return m
+
+
+def data(n, d, m, seed=3):
+    rng = np.random.default_rng(seed)
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    Y = np.sign(rng.standard_normal((n, m))).astype(np.float32)
+    return X, Y
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+# 1, 3, 6 and 20 feature tiles (none, clusters of 4 and 8); d below, at and past a K stage; one to
+# sixteen 16-column runs, the parked and the float-float sums, every number of M rows per stage
+@pytest.mark.parametrize("D,C,d,m", [(100, 1, 1, 1), (300, 2, 32, 20), (700, 1, 33, 70), (2500, 3, 66, 150),
+                                     (300, 1, 5, 256)])
+def test_fp32_scores_do_not_depend_on_the_batch(rff, D, C, d, m):
+    X, Y = data(300, d, m)
+    s = rff.Solver(loss="squared", reg="l2", lam=1e-3, sigma=4.0, rho=1.0, D=D, R=1, C=C, seed=9, m=m, prec="fp32")
+    s.set_data(X, Y)
+    s.solve(2)
+    W = s.weights()
+    Q = np.random.default_rng(5).standard_normal((155 * 128 + 45, d)).astype(np.float32)
+    full = s.predict(Q)
+    for q in (1, 127, 129, 1000, 152 * 128 + 1):
+        assert np.array_equal(s.predict(np.ascontiguousarray(Q[:q])), full[:q])
+    rows = np.r_[0:40, Q.shape[0] - 40:Q.shape[0]]
+    ref = orff.features_block(Q[rows], 9, 4.0, D, 0, D) @ W.astype(np.float64)
+    # FP32 sums of D products of magnitude |z| |w|: the path's 1e-5
+    assert rel(full[rows], ref) <= 1e-5
+    s.close()
+
+
+# passes, factor products and Gram matrices on ragged blocks: a Gram form with one short tile and
+# K = 87 (the tail of a 32-K chunk), one with m = 150 (parked factor sums), one whose factor
+# products go to clusters, and outer forms (fewer rows than features) of 5 and 7 uneven row blocks
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("split_bf16", 1e-4)])
+@pytest.mark.parametrize("n,d,m,D,R,C", [(1003, 17, 1, 87, 1, 1), (1003, 5, 150, 261, 2, 2), (700, 9, 3, 600, 1, 1),
+                                         (651, 40, 2, 1200, 5, 3), (903, 12, 20, 300, 7, 1)])
+def test_ragged_solves_match_the_oracle(rff, prec, tol, n, d, m, D, R, C):
+    X, Y = data(n, d, m, seed=n)
+    kw = dict(loss="squared", reg="l2", lam=1e-3, sigma=4.0, rho=1.0, D=D, R=R, C=C, seed=5)
+    ref = admm.admm(admm.Problem(X, Y, **kw), 8)["Wbar"]
+    s = rff.Solver(prec=prec, m=m, **kw)
+    s.set_data(X, Y)
+    s.solve(8, stats=False)
+    assert rel(s.weights(), ref) <= tol
+    s.close()
+
+
+# With a memory limit the forward sweep runs after the factorisation instead of beside it, the outer
+# form takes fewer row blocks at once, and TensorSketch features are formed in row chunks
+@pytest.mark.parametrize("kw,d,n", [
+    (dict(D=900, R=2, C=3, prec="split_bf16"), 10, 2000),
+    (dict(D=900, R=2, C=1, prec="fp32"), 10, 2000),
+    (dict(D=2000, R=6, C=2, prec="fp32"), 10, 1500),
+    (dict(D=600, R=1, C=2, prec="cached_z", feature_map="tensorsketch", degree=3, coef0=1.0), 20, 1500)])
+def test_a_memory_limit_changes_no_result(rff, kw, d, n):
+    X, Y = data(n, d, 4)
+    got = []
+    for limit in (0, 4 << 30):
+        s = rff.Solver(loss="hinge", reg="l2", lam=1e-4, sigma=4.0, rho=1.0, seed=5, m=4, **kw)
+        if limit:
+            rff.rff_admm_set_memory_limit(s.h, limit)
+        s.set_data(X, Y)
+        s.solve(4, stats=False)
+        got.append(s.weights())
+        s.close()
+    assert np.array_equal(got[0], got[1])
