@@ -124,7 +124,7 @@ __device__ __forceinline__ float warp_max(float x) {
 }
 
 // Multinomial logistic prox of one row, one warp, lanes over the m outputs (up
-// to 8 per lane), c = argmax_k y_k (first maximum).  The optimality condition
+// to PL <= 8 per lane), c = argmax_k y_k (first maximum).  The optimality condition
 // o = v - t (softmax(o) - e_c) is solved through s = log sum_k exp(o_k): with
 // w = v + t e_c, each p_k = exp(o_k - s) satisfies log p_k + t p_k = w_k - s,
 // a scalar equation solved by Newton from a Lambert-W estimate, and s is the
@@ -149,12 +149,13 @@ __device__ __forceinline__ float solve_logp(float a, float t, float logt) {
 }
 
 // class index of a row, the first maximum of y over the m outputs (a warp, lanes over outputs)
-__device__ __forceinline__ int row_class(const float (&y)[MAXPL], int m) {
+template <int PL>
+__device__ __forceinline__ int row_class(const float (&y)[PL], int m) {
   const int lane = threadIdx.x & 31;
   float best = -INFINITY;
   int bidx = 1 << 30;
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     const int k = lane + 32 * q;
     if (k < m && (y[q] > best)) { best = y[q]; bidx = k; }
   }
@@ -167,19 +168,20 @@ __device__ __forceinline__ int row_class(const float (&y)[MAXPL], int m) {
   return bidx;
 }
 
-__device__ void prox_multinomial_row(const float (&v)[MAXPL], const float (&y)[MAXPL], int m, float t, int iters,
-                                     float (&o)[MAXPL]) {
+template <int PL>
+__device__ void prox_multinomial_row(const float (&v)[PL], const float (&y)[PL], int m, float t, int iters,
+                                     float (&o)[PL]) {
   const int lane = threadIdx.x & 31;
   if (!(t > 1e-30f)) {
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) o[q] = v[q];
+    for (int q = 0; q < PL; ++q) o[q] = v[q];
     return;
   }
   const int bidx = row_class(y, m);
-  float w[MAXPL];
+  float w[PL];
   float wmax = -INFINITY;
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     const int k = lane + 32 * q;
     w[q] = v[q] + (k == bidx ? t : 0.f);
     if (k < m) wmax = fmaxf(wmax, w[q]);
@@ -187,9 +189,9 @@ __device__ void prox_multinomial_row(const float (&v)[MAXPL], const float (&y)[M
   wmax = warp_max(wmax);
   const float logt = logf(t);
   float s = wmax - t;
-  float lq[MAXPL], pv[MAXPL];   // log p_k and p_k at the current s
+  float lq[PL], pv[PL];   // log p_k and p_k at the current s
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     lq[q] = 0.f;
     pv[q] = 0.f;
     if (lane + 32 * q < m) {
@@ -199,9 +201,9 @@ __device__ void prox_multinomial_row(const float (&v)[MAXPL], const float (&y)[M
   }
   for (int it = 0; it < iters; ++it) {
     float F = 0.f, dF = 0.f;
-    float rinv[MAXPL];
+    float rinv[PL];
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) {
+    for (int q = 0; q < PL; ++q) {
       rinv[q] = 1.f / (1.f + t * pv[q]);
       if (lane + 32 * q < m) {
         F += pv[q];
@@ -213,7 +215,7 @@ __device__ void prox_multinomial_row(const float (&v)[MAXPL], const float (&y)[M
     const float ds = F / dF;
     s += ds;
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) {
+    for (int q = 0; q < PL; ++q) {
       if (lane + 32 * q < m) {
         const float a = w[q] - s;
         float x = lq[q] - ds * rinv[q];
@@ -228,7 +230,7 @@ __device__ void prox_multinomial_row(const float (&v)[MAXPL], const float (&y)[M
     }
   }
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     const int k = lane + 32 * q;
     o[q] = (k < m) ? w[q] - t * pv[q] : 0.f;
   }
@@ -245,20 +247,21 @@ __device__ void prox_multinomial_row(const float (&v)[MAXPL], const float (&y)[M
 // w_k - max_k w_k: the entries of the final set lie within t of the maximum (tau >= max w - t),
 // so tau is formed from values of the size of t rather than of |w|.  The warp sums are
 // butterflies, so every lane holds the same tau and takes the same exit.
-__device__ void prox_crammer_singer_row(const float (&v)[MAXPL], const float (&y)[MAXPL], int m, float t,
-                                        float (&o)[MAXPL]) {
+template <int PL>
+__device__ void prox_crammer_singer_row(const float (&v)[PL], const float (&y)[PL], int m, float t,
+                                        float (&o)[PL]) {
   const int lane = threadIdx.x & 31;
   if (!(t > 0.f)) {
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) o[q] = v[q];
+    for (int q = 0; q < PL; ++q) o[q] = v[q];
     return;
   }
   const int c = row_class(y, m);
-  float w[MAXPL];
-  bool in[MAXPL];
+  float w[PL];
+  bool in[PL];
   float wmax = -INFINITY;
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     const int k = lane + 32 * q;
     in[q] = k < m;
     w[q] = v[q] + (k == c ? t : 1.f);
@@ -267,7 +270,7 @@ __device__ void prox_crammer_singer_row(const float (&v)[MAXPL], const float (&y
   wmax = warp_max(wmax);
   float sum = 0.f;
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     w[q] -= wmax;   // shifted: tau below is relative to the maximum
     if (in[q]) sum += w[q];
   }
@@ -277,25 +280,26 @@ __device__ void prox_crammer_singer_row(const float (&v)[MAXPL], const float (&y
     float s2 = 0.f;
     int c2 = 0;
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q)
+    for (int q = 0; q < PL; ++q)
       if (in[q] && w[q] > tau) { s2 += w[q]; ++c2; }
     s2 = warp_sum(s2);
     c2 = __reduce_add_sync(0xffffffffu, c2);
     if (c2 == cnt || c2 == 0) break;
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) in[q] = in[q] && w[q] > tau;
+    for (int q = 0; q < PL; ++q) in[q] = in[q] && w[q] > tau;
     cnt = c2;
     tau = (s2 - t) / (float)cnt;
   }
 #pragma unroll
-  for (int q = 0; q < MAXPL; ++q) {
+  for (int q = 0; q < PL; ++q) {
     const int k = lane + 32 * q;
     o[q] = (k < m) ? (fminf(w[q], tau) + wmax) - (k == c ? 0.f : 1.f) : 0.f;
   }
 }
 
-__device__ __forceinline__ void prox_row(int loss, const float (&v)[MAXPL], const float (&y)[MAXPL], int m, float t,
-                                         int iters, float (&o)[MAXPL]) {
+template <int PL>
+__device__ __forceinline__ void prox_row(int loss, const float (&v)[PL], const float (&y)[PL], int m, float t,
+                                         int iters, float (&o)[PL]) {
   if (loss == LOSS_MULTINOMIAL) prox_multinomial_row(v, y, m, t, iters, o);
   else prox_crammer_singer_row(v, y, m, t, o);
 }
@@ -354,8 +358,9 @@ __global__ void k_prox_reg(int reg, const float* __restrict__ V, const float* __
 // and columns are written as zeros.
 constexpr int EX_ROWS = 32;
 
-template <int LOSS>
-__global__ void __launch_bounds__(256, row_loss(LOSS) ? 3 : 4) k_exchange(RowEpiArgs a) {
+// PL: outputs per lane of the row losses (m_pad <= 32 PL; 1 for the elementwise ones)
+template <int LOSS, int PL>
+__global__ void __launch_bounds__(256, row_loss(LOSS) && PL > 5 ? 3 : 4) k_exchange(RowEpiArgs a) {
   extern __shared__ float ex_smem[];
   const int mp = a.mpad;
   float* tile = ex_smem;   // U of the 32 rows, [32][mpad + 1] (zero where not live)
@@ -448,10 +453,10 @@ __global__ void __launch_bounds__(256, row_loss(LOSS) ? 3 : 4) k_exchange(RowEpi
     const int64_t p = p0 + r;
     const bool ok = a.row_ok[p] >= 0;
     const int64_t base = p * mp;
-    float w_in[MAXPL], y[MAXPL], Ov[MAXPL], nuv[MAXPL], Sv[MAXPL];
+    float w_in[PL], y[PL], Ov[PL], nuv[PL], Sv[PL];
     // all of the row's loads first (independent, so they are in flight together)
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) {
+    for (int q = 0; q < PL; ++q) {
       const int k = lane + 32 * q;
       const bool in = k < mp;
       Ov[q] = in ? a.O[base + k] : 0.f;
@@ -462,13 +467,13 @@ __global__ void __launch_bounds__(256, row_loss(LOSS) ? 3 : 4) k_exchange(RowEpi
     for (int j = 0; j < a.C; ++j) {
       const float* opj = a.Op + j * jstride + base;
 #pragma unroll
-      for (int q = 0; q < MAXPL; ++q) {
+      for (int q = 0; q < PL; ++q) {
         const int k = lane + 32 * q;
         if (k < mp) Sv[q] += opj[k];
       }
     }
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) {
+    for (int q = 0; q < PL; ++q) {
       const int k = lane + 32 * q;
       w_in[q] = 0.f;
       if (k >= mp) continue;
@@ -486,15 +491,15 @@ __global__ void __launch_bounds__(256, row_loss(LOSS) ? 3 : 4) k_exchange(RowEpi
       if (live) w_in[q] = Obar - nu;
       else y[q] = 0.f;
     }
-    float o[MAXPL];
+    float o[PL];
     if (row_loss(LOSS)) {
       prox_row(LOSS, w_in, y, a.m, a.t_loss, a.newton, o);
     } else {
 #pragma unroll
-      for (int q = 0; q < MAXPL; ++q) o[q] = prox_scalar(LOSS, w_in[q], y[q], a.t_loss, a.newton);
+      for (int q = 0; q < PL; ++q) o[q] = prox_scalar(LOSS, w_in[q], y[q], a.t_loss, a.newton);
     }
 #pragma unroll
-    for (int q = 0; q < MAXPL; ++q) {
+    for (int q = 0; q < PL; ++q) {
       const int k = lane + 32 * q;
       const bool live = ok && k < a.m;
       if (k < mp) a.O[base + k] = live ? o[q] : 0.f;
@@ -786,11 +791,13 @@ __global__ void __launch_bounds__(256) k_reg_sum(int reg, const float* __restric
 
 // flag |= 1 for a NaN/Inf entry; with pm1, flag |= 2 for an entry outside {-1, +1}
 // flag |= 1 for NaN/Inf, 2 for a value other than +-1 (pm1); maxbits = max |x| of the
-// finite values as float bits (unsigned order equals float order for x >= 0)
-__global__ void k_finite(const float* __restrict__ x, int64_t n, int pm1, int* __restrict__ flag,
+// finite values as float bits (unsigned order equals float order for x >= 0).  One atomic per
+// block: a warp's each, 32 thousand on one word, took 15 of the 17 us of a 10 MB array
+__global__ void __launch_bounds__(256) k_finite(const float* __restrict__ x, int64_t n, int pm1, int* __restrict__ flag,
                          unsigned* __restrict__ maxbits) {
   int f = 0;
   float mx = 0.f;
+#pragma unroll 4
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const float v = x[e];
     if (!isfinite(v)) f |= 1;
@@ -800,9 +807,16 @@ __global__ void k_finite(const float* __restrict__ x, int64_t n, int pm1, int* _
   }
   if (f) atomicOr(flag, f);
   if (maxbits) {
+    __shared__ float wmx[8];
+    mx = warp_max(mx);
+    if ((threadIdx.x & 31) == 0) wmx[threadIdx.x / 32] = mx;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+      mx = wmx[threadIdx.x];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0 && mx > 0.f) atomicMax(maxbits, __float_as_uint(mx));
+      for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffu, mx, o));
+      if (threadIdx.x == 0 && mx > 0.f) atomicMax(maxbits, __float_as_uint(mx));
+    }
   }
 }
 
@@ -867,40 +881,38 @@ cudaError_t launch_prox_reg(int reg, const float* V, const float* mu, int64_t n,
   return cudaGetLastError();
 }
 
+namespace {
+// the row losses by outputs per lane: at m = 147 five instead of eight (multinomial, 40,000 rows: 409 -> 340 us)
+template <int LOSS>
+cudaError_t launch_exchange(const RowEpiArgs& a, unsigned grid, size_t smem, cudaStream_t st) {
+  const int pl = row_loss(LOSS) ? (int)ceil_div(a.mpad, 32) : 1;
+  if (pl <= 1) k_exchange<LOSS, 1><<<grid, 256, smem, st>>>(a);
+  else if constexpr (row_loss(LOSS)) {
+    if (pl == 2) k_exchange<LOSS, 2><<<grid, 256, smem, st>>>(a);
+    else if (pl <= 3) k_exchange<LOSS, 3><<<grid, 256, smem, st>>>(a);
+    else if (pl <= 5) k_exchange<LOSS, 5><<<grid, 256, smem, st>>>(a);
+    else k_exchange<LOSS, MAXPL><<<grid, 256, smem, st>>>(a);
+  }
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_row_epilogue(const RowEpiArgs& a, cudaStream_t st) {
   if (a.nslots <= 0) return cudaSuccess;
   if (a.mpad > 32 * MAXPL || a.nslots % EX_ROWS) return cudaErrorInvalidValue;
   const bool split = a.VThi && a.VTlo && a.amax;
   if (!a.V32 && !split) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)EX_ROWS * (a.mpad + 1) * sizeof(float);
+  const size_t smem = (size_t)EX_ROWS * (a.mpad + 1) * sizeof(float);   // at most 33 KB
   const unsigned grid = (unsigned)(a.nslots / EX_ROWS);
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    const int mx = EX_ROWS * (32 * MAXPL + 1) * (int)sizeof(float);
-    attr = cudaFuncSetAttribute(k_exchange<LOSS_SQUARED>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_exchange<LOSS_HINGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_exchange<LOSS_LOGISTIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_exchange<LOSS_MULTINOMIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_exchange<LOSS_L1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_exchange<LOSS_CRAMMER_SINGER>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  });
-  if (attr != cudaSuccess) return attr;
   switch (a.loss) {
-    case LOSS_SQUARED: k_exchange<LOSS_SQUARED><<<grid, 256, smem, st>>>(a); break;
-    case LOSS_HINGE: k_exchange<LOSS_HINGE><<<grid, 256, smem, st>>>(a); break;
-    case LOSS_LOGISTIC: k_exchange<LOSS_LOGISTIC><<<grid, 256, smem, st>>>(a); break;
-    case LOSS_MULTINOMIAL: k_exchange<LOSS_MULTINOMIAL><<<grid, 256, smem, st>>>(a); break;
-    case LOSS_L1: k_exchange<LOSS_L1><<<grid, 256, smem, st>>>(a); break;
-    case LOSS_CRAMMER_SINGER: k_exchange<LOSS_CRAMMER_SINGER><<<grid, 256, smem, st>>>(a); break;
+    case LOSS_SQUARED: return launch_exchange<LOSS_SQUARED>(a, grid, smem, st);
+    case LOSS_HINGE: return launch_exchange<LOSS_HINGE>(a, grid, smem, st);
+    case LOSS_LOGISTIC: return launch_exchange<LOSS_LOGISTIC>(a, grid, smem, st);
+    case LOSS_MULTINOMIAL: return launch_exchange<LOSS_MULTINOMIAL>(a, grid, smem, st);
+    case LOSS_L1: return launch_exchange<LOSS_L1>(a, grid, smem, st);
+    case LOSS_CRAMMER_SINGER: return launch_exchange<LOSS_CRAMMER_SINGER>(a, grid, smem, st);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_rhs(const float* Wbar, const float* muij, const float* Rpart, int nsplit, int R, int64_t nfe,
@@ -979,7 +991,7 @@ cudaError_t launch_reg_partials(int reg, const float* W, int64_t n, double* part
 
 cudaError_t launch_finite_check(const float* x, int64_t n, int pm1, int* flag, cudaStream_t st, unsigned* maxbits) {
   if (n <= 0) return cudaSuccess;
-  k_finite<<<(unsigned)std::min<int64_t>(ceil_div(n, 256), 4096), 256, 0, st>>>(x, n, pm1, flag, maxbits);
+  k_finite<<<(unsigned)std::min<int64_t>(ceil_div(n, 1024), 1216), 256, 0, st>>>(x, n, pm1, flag, maxbits);
   return cudaGetLastError();
 }
 
