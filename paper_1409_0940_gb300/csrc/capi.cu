@@ -1511,14 +1511,10 @@ rff_status exchange_and_average(rff_admm_t h, int k) {
     e.VThi = s.VThi;
     e.VTlo = s.VTlo;
     e.amax = s.amax;
-    CK(cudaMemsetAsync(s.amax + AMAX_V, 0, 4, s.st));
-    CK(cudaMemsetAsync(s.amax + AMAX_O_NEXT, 0, 8, s.st));
   }
   CK(launch_row_epilogue(e, s.st));
-  if (vsplit)   // the outputs' maxima become the next exchange's inputs
-    CK(cudaMemcpyAsync(s.amax + AMAX_O, s.amax + AMAX_O_NEXT, 8, cudaMemcpyDeviceToDevice, s.st));
   if ((r = mark(h, k, 5)) != RFF_OK) return r;
-  CK(launch_avg_dual(s.W, s.What, s.R, nfe, s.Wbar, s.mu, s.muij, s.st));
+  CK(launch_avg_dual(s.W, s.What, s.R, nfe, s.Wbar, s.mu, s.muij, s.st, vsplit ? s.amax : nullptr));
   return mark(h, k, 6);
 }
 
@@ -1659,7 +1655,10 @@ rff_status phase_project(rff_admm_t h, int k) {
     // the transposed FP16 split of W' that pass 2 reads
     CK(launch_rhs_split3T(s.Wbar, s.muij, s.Rpart, s.cached_z() ? s.nsplit_cz : s.nsplit, s.R, s.fslots,
                           (int)s.mpad, s.feat_of_slot, s.rT1, s.rT2, s.rT3, s.st, s.What));
-    CK(cudaMemsetAsync(s.amax + AMAX_W, 0, 4, s.st));
+    // the maxima that the rest of the iteration forms: V (pass 1 has read the last one), W and O'
+    // (the words between them hold nothing beyond a call's kernels)
+    static_assert(AMAX_V == 0 && AMAX_W < AMAX_OP && AMAX_OP < AMAX_O, "one run of words up to O'");
+    CK(cudaMemsetAsync(s.amax, 0, (AMAX_OP + 1) * 4, s.st));
     CK(split_gemm(qgemm_view(s)));
     CK(launch_transpose_split_f16(s.What, s.fslots, (int)s.mpad, s.R, s.fslots * s.mpad, s.WThi, s.WTlo, s.fslots,
                                   s.mpad * s.fslots, 1.f, s.amax + AMAX_W, s.st));
@@ -1668,7 +1667,6 @@ rff_status phase_project(rff_admm_t h, int k) {
     CK(launch_gemm_f32_nn(s.gdesc, (int)nblocks, (int)smax, (int)smax, (int)s.mpad, 1.f, 1.f, s.st, s.act()));
   }
   if ((r = mark(h, k, 3)) != RFF_OK) return r;
-  if (s.split_path()) CK(cudaMemsetAsync(s.amax + AMAX_OP, 0, 4, s.st));   // max |O'| for the exchange
   return RFF_OK;
 }
 
@@ -2505,6 +2503,8 @@ rff_status rff_admm_set_state(rff_admm_t h, const void* buf, size_t bytes) {
     CK(cudaMemcpyAsync(pc.ptr, in + off, pc.bytes, cudaMemcpyHostToDevice, s.st));
     off += pc.bytes;
   }
+  // (states written before the averaging cleared these words still hold the maxima in them)
+  CK(cudaMemsetAsync(s.amax + AMAX_O_NEXT, 0, 8, s.st));
   CK(cudaStreamSynchronize(s.st));
   s.iters_done = hd.iters_done;
   return RFF_OK;

@@ -641,8 +641,14 @@ __device__ __forceinline__ float ff_round_sum(float y, float x, FF m) {
 // iterations, and an FP32 average would hand them its rounding every time (an error that
 // grows with the iteration count).
 __global__ void k_avg_dual(const float* __restrict__ W, const float* __restrict__ What, int R, int64_t nfe,
-                           float* __restrict__ Wbar, float* __restrict__ mu, float* __restrict__ muij) {
+                           float* __restrict__ Wbar, float* __restrict__ mu, float* __restrict__ muij,
+                           unsigned* __restrict__ amax) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (amax && e == 0) {   // the exchange's maxima become the next one's inputs
+    amax[AMAX_O] = amax[AMAX_O_NEXT];
+    amax[AMAX_NU] = amax[AMAX_NU_NEXT];
+    amax[AMAX_O_NEXT] = amax[AMAX_NU_NEXT] = 0u;
+  }
   if (e >= nfe) return;
   const float w = W[e];
   FF s{w, 0.f};
@@ -947,8 +953,8 @@ cudaError_t launch_outer_update(float* Op, const float* U, const float* y, int64
 }
 
 cudaError_t launch_avg_dual(const float* W, const float* What, int R, int64_t nfe, float* Wbar, float* mu,
-                            float* muij, cudaStream_t st) {
-  k_avg_dual<<<nblk(nfe), 256, 0, st>>>(W, What, R, nfe, Wbar, mu, muij);
+                            float* muij, cudaStream_t st, unsigned* amax) {
+  k_avg_dual<<<nblk(nfe), 256, 0, st>>>(W, What, R, nfe, Wbar, mu, muij, amax);
   return cudaGetLastError();
 }
 

@@ -265,8 +265,9 @@ cudaError_t launch_outer_residual(float* u, const float* Op, const float* U, int
 //   O'_ij += U_i + y_ij for the active blocks (bmask per row block i, column block j; null: all)
 cudaError_t launch_outer_update(float* Op, const float* U, const float* y, int64_t nslots, int mpad, int R, int C,
                                 const int64_t* d_row_slot, const uint8_t* bmask, cudaStream_t st);
+// amax (or null): the words AMAX_O, AMAX_NU take over AMAX_O_NEXT, AMAX_NU_NEXT, which become 0
 cudaError_t launch_avg_dual(const float* W, const float* What, int R, int64_t nfe, float* Wbar, float* mu,
-                            float* muij, cudaStream_t st);
+                            float* muij, cudaStream_t st, unsigned* amax = nullptr);
 // hi/lo FP16 split of src^T scaled by f16_scale(*amax) (amax non-null) or by scale
 cudaError_t launch_transpose_split_f16(const float* src, int64_t rows, int cols, int nbatch, int64_t src_batch_stride,
                                        __half* hi, __half* lo, int64_t dst_ld, int64_t dst_batch_stride, float scale,
