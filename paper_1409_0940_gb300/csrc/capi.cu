@@ -2378,18 +2378,20 @@ rff_status rff_admm_predict(rff_admm_t h, const float* Xq, int64_t q, float* sco
     CK(cudaMemsetAsync(s.flag, 0, 16, s.st));
     CK(launch_finite_check(stage, nq * s.d, s.p.feature_map == RFF_MAP_LAPLACE ? 2 : 0, s.flag, s.st,
                            reinterpret_cast<unsigned*>(s.flag + 2)));
-    int fl[3] = {0, 0, 0};
-    CK(cudaMemcpyAsync(fl, s.flag, 12, cudaMemcpyDeviceToHost, s.st));
-    CK(cudaStreamSynchronize(s.st));
-    if (fl[0] & 1) return h->fail(RFF_EINVAL, "queries contain NaN or Inf");
-    if (fl[0] & 4) return h->fail(RFF_EINVAL, "the random Laplace map takes nonnegative queries");
-    if ((r = check_query_range(h, fl[2])) != RFF_OK) return r;
     // rows q0..q0+nq into a slot-padded block (rows beyond nq are zero and discarded)
     CK(cudaMemsetAsync(xq32, 0, nqp * s.dld * 4, s.st));
     CK(launch_gather_rows(stage, s.d, s.d, nullptr, nq, xq32, s.dld, s.st));
     if (s.bias_col >= 0) CK(launch_set_column(xq32, s.dld, nqp, s.bias_col, 1.f, s.st));
     if (s.tc_scores()) CK(launch_split_f16(xq32, nqp * s.dld, s.xscale, xh, xl, s.st));
     if ((r = scores_pass(h, xq32, xh, xl, nqp, nullptr, sc, part, partb)) != RFF_OK) return r;
+    // The check's outcome is read with the scores formed, not before: waiting for it in front of a
+    // dozen launches left the GPU idle while they were made.  Refused queries leave `scores` alone.
+    int fl[3] = {0, 0, 0};
+    CK(cudaMemcpyAsync(fl, s.flag, 12, cudaMemcpyDeviceToHost, s.st));
+    CK(cudaStreamSynchronize(s.st));
+    if (fl[0] & 1) return h->fail(RFF_EINVAL, "queries contain NaN or Inf");
+    if (fl[0] & 4) return h->fail(RFF_EINVAL, "the random Laplace map takes nonnegative queries");
+    if ((r = check_query_range(h, fl[2])) != RFF_OK) return r;
     CK(cudaMemcpy2DAsync(scores + q0 * s.m, s.m * 4, sc, s.mpad * 4, s.m * 4, nq, kout, s.st));
   }
   CK(cudaStreamSynchronize(s.st));
