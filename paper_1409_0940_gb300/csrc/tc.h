@@ -54,7 +54,7 @@ cudaError_t tc_pass2(const TcView& v, const __half* Mhi, const __half* Mlo, int6
 // take (outs = Rpart or O'; Mhi, Mlo, m_amax, out_amax for pass 2 only, else null).  The solves'
 // arguments go to device memory that the object owns (a synchronous copy: create it outside
 // stream capture); every launch then reads them, so the object must outlive the launches.
-// Every solve runs the default geometry (K chunk 64, Z tile in TMEM, one CTA per MMA).
+// Every solve runs one geometry (K chunk 64, Z tile in TMEM, one CTA per MMA).
 struct TcMulti;
 cudaError_t tc_multi_create(const TcView* views, int n, int which, float* const* outs, const __half* const* Mhi,
                             const __half* const* Mlo, const unsigned* const* m_amax, unsigned* const* out_amax,
