@@ -58,6 +58,7 @@ struct QArgs {
   unsigned* amax;
   const uint8_t* bmask;      // active blocks of a stochastic iteration, or null
   int accumulate;            // 1: out += result (amax of the sum)
+  int cl;                    // CTAs (a cluster) that share a job's K stages
   int* err;
   long long timeout_cycles;
 };
@@ -83,6 +84,15 @@ __device__ __forceinline__ bool qwait(uint32_t bar, uint32_t parity, QShared& sh
   }
 }
 
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+
 // split-product order (A term, B term): exponents summing to at most 2^-16
 __host__ __device__ constexpr int prod_a(int p) { return p == 2 || p == 4 ? 1 : p == 5 ? 2 : 0; }
 __host__ __device__ constexpr int prod_b(int p) { return p == 1 || p == 4 ? 1 : p == 3 ? 2 : 0; }
@@ -99,6 +109,9 @@ __device__ __forceinline__ bool q_skip(const SgJob& j, const QArgs& a) {
 // swizzle: fewer shared-memory wavefronts per product, half as many stages); a job's nk counts
 // chunks of 32, so with KC = 64 an odd count reads 32 more K columns, which the caller keeps
 // zero in A (or beyond the tensor, where the copy fills zeros).
+//
+// cl > 1: a cluster of cl CTAs takes one job, each a run of its K stages; the partial results meet
+// in distributed shared memory and are added in rank order, each CTA finishing 128 / cl rows.
 template <int NA, int NB, int F16, int KC>
 __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArgs a) {
   constexpr int NPROD = (NA == 3 && NB == 3) ? 6 : 3;
@@ -112,6 +125,14 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
   const uint32_t bar_accf = smem_u32(&sh.acc_full[0]), bar_acce = smem_u32(&sh.acc_empty[0]);
   const uint32_t bar_done = smem_u32(&sh.mma_done);
   const uint32_t mb = (uint32_t)a.mpad * (KC * 2);   // one B term: m_pad rows
+  const int rank = a.cl > 1 ? (int)cluster_rank() : 0;
+  const int job0 = blockIdx.x / a.cl, job_step = gridDim.x / a.cl;
+  // this CTA's stages of KC elements of a job of nk chunks
+  auto stages_of = [&](int nk, int& s0, int& s1) {
+    const int n = (nk * QKC + KC - 1) / KC;
+    s0 = rank * n / a.cl;
+    s1 = (rank + 1) * n / a.cl;
+  };
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
     for (int i = 0; i < a.ns; ++i) {
@@ -140,11 +161,12 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
     if (lane == 0) {
       uint32_t issued = 0;   // ring stages filled, over all of this CTA's jobs
       bool ok = true;
-      for (int jx = blockIdx.x; ok && jx < a.njobs; jx += gridDim.x) {
+      for (int jx = job0; ok && jx < a.njobs; jx += job_step) {
         const SgJob job = a.jobs[jx];
         if (q_skip(job, a)) continue;
-        const int nkc = (job.nk * QKC + KC - 1) / KC;   // stages of KC elements
-        for (int kc = 0; kc < nkc; ++kc) {
+        int s0, s1;
+        stages_of(job.nk, s0, s1);
+        for (int kc = s0; kc < s1; ++kc) {
           const int st = issued % a.ns;
           const uint32_t use = issued / a.ns;
           if (use > 0 && !qwait(bar_empty + 8 * st, (use - 1) & 1, sh, a)) {
@@ -175,7 +197,7 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
       const uint32_t idesc = F16 ? idesc_f16(128, a.mpad) : idesc_bf16(128, a.mpad);
       bool ok = true;
       uint32_t used = 0, done_jobs = 0;   // ring stages consumed, jobs multiplied
-      for (int jx = blockIdx.x; ok && jx < a.njobs; jx += gridDim.x) {
+      for (int jx = job0; ok && jx < a.njobs; jx += job_step) {
         const SgJob job = a.jobs[jx];
         if (q_skip(job, a)) continue;
         const uint32_t buf = done_jobs % a.nbuf, round = done_jobs / a.nbuf;
@@ -185,8 +207,9 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
         }
         fence_after();
         const uint32_t acc = tmem + buf * a.buf_cols;
-        const int nkc = (job.nk * QKC + KC - 1) / KC;   // stages of KC elements
-        for (int kc = 0; kc < nkc; ++kc, ++used) {
+        int s0, s1;
+        stages_of(job.nk, s0, s1);
+        for (int kc = s0; kc < s1; ++kc, ++used) {
           const int st = used % a.ns;
           if (!qwait(bar_full + 8 * st, (used / a.ns) & 1, sh, a)) {
             ok = false;
@@ -204,9 +227,9 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
               if (a.acc_b) {
                 // hi.hi alone in the first accumulator, the smaller products in the second
                 const uint32_t d = p == 0 ? acc : acc + a.acc_b;
-                mma_bf16(d, da, db, idesc, (kc > 0 || kk > 0 || p > 1) ? 1u : 0u);
+                mma_bf16(d, da, db, idesc, (kc > s0 || kk > 0 || p > 1) ? 1u : 0u);
               } else {
-                mma_bf16(acc, da, db, idesc, (kc > 0 || kk > 0 || p > 0) ? 1u : 0u);
+                mma_bf16(acc, da, db, idesc, (kc > s0 || kk > 0 || p > 0) ? 1u : 0u);
               }
             }
           }
@@ -227,7 +250,7 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
     const int row = quarter * 32 + lane;
     uint32_t done_jobs = 0;
     float mx = 0.f;
-    for (int jx = blockIdx.x; jx < a.njobs; jx += gridDim.x) {
+    for (int jx = job0; jx < a.njobs; jx += job_step) {
       const SgJob job = a.jobs[jx];
       if (q_skip(job, a)) continue;
       const uint32_t buf = done_jobs % a.nbuf, round = done_jobs / a.nbuf;
@@ -247,6 +270,15 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
         float x[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) x[t] = sc * (__uint_as_float(r8[t]) + __uint_as_float(s8[t]));
+        if (a.cl > 1) {   // the ring is free: this job is the CTA's only one
+          int s0, s1;
+          stages_of(job.nk, s0, s1);
+          float4* dst = reinterpret_cast<float4*>(base + ((size_t)row * a.mpad + c) * 4);
+          const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);   // (no stage: nothing was accumulated)
+          dst[0] = s1 > s0 ? make_float4(x[0], x[1], x[2], x[3]) : z;
+          dst[1] = s1 > s0 ? make_float4(x[4], x[5], x[6], x[7]) : z;
+          continue;
+        }
         float4* dst = reinterpret_cast<float4*>(orow_p + c);
         const bool in = RFF_SPAN(job.out + (int64_t)row * a.mpad + c, 8, a.out_elems);
         if (a.accumulate && in) {
@@ -266,11 +298,44 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
       if (lane == 0) mbar_arrive(bar_acce + 8 * buf);   // the set is free for the job after next
       ++done_jobs;
     }
-    if (a.amax) {
+    if (a.amax && a.cl == 1) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       if (lane == 0 && mx > 0.f) atomicMax(a.amax, __float_as_uint(mx));
     }
+  }
+  if (a.cl > 1) {
+    __syncwarp();   // (the roles' single threads rejoin their warps)
+    cluster_sync_all();
+    const SgJob job = a.jobs[job0];
+    if (!q_skip(job, a)) {
+      const int rows = 128 / a.cl, n4 = rows * a.mpad / 4;
+      const uint32_t src = smem_u32(base) + (uint32_t)(rank * rows * a.mpad * 4);
+      float mx = 0.f;
+      for (int e = threadIdx.x; e < n4; e += QNT) {
+        float4 x = ld_cluster4(mapa_rank(src + 16 * e, 0));
+        for (int r = 1; r < a.cl; ++r) {
+          const float4 v = ld_cluster4(mapa_rank(src + 16 * e, r));
+          x = make_float4(x.x + v.x, x.y + v.y, x.z + v.z, x.w + v.w);
+        }
+        const int64_t o = job.out + (int64_t)rank * rows * a.mpad + 4 * e;
+        if (!RFF_SPAN(o, 4, a.out_elems)) continue;
+        float4* dst = reinterpret_cast<float4*>(a.out + o);
+        if (a.accumulate) {
+          const float4 p0 = *dst;
+          x = make_float4(x.x + p0.x, x.y + p0.y, x.z + p0.z, x.w + p0.w);
+        }
+        *dst = x;
+        mx = fmaxf(mx, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+      }
+      __syncwarp();
+      if (a.amax) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0 && mx > 0.f) atomicMax(a.amax, __float_as_uint(mx));
+      }
+    }
+    cluster_sync_all();   // nobody leaves while others read its shared memory
   }
   fence_before();
   __syncthreads();
@@ -466,14 +531,29 @@ cudaError_t split_gemm(const SgView& v) {
       a.tmem_cols *= 2;
     }
   }
-  if (v.na == 3) {
-    if (kc == 64) k_split_gemm<3, 3, 0, 64><<<(unsigned)grid, QNT, smem, v.st>>>(a);
-    else k_split_gemm<3, 3, 0, 32><<<(unsigned)grid, QNT, smem, v.st>>>(a);
-  } else {
-    if (kc == 64) k_split_gemm<2, 2, 1, 64><<<(unsigned)grid, QNT, smem, v.st>>>(a);
-    else k_split_gemm<2, 2, 1, 32><<<(unsigned)grid, QNT, smem, v.st>>>(a);
-  }
-  return cudaGetLastError();
+  // A table of few jobs (one per 128 rows of the cached inverses) leaves most SMs idle while each
+  // CTA walks its K stages at the pace of the copies: clusters share them, as many CTAs as fit
+  // side by side.  A sweep of four solves (16 to 64 jobs of K = 1024 or 2048, m = 8): 47 -> 24 us a
+  // product, 12.4 -> 11.5 ms over 10 iterations; 48 jobs of K = 1000: 50 iterations 17.7 -> 17.0 ms
+  a.cl = 1;
+  if (!v.persistent && v.na == 3 && v.mpad <= 64)
+    while (a.cl < 8 && 2 * a.cl * (int64_t)v.njobs <= qsm_count()) a.cl *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(grid * a.cl));
+  cfg.blockDim = dim3(QNT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = v.st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)a.cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (v.na == 3)
+    return kc == 64 ? cudaLaunchKernelEx(&cfg, k_split_gemm<3, 3, 0, 64>, a)
+                    : cudaLaunchKernelEx(&cfg, k_split_gemm<3, 3, 0, 32>, a);
+  return kc == 64 ? cudaLaunchKernelEx(&cfg, k_split_gemm<2, 2, 1, 64>, a)
+                  : cudaLaunchKernelEx(&cfg, k_split_gemm<2, 2, 1, 32>, a);
 }
 
 RFF_CHECK_UNIT(qgemm)
