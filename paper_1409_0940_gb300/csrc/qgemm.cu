@@ -519,41 +519,55 @@ cudaError_t split_gemm(const SgView& v) {
   // share an SM holds them
   a.buf_cols = a.tmem_cols;
   a.nbuf = 1;
-  int64_t grid = v.njobs;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern(), QNT, smem);
+  if (e != cudaSuccess) return e;
+  per_sm = std::min(std::max(per_sm, 1), std::max(1, 512 / (int)a.tmem_cols));
+  const int64_t slots = (int64_t)qsm_count() * per_sm;
+  auto run = [&](int64_t grid, int cl) -> cudaError_t {
+    a.cl = cl;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(grid * cl));
+    cfg.blockDim = dim3(QNT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = v.st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (v.na == 3)
+      return kc == 64 ? cudaLaunchKernelEx(&cfg, k_split_gemm<3, 3, 0, 64>, a)
+                      : cudaLaunchKernelEx(&cfg, k_split_gemm<3, 3, 0, 32>, a);
+    return kc == 64 ? cudaLaunchKernelEx(&cfg, k_split_gemm<2, 2, 1, 64>, a)
+                    : cudaLaunchKernelEx(&cfg, k_split_gemm<2, 2, 1, 32>, a);
+  };
   if (v.persistent) {
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern(), QNT, smem);
-    if (e != cudaSuccess) return e;
-    per_sm = std::max(per_sm, 1);
-    grid = std::min<int64_t>(v.njobs, (int64_t)qsm_count() * per_sm);
     if (2u * a.tmem_cols * (uint32_t)per_sm <= 512u) {
       a.nbuf = 2;
       a.tmem_cols *= 2;
     }
+    return run(std::min<int64_t>(v.njobs, slots), 1);
   }
-  // A table of few jobs (one per 128 rows of the cached inverses) leaves most SMs idle while each
-  // CTA walks its K stages at the pace of the copies: clusters share them, as many CTAs as fit
-  // side by side.  A sweep of four solves (16 to 64 jobs of K = 1024 or 2048, m = 8): 47 -> 24 us a
-  // product, 12.4 -> 11.5 ms over 10 iterations; 48 jobs of K = 1000: 50 iterations 17.7 -> 17.0 ms
-  a.cl = 1;
-  if (!v.persistent && v.na == 3 && v.mpad <= 64)
-    while (a.cl < 8 && 2 * a.cl * (int64_t)v.njobs <= qsm_count()) a.cl *= 2;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(grid * a.cl));
-  cfg.blockDim = dim3(QNT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = v.st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)a.cl;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (v.na == 3)
-    return kc == 64 ? cudaLaunchKernelEx(&cfg, k_split_gemm<3, 3, 0, 64>, a)
-                    : cudaLaunchKernelEx(&cfg, k_split_gemm<3, 3, 0, 32>, a);
-  return kc == 64 ? cudaLaunchKernelEx(&cfg, k_split_gemm<2, 2, 1, 64>, a)
-                  : cudaLaunchKernelEx(&cfg, k_split_gemm<2, 2, 1, 32>, a);
+  // The jobs past the last whole wave would leave most SMs idle while each CTA walks its K stages at
+  // the pace of the copies: clusters share those jobs' stages, as many CTAs as fit side by side
+  // (where a partial result fits the ring's memory).  A sweep of four solves (16 to 64 jobs of K =
+  // 1024 or 2048, m = 8): 47 -> 24 us a product, 12.4 -> 11.5 ms over 10 iterations; 48 jobs of K =
+  // 1000: 50 iterations 17.7 -> 17.0 ms; the streamed passes of 40,000 rows at D = 8192, 2 x 2 (pass 2:
+  // 626 jobs on 304 slots): 10 iterations 14.2 -> 13.7 ms.
+  const int64_t rest = v.njobs % slots, full = v.njobs - rest;
+  int cl = 1;
+  if ((size_t)128 * v.mpad * 4 <= (size_t)a.ns * a.stage_bytes)
+    while (cl < 8 && 2 * cl * rest <= slots) cl *= 2;
+  if (cl == 1 || rest == 0) return run(v.njobs, 1);
+  if (full > 0) {
+    a.njobs = (int)full;
+    if ((e = run(full, 1)) != cudaSuccess) return e;
+  }
+  a.jobs = v.jobs + full;
+  a.njobs = (int)rest;
+  return run(rest, cl);
 }
 
 RFF_CHECK_UNIT(qgemm)
