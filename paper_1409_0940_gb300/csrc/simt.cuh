@@ -10,6 +10,13 @@
 // touch waits in tensor memory (256 words per thread of a 256-thread CTA that holds all 512
 // columns: warp w owns the lanes 32 (w mod 4) .. and the columns from 256 (w / 4)); the words are
 // private to the thread, so only its own stores and loads have to be ordered.
+//
+// Clusters and tensor memory: a CTA that waits for tensor memory while its cluster waits for it is
+// safe only as long as the holder does not wait for that cluster in turn.  Two kernels whose
+// clusters' CTAs hold tensor memory never share an SM beyond its 512 columns: the passes' CTAs take
+// 178 KB of shared memory, the factor products' that park 115 KB with 256 columns or 122 KB and
+// more, the streamed split products' 85 to 112 KB with at most 256 columns, the projection's 160 KB
+// and more.
 #pragma once
 #include "common.cuh"
 #include "tcgen05.cuh"
