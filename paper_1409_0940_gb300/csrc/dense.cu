@@ -229,6 +229,7 @@ __global__ void __launch_bounds__(256) k_gemm_f32_nn(const GemmDesc* __restrict_
         D[(int64_t)gm * g.ldd + tx + 16 * q] = v;
       }
     }
+    if (PARK) tmem_return(tmem_word, gemm_tmem_cols(MQ));
   } else {
     __syncthreads();   // everyone is done reading the ring
 #pragma unroll
@@ -244,6 +245,7 @@ __global__ void __launch_bounds__(256) k_gemm_f32_nn(const GemmDesc* __restrict_
         gm_smem[(GEMM_M + ty + 16 * i) * N + tx + 16 * q] = PARK ? l[i] : lo[PARK ? 0 : q][i];
       }
     }
+    if (PARK) tmem_return(tmem_word, gemm_tmem_cols(MQ));   // before the cluster is waited for
     tc5::cluster_sync_all();
     constexpr int SHARE = GEMM_M * N / GEMM_CL;
     const uint32_t base = tc5::smem_u32(gm_smem);
@@ -268,12 +270,6 @@ __global__ void __launch_bounds__(256) k_gemm_f32_nn(const GemmDesc* __restrict_
       }
     }
     tc5::cluster_sync_all();   // nobody leaves while others read its shared memory
-  }
-  if (PARK) {
-    tc5::fence_before();
-    __syncthreads();
-    tc5::fence_after();
-    if (tid < 32) tc5::tmem_dealloc<1>(tmem_word, gemm_tmem_cols(MQ));
   }
 }
 
@@ -515,10 +511,7 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
       if (gm < s && gn < s) H[gm * s + gn] += (double)hi[j] + (double)lo[j];
     }
   }
-  tc5::fence_before();
-  __syncthreads();
-  tc5::fence_after();
-  if (tid < 32) tc5::tmem_dealloc<1>(tmem_word, 512);
+  tmem_return(tmem_word, 512);
 }
 
 // ------------------------------------------------------------------ diagonal potrf

@@ -304,8 +304,15 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
       if (lane == 0 && mx > 0.f) atomicMax(a.amax, __float_as_uint(mx));
     }
   }
+  // (the roles' single threads rejoin their warps; a cluster is waited for only afterwards, see simt.cuh)
+  __syncwarp();
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (warp == 1) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
+  }
   if (a.cl > 1) {
-    __syncwarp();   // (the roles' single threads rejoin their warps)
     cluster_sync_all();
     const SgJob job = a.jobs[job0];
     if (!q_skip(job, a)) {
@@ -336,12 +343,6 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
       }
     }
     cluster_sync_all();   // nobody leaves while others read its shared memory
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-  if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
   }
 }
 

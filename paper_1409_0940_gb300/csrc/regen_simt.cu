@@ -448,6 +448,7 @@ __global__ void __launch_bounds__(NT, 1) k_pass2_simt(const __grid_constant__ Pa
 #pragma unroll
       for (int i = 0; i < 8; ++i) out[(int64_t)chain_row(b.ty, i) * p.mpad + b.tx + 16 * q] = v[i];
     }
+    tmem_return(tmem_word, 512);
   } else {
     // this part's sums to shared memory (the ring's), then 16 rows per CTA over all parts
     __syncthreads();   // everyone is done reading the ring
@@ -464,6 +465,7 @@ __global__ void __launch_bounds__(NT, 1) k_pass2_simt(const __grid_constant__ Pa
         for (int i = 0; i < 8; ++i) smem[elems + chain_row(b.ty, i) * p.mpad + b.tx + 16 * q] = v[i];
       }
     }
+    tmem_return(tmem_word, 512);   // before the cluster is waited for
     tc5::cluster_sync_all();
     const int share = elems / cl;
     const uint32_t base = tc5::smem_u32(smem);
@@ -488,10 +490,6 @@ __global__ void __launch_bounds__(NT, 1) k_pass2_simt(const __grid_constant__ Pa
     }
     tc5::cluster_sync_all();   // nobody leaves while others read its shared memory
   }
-  tc5::fence_before();
-  __syncthreads();
-  tc5::fence_after();
-  if (threadIdx.x < 32) tc5::tmem_dealloc<1>(tmem_word, 512);
 }
 
 // Pass 1: one CTA per (128 feature slots, row block i, row split); runs over the
@@ -537,10 +535,7 @@ __global__ void __launch_bounds__(NT, 1) k_pass1_simt(const __grid_constant__ Pa
 #pragma unroll
     for (int ii = 0; ii < 8; ++ii) out[(int64_t)chain_row(b.ty, ii) * p.mpad + b.tx + 16 * q] = v[ii];
   }
-  tc5::fence_before();
-  __syncthreads();
-  tc5::fence_after();
-  if (threadIdx.x < 32) tc5::tmem_dealloc<1>(tmem_word, 512);
+  tmem_return(tmem_word, 512);
 }
 
 // half H of T as Z (or Z^T) to out, rows a0.., features b0..

@@ -11,12 +11,11 @@
 // columns: warp w owns the lanes 32 (w mod 4) .. and the columns from 256 (w / 4)); the words are
 // private to the thread, so only its own stores and loads have to be ordered.
 //
-// Clusters and tensor memory: a CTA that waits for tensor memory while its cluster waits for it is
-// safe only as long as the holder does not wait for that cluster in turn.  Two kernels whose
-// clusters' CTAs hold tensor memory never share an SM beyond its 512 columns: the passes' CTAs take
-// 178 KB of shared memory, the factor products' that park 115 KB with 256 columns or 122 KB and
-// more, the streamed split products' 85 to 112 KB with at most 256 columns, the projection's 160 KB
-// and more.
+// Clusters and tensor memory: a CTA whose columns are taken waits in tcgen05.alloc until their
+// holders give them back.  CTAs of two kernels that both held columns while they waited for the rest
+// of their clusters could wait for one another on two SMs without end.  So a CTA of a cluster gives
+// its columns back (tmem_return) before the first barrier of the cluster: whoever holds columns
+// finishes on its own, whatever else shares the SM.
 #pragma once
 #include "common.cuh"
 #include "tcgen05.cuh"
@@ -71,6 +70,14 @@ __device__ __forceinline__ void unpark8(uint32_t taddr, float (&v)[8]) {   // co
   tc5::tmem_wait_ld();
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// every thread is done with the CTA's tensor memory: warp 0 gives it back
+__device__ __forceinline__ void tmem_return(uint32_t tmem, uint32_t cols) {
+  tc5::fence_before();
+  __syncthreads();
+  tc5::fence_after();
+  if (threadIdx.x < 32) tc5::tmem_dealloc<1>(tmem, cols);
 }
 
 __device__ __forceinline__ float ld_cluster(uint32_t addr, uint32_t rank) {   // a CTA's shared memory in the cluster
