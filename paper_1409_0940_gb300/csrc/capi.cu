@@ -27,6 +27,9 @@ struct DevBuf {
 };
 
 constexpr int64_t TS_SCORE_ROWS = 2048;   // TensorSketch scoring: rows sketched per product
+// working_set_bytes adds WS_ALLOWANCE for the allocations' rounding and small tables; pass 1's partial
+// sums beyond the counted row splits take up to WS_FILL of it
+constexpr size_t WS_ALLOWANCE = size_t(64) << 20, WS_FILL = size_t(32) << 20;
 
 // A named host range for profilers (NVTX; nothing happens unless a tool is attached): the
 // set-up stages, the iterations and scoring show up by name on a timeline.
@@ -51,6 +54,7 @@ struct rff_admm_s {
   size_t mem_limit = 0;   // device bytes this handle may use (0: whatever is free)
   int64_t n = 0, d = 0, dld = 0, m = 0, mpad = 0, D = 0, nslots = 0, fslots = 0;
   int R = 1, C = 1, nsplit = 1, nsplit_max = 1, iters_done = 0;
+  int nsplit_counted = 1;   // the row splits of pass 1 that working_set_bytes counts (see compute_geometry)
   int tc_kc = 0;  // ring K chunk of the tensor-core passes, chosen by the autotuner
   int tc_zt = 0;  // 1: Z tile of the tensor-core passes in TMEM (autotuned)
   int tc_cg = 1;  // 2: the tensor-core passes run as CTA pairs (autotuned)
@@ -299,7 +303,7 @@ size_t working_set_bytes(const rff_admm_s& s) {
   t += (size_t)s.C * s.nslots * s.mpad * f * (s.split_path() && !s.outer ? 1 : 2);   // Op (+ FP32 V)
   if (s.split_path()) t += (size_t)s.C * s.nslots * s.mpad * b2 * 2;
   t += (size_t)s.fslots * s.mpad * f * 5;                       // W, Wbar, mu, mu_old, Wbar_old
-  t += (size_t)s.R * s.fslots * s.mpad * f * (3 + s.nsplit_max);    // What, muij, muij_old, Rpart
+  t += (size_t)s.R * s.fslots * s.mpad * f * (3 + s.nsplit_counted);   // What, muij, muij_old, Rpart
   if (s.split_path()) {
     t += (size_t)s.R * s.fslots * s.mpad * b2 * 2 + (size_t)s.fslots * s.mpad * b2 * 2;         // WT, WbT
     if (!s.outer) {
@@ -309,7 +313,7 @@ size_t working_set_bytes(const rff_admm_s& s) {
     if (s.cached_z()) {
       t += (size_t)s.nslots * s.fslots * b2 * 4;                                                // Z, Z^T hi/lo
       t += (size_t)(s.nslots / 128 * s.C + s.fslots / 128 * s.R * s.nsplit_cz) * sizeof(SgJob);
-      t += (size_t)s.R * s.fslots * s.mpad * f * (s.nsplit_cz > s.nsplit_max ? s.nsplit_cz - s.nsplit_max : 0);
+      t += (size_t)s.R * s.fslots * s.mpad * f * (s.nsplit_cz > s.nsplit_counted ? s.nsplit_cz - s.nsplit_counted : 0);
     }
   }
   if (!s.split_path() || s.outer) {
@@ -318,7 +322,7 @@ size_t working_set_bytes(const rff_admm_s& s) {
   }
   if (s.outer) t += (size_t)s.C * s.nslots * s.mpad * f * 2;                                   // e = V - Z c, y
   if (s.tensorsketch()) t += (size_t)TS_SCORE_ROWS * s.fslots * f + 256;   // scoring rows
-  return t + (64u << 20);
+  return t + WS_ALLOWANCE;
 }
 
 // relative weights lambda_c / lambda of the output columns (padding columns 0)
@@ -333,9 +337,10 @@ rff_status upload_lambdas(rff_admm_t h) {
   return RFF_OK;
 }
 
-// Block grid, slot layout and prox steps of a data set of n rows and d inputs.  fill: pass 1's row
-// splits may be raised to fill its last wave (more partial sums: more memory).
-void compute_geometry(rff_admm_s& s, int64_t n, int64_t d, bool fill = true) {
+// Block grid, slot layout and prox steps of a data set of n rows and d inputs.  They depend on the
+// sizes and the device only, never on the memory that is free: a solve's bits and its checkpoints do
+// not depend on what else the device holds.
+void compute_geometry(rff_admm_s& s, int64_t n, int64_t d) {
   s.n = n;
   s.d = d;
   s.dld = round_up(d, 64);
@@ -409,21 +414,24 @@ void compute_geometry(rff_admm_s& s, int64_t n, int64_t d, bool fill = true) {
     want = std::max<int64_t>(want, ceil_div(min_rows, s.split_path() ? 6400 : 1600));
     const int64_t cap = std::min<int64_t>(ceil_div(min_rows, tile), 64);
     s.nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
+    s.nsplit_counted = s.nsplit;
     // on the tensor cores up to twice as many, where that fills the last wave of CTAs (waves times
     // row tiles per CTA, one tile for a CTA's start; shorter chains are no less accurate): 50 iterations
     // of 20,011 rows at D = 3000, 2 x 3 (336 -> 432 CTAs) 17.0 -> 16.3 ms, 20 of 50,000 rows at D = 8192,
-    // 2 x 2 (512 -> 896) 95 -> 93 ms
-    if (fill && s.split_path() && !s.cached_z()) {
+    // 2 x 2 (512 -> 896) 95 -> 93 ms.  Their partial sums stay within WS_FILL, so the memory a solve is
+    // counted with, and with it what set_data and a server admit, is that of the splits above
+    if (s.split_path() && !s.cached_z()) {
+      const int64_t per_split = (int64_t)s.R * s.fslots * s.mpad * (int64_t)sizeof(float);
       const int64_t nrt = ceil_div(*std::max_element(s.row_size.begin(), s.row_size.end()), 128);
       auto cost = [&](int64_t ns) { return ceil_div(ftiles * s.R * ns, (int64_t)nsm) * (ceil_div(nrt, ns) + 1); };
       const int64_t base = s.nsplit;
-      for (int64_t ns = base + 1; ns <= std::min(2 * base, cap); ++ns)
+      for (int64_t ns = base + 1; ns <= std::min(2 * base, cap) && (ns - base) * per_split <= (int64_t)WS_FILL; ++ns)
         if (cost(ns) < cost(s.nsplit)) s.nsplit = (int)ns;
     }
     // RFF_PASS1_SPLITS=k fixes the row splits of pass 1 (bounded by one 128-row tile each)
     if (const char* e = getenv("RFF_PASS1_SPLITS")) {
       const int k = atoi(e);
-      if (k >= 1) s.nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(k, ceil_div(min_rows, tile)));
+      if (k >= 1) s.nsplit = s.nsplit_counted = (int)std::max<int64_t>(1, std::min<int64_t>(k, ceil_div(min_rows, tile)));
     }
     s.nsplit_max = s.nsplit;
     // cached-Z pass 1 (one CTA per 128 features x row range, two CTAs per SM): about
@@ -581,12 +589,8 @@ rff_status set_data_impl(rff_admm_t h, const XInput& xin, const float* Yin, int6
   // memory check before any allocation
   size_t fr = 0, tot = 0;
   CK(cudaMemGetInfo(&fr, &tot));
-  size_t need = working_set_bytes(s) + setup_bytes(s, 1);
+  const size_t need = working_set_bytes(s) + setup_bytes(s, 1);
   const size_t avail = s.mem_limit ? std::min(fr, s.mem_limit) : fr;
-  if (need > avail) {   // with the fewest partial sums of pass 1 before it is refused
-    compute_geometry(s, n, d, false);
-    need = working_set_bytes(s) + setup_bytes(s, 1);
-  }
   if (need > avail) {
     return h->fail(RFF_ENOMEM, "working set " + std::to_string(need >> 20) + " MiB exceeds the " +
                                    std::to_string(avail >> 20) + " MiB available");
