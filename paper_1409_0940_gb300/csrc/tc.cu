@@ -140,7 +140,13 @@ struct TcArgs {
 
 using namespace tc5;
 
-// *p += v, added in the L2 without a reply: a thread's additions to one address keep its order
+// *p += v, added in the L2 without a reply: a thread's additions to one address keep its order.  The
+// L2 flushes subnormal operands and sums, so this is for sums that cannot be subnormal: a scoring
+// group's accumulators are sums of products of FP16 terms, multiples of 2^-48; times sc they are zero
+// or at least sc 2^-48, multiples of sc 2^-72, and so are their sums.  From sc = RED_MIN_SC on those
+// are normal numbers; below it (weights under about 2^-31 at D = 16,384) the rows are read, added and
+// stored, a round trip per 8 columns (50,001 rows at d = 440, m = 147: 2.54 -> 2.7 to 2.9 ms).
+constexpr float RED_MIN_SC = 0x1p-53f;
 __device__ __forceinline__ void red_add_v4(float4* p, float4 v) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                : "memory");
@@ -764,10 +770,15 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
               float4 v1 = make_float4(sc * __uint_as_float(r8[4]), sc * __uint_as_float(r8[5]),
                                       sc * __uint_as_float(r8[6]), sc * __uint_as_float(r8[7]));
               const bool in = RFF_SPAN(orow + c0 + c - a.out, 8, a.out_elems);
-              if (in && add_rows) {   // this thread wrote these values for the groups before
+              if (in && add_rows && sc >= RED_MIN_SC) {   // this thread wrote these values for the groups before
                 red_add_v4(dst, v0);
                 red_add_v4(dst + 1, v1);
               } else if (in) {
+                if (add_rows) {
+                  const float4 p0 = dst[0], p1 = dst[1];
+                  v0 = make_float4(p0.x + v0.x, p0.y + v0.y, p0.z + v0.z, p0.w + v0.w);
+                  v1 = make_float4(p1.x + v1.x, p1.y + v1.y, p1.z + v1.z, p1.w + v1.w);
+                }
                 dst[0] = v0;
                 dst[1] = v1;
               }
@@ -1138,10 +1149,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
               float4 v1 = make_float4(sc * __uint_as_float(r8[4]), sc * __uint_as_float(r8[5]),
                                       sc * __uint_as_float(r8[6]), sc * __uint_as_float(r8[7]));
               const bool in = RFF_SPAN(orow + c0 + c - a.out, 8, a.out_elems);
-              if (in && add_rows) {
+              if (in && add_rows && sc >= RED_MIN_SC) {
                 red_add_v4(dst, v0);
                 red_add_v4(dst + 1, v1);
               } else if (in) {
+                if (add_rows) {
+                  const float4 p0 = dst[0], p1 = dst[1];
+                  v0 = make_float4(p0.x + v0.x, p0.y + v0.y, p0.z + v0.z, p0.w + v0.w);
+                  v1 = make_float4(p1.x + v1.x, p1.y + v1.y, p1.z + v1.z, p1.w + v1.w);
+                }
                 dst[0] = v0;
                 dst[1] = v1;
               }

@@ -38,3 +38,28 @@ def test_scores_do_not_depend_on_the_batch(rff, prec, D, C):
     ref = orff.features_block(Q[rows], 9, 4.0, D, 0, D) @ W.astype(np.float64)
     assert np.linalg.norm(full[rows] - ref) <= 1e-4 * np.linalg.norm(ref)
     s.close()
+
+
+# sums below the smallest normal FP32 number keep their value whichever way they are added: targets
+# of 1e-36 and 1e-38 train weights, and give group sums, that are mostly subnormal
+@pytest.mark.parametrize("prec", ["split_bf16", "cached_z"])
+@pytest.mark.parametrize("scale", [1e-36, 1e-38])
+def test_tiny_scores_do_not_depend_on_the_batch(rff, prec, scale):
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((400, 21)).astype(np.float32)
+    Y = (np.sign(rng.standard_normal((400, 3))) * scale).astype(np.float32)
+    s = rff.Solver(loss="squared", reg="l2", lam=1e-3, sigma=4.0, rho=1.0, D=13000, R=1, C=3, seed=9, m=3, prec=prec)
+    s.set_data(X, Y)
+    s.solve(2)
+    W = s.weights()
+    Q = rng.standard_normal((160 * 128 + 45, 21)).astype(np.float32)
+    full = s.predict(Q)
+    for q in (1, 1000):
+        assert np.array_equal(s.predict(np.ascontiguousarray(Q[:q])), full[:q])
+    # The weights' FP16 split is scaled by at most 2^108, so a weight is off by up to 2^-133 (uniformly:
+    # 2^-133 / sqrt 3 in the root mean square), and a score, with D features of square sum about 1, by
+    # as much; four times that, beside the split path's 1e-4
+    ref = orff.features_block(Q[:50], 9, 4.0, 13000, 0, 13000) @ W.astype(np.float64)
+    split = 4 * np.sqrt(ref.size / 3.0) * 2.0 ** -133
+    assert np.linalg.norm(full[:50].astype(np.float64) - ref) <= 1e-4 * np.linalg.norm(ref) + split
+    s.close()
