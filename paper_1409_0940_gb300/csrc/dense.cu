@@ -539,9 +539,9 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
   __shared__ double col[64];    // t of the current step
   __shared__ double u[64];
   __shared__ double piv[64];    // the pivots d_c, then their square roots
-  __shared__ double rinv[64];   // 1 / d_c, then 1 / sqrt(d_c)
+  __shared__ double rinv[64];   // 1 / d_c (or -1 / (2^shift d_c)), then 1 / sqrt(d_c)
   __shared__ uint16_t elem[64 * 65 / 2];   // (r << 8) | q, r = 63 first
-  __shared__ int bad;
+  __shared__ int bad, shift;    // shift: of the last pivot that needed one
   const int tid = threadIdx.x;
   for (int t = tid; t < 64 * 64; t += 256) {
     const int r = t / 64, c = t % 64;
@@ -558,18 +558,23 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
       d = 1.0;
     }
     piv[c] = d;
-    // 1 / d by Newton's iteration from the FP32 reciprocal (within an ulp or two), shorter than a
-    // division: everything waits for it
+    // 1 / d by Newton's iteration from the FP32 reciprocal, shorter than a division: everything
+    // waits for it.  The second step's error is 2^-92 before its rounding (0.5000 ulp at most in
+    // 20,000 random pivots).  Pivots out of FP32's range are moved into it by 2^shift first: 1 / d
+    // of a subnormal pivot would be infinite, though its square root is an ordinary number
     const float f = (float)d;
     double r;
+    int sh = 0;
     if (f > 1e-30f && f < 1e30f) {
       r = (double)(1.f / f);
       r = fma(r, fma(-d, r, 1.0), r);
       r = fma(r, fma(-d, r, 1.0), r);
     } else {
-      r = 1.0 / d;
+      sh = d < 1.0 ? 512 : -512;
+      r = 1.0 / (d * (sh > 0 ? 0x1p+512 : 0x1p-512));
     }
-    rinv[c] = r;
+    rinv[c] = sh ? -r : r;
+    if (sh) shift = sh;
   };
   for (int t = tid; t < 64 * 64; t += 256) {
     const int r = t / 64, c = t % 64;
@@ -583,7 +588,8 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
       double v;
       if (tid > c) {
         v = M[tid][c];
-        col[tid] = v * rinv[c];
+        const double ri = rinv[c];
+        col[tid] = __double2hiint(ri) >= 0 ? v * ri : v * (shift > 0 ? -0x1p+512 : -0x1p-512) * ri;
         L[tid][c] = v;
         M[tid][c] = 0.0;   // X_rc starts from the identity's zero
       } else {

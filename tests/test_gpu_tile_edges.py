@@ -87,3 +87,19 @@ def test_a_memory_limit_changes_no_result(rff, kw, d, n):
         got.append(s.weights())
         s.close()
     assert np.array_equal(got[0], got[1])
+
+
+# the diagonal blocks multiply by 1 / pivot: pivots whose reciprocal or square is out of range factor
+# as any other (20 copies of one 3 x 3 block with an exact factor; one subnormal pivot among ones)
+@pytest.mark.parametrize("e", [-1060, -1000, -100, 0, 100, 1000, 1018])
+def test_cholesky_of_tiny_and_huge_pivots(rff, e):
+    torch = pytest.importorskip("torch")
+    T = np.array([[2.0, 0, 0], [1, 2, 0], [0, 1, 4]])
+    L = np.kron(np.eye(20), T) * 2.0 ** (e // 2)
+    A = np.kron(np.eye(20), T @ T.T) * 2.0 ** (e - e // 2) * 2.0 ** (e // 2)
+    if e == -1060:
+        L[3:6, 3:6], A[3:6, 3:6] = np.diag([1.0, 2.0 ** -525, 1.0]), np.diag([1.0, 2.0 ** -525 * 2.0 ** -525, 1.0])
+    At, info = torch.from_numpy(A[None].copy()).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    rff.rff_cholesky_f64(At, info)
+    assert info.item() == 0
+    assert np.array_equal(At[0].cpu().numpy(), L)
