@@ -27,9 +27,10 @@ struct DevBuf {
 };
 
 constexpr int64_t TS_SCORE_ROWS = 2048;   // TensorSketch scoring: rows sketched per product
-// working_set_bytes adds WS_ALLOWANCE for the allocations' rounding and small tables; pass 1's partial
-// sums beyond the counted row splits take up to WS_FILL of it
-constexpr size_t WS_ALLOWANCE = size_t(64) << 20, WS_FILL = size_t(32) << 20;
+// working_set_bytes adds WS_ALLOWANCE for the allocations' rounding and small tables.  Pass 1's partial
+// sums beyond the counted row splits take up to WS_FILL of it, the padding of the factors' rows to 16
+// bytes up to WS_PAD, and that of the set-up's chunk of Z at most 0.4 MB
+constexpr size_t WS_ALLOWANCE = size_t(64) << 20, WS_FILL = size_t(32) << 20, WS_PAD = size_t(8) << 20;
 
 // A named host range for profilers (NVTX; nothing happens unless a tool is attached): the
 // set-up stages, the iterations and scoring show up by name on a timeline.
@@ -60,6 +61,7 @@ struct rff_admm_s {
   int tc_cg = 1;  // 2: the tensor-core passes run as CTA pairs (autotuned)
   float t_loss = 0.f, t_reg = 0.f;
   std::vector<int64_t> row_start, row_size, row_slot, col_start, col_size, col_slot, foff;
+  int64_t factor_pad = 0;   // elements of foff.back() that pad the factors' rows
 
   // ---- device memory (owned)
   std::vector<DevBuf> bufs;
@@ -319,6 +321,7 @@ size_t working_set_bytes(const rff_admm_s& s) {
   if (!s.split_path() || s.outer) {
     t += (size_t)s.R * s.fslots * s.mpad * f;                                                   // rhs
     t += (size_t)s.foff.back() * f + (size_t)s.R * s.C * sizeof(GemmDesc);                     // factors
+    t -= std::min<size_t>((size_t)s.factor_pad * f, WS_PAD);
   }
   if (s.outer) t += (size_t)s.C * s.nslots * s.mpad * f * 2;                                   // e = V - Z c, y
   if (s.tensorsketch()) t += (size_t)TS_SCORE_ROWS * s.fslots * f + 256;   // scoring rows
@@ -370,10 +373,12 @@ void compute_geometry(rff_admm_s& s, int64_t n, int64_t d) {
     s.outer = s.p.prec != RFF_PREC_CACHED_Z && nmax < smin;
   }
   s.foff.assign((size_t)s.R * s.C + 1, 0);
+  s.factor_pad = 0;
   for (int i = 0; i < s.R; ++i)
     for (int j = 0; j < s.C; ++j) {
       const int64_t fd = s.outer ? s.row_size[i] : s.col_size[j];
       s.foff[(size_t)i * s.C + j + 1] = s.foff[(size_t)i * s.C + j] + fd * round_up(fd, 4);
+      s.factor_pad += fd * (round_up(fd, 4) - fd);
     }
   s.qrow.assign((size_t)s.R * s.C, 0);
   s.q_rows = 0;
@@ -484,7 +489,7 @@ size_t setup_bytes(const rff_admm_s& s, int64_t batch) {
   int64_t smax = 0;
   for (int j = 0; j < s.C; ++j) smax = std::max(smax, s.col_size[j]);
   const int64_t chunk_rows = std::min<int64_t>(32768, round_up(*std::max_element(s.row_size.begin(), s.row_size.end()), SLOT));
-  const size_t t = (size_t)batch * smax * smax * 8 * 2 + (size_t)chunk_rows * round_up(smax, SLOT) * 4 +
+  const size_t t = (size_t)batch * smax * smax * 8 * 2 + (size_t)chunk_rows * smax * 4 +
                    factor_scratch_bytes((int)batch, (int)smax) + (size_t)batch * 4 + 4096 +
                    (tc_gram(s) ? tc_gram_bytes(chunk_rows, smax) : 0);
   // the cached-Z precision forms Z in the same scratch first, in row chunks of ~256 MB
@@ -1235,12 +1240,12 @@ rff_status setup_factors(rff_admm_t h) {
   // of work for the regeneration and 30 for the Gram (512 launches of each, 243 ms, on the
   // 20k x 32,768 workload at 32 x 8; in 16 launches of each, 19 ms)
   const int64_t chunk_feat = std::min<int64_t>(2048, round_up(smax, SLOT));
-  const int64_t smax_pad = round_up(smax, SLOT);
+  const int64_t ldzc = round_up(smax, 4);   // rows of the chunk of Z: 16 bytes for the Gram's copies
   const int64_t zt_blocks = std::max<int64_t>(
       1, std::min<int64_t>(s.R, (int64_t)(std::min<size_t>(OUTER_ZT_BYTES, budget / 8) /
                                           ((size_t)round_up(nmax, SLOT) * chunk_feat * 4))));
   const size_t zbytes = (s.outer ? (size_t)zt_blocks * round_up(nmax, SLOT) * chunk_feat * 4
-                                 : (size_t)chunk_rows * smax_pad * 4) +
+                                 : (size_t)chunk_rows * ldzc * 4) +
                         (tc_gram(s) ? tc_gram_bytes(chunk_rows, smax) : 0);
   budget = budget > zbytes + (256u << 20) ? budget - zbytes - (256u << 20) : 0;
   int64_t batch = std::max<int64_t>(1, std::min<int64_t>(nblocks, (int64_t)(budget / std::max<size_t>(per_block + factor_scratch_bytes(1, (int)fmax), 1))));
@@ -1258,7 +1263,7 @@ rff_status setup_factors(rff_admm_t h) {
   float* Zc = reinterpret_cast<float*>(Q64 + batch * fmax * fmax);
   // tensor-core Gram buffers after the row chunk, on a 256-byte boundary (tc_gram_bytes keeps 1 KB of slack)
   char* gbase = reinterpret_cast<char*>(
-      round_up((uintptr_t)(reinterpret_cast<char*>(Zc) + (size_t)chunk_rows * smax_pad * 4), (uintptr_t)256));
+      round_up((uintptr_t)(reinterpret_cast<char*>(Zc) + (size_t)chunk_rows * ldzc * 4), (uintptr_t)256));
   int32_t* info = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(Zc) + zbytes);
   void* fscr = reinterpret_cast<char*>(info) + round_up(batch * 4, 256);
 
@@ -1280,8 +1285,8 @@ rff_status setup_factors(rff_admm_t h) {
       for (int64_t r = 0; !s.outer && r < s.row_size[i]; r += chunk_rows) {
         const int64_t nr = std::min(chunk_rows, s.row_size[i] - r);
         if (s.split_path() && getenv("RFF_DIAG_SIMT_GRAM")) {
-          CK(tc_write_z(tc_view(s), s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, smax_pad));
-          CK(launch_gram_f32_to_f64(Zc, smax_pad, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
+          CK(tc_write_z(tc_view(s), s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, ldzc));
+          CK(launch_gram_f32_to_f64(Zc, ldzc, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
           continue;
         }
         if (tc_gram(s)) {   // Z^T's split written by the regeneration itself, or the stored one
@@ -1293,9 +1298,9 @@ rff_status setup_factors(rff_admm_t h) {
         }
         // FP32 precision: Z on the SIMT pipes, its Gram from FP32 products with float-float sums
         ZArgs za{s.X32, s.dld, s.Gt32, s.dld, (int)round_up(s.d, 4), s.bias, scale, s.row_of_slot, s.feat_of_slot,
-                 s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, smax_pad, s.p.feature_map, 0};
+                 s.row_slot[i] + r, nr, s.col_slot[j], sj, Zc, ldzc, s.p.feature_map, 0};
         CK(launch_write_z_simt(za, s.st));
-        CK(launch_gram_f32_to_f64(Zc, smax_pad, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
+        CK(launch_gram_f32_to_f64(Zc, ldzc, nr, nullptr, nullptr, sj, 1, Hb, 0, s.st));
       }
     }
     // outer form: H = I + Z Z^T accumulated over feature chunks (the rows of Z^T); the batch's row

@@ -433,18 +433,21 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
   const int tid = threadIdx.x, tx = thread_tx(), ty = thread_ty();
   if (tid < 32) tc5::tmem_alloc<1>(tc5::smem_u32(&tmem_word), 512);
   const int64_t nst = ceil_div(n, GR_K);
+  // this thread's four columns of either operand: zeros past the matrix (rows are padded to 16 bytes)
+  const int c4 = 4 * (tid % 32);
+  const bool a_in = a0 + c4 < s, b_in = b0 + c4 < s;
+  const int64_t a_col = a_in ? a0 + c4 : 0, b_col = b_in ? b0 + c4 : 0;
   auto issue = [&](int64_t st) {
     if (st < nst) {
       float* As = gr_smem + (st % GR_NS) * (2 * GR_K * GR_T);
       float* Bs = As + GR_K * GR_T;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int e = tid + 256 * q, r = e / 32, c = 4 * (e % 32);
+        const int r = tid / 32 + 8 * q;
         const int64_t gr = st * GR_K + r;
         const float* row = Z + (gr < n ? gr : n - 1) * ldz;   // rows past n: zeros
-        const int bytes = gr < n ? 16 : 0;
-        cp_async16_fill(As + r * GR_T + c, row + a0 + c, bytes);
-        cp_async16_fill(Bs + r * GR_T + c, row + b0 + c, bytes);
+        cp_async16_fill(As + r * GR_T + c4, row + a_col, gr < n && a_in ? 16 : 0);
+        cp_async16_fill(Bs + r * GR_T + c4, row + b_col, gr < n && b_in ? 16 : 0);
       }
     }
     cp_commit();

@@ -41,6 +41,17 @@ def test_estimates_count_the_fewest_splits(rff, monkeypatch):
     assert estimate(rff, monkeypatch)[0] < estimate(rff, monkeypatch, 9)[0]
 
 
+def test_estimates_count_features_not_tiles(rff):
+    """Rows padded for the kernels' 16-byte copies come out of the allowance."""
+    def fp32(D, C, n):
+        return rff.rff_admm_estimate_bytes(rff.make_params(prec="fp32", D=D, R=1, C=C, m=1), n, 10)
+    # the set-up's chunk of Z: 32,768 rows of D floats (the factorisation's scratch is the same for both)
+    (r1, p1), (r2, p2) = fp32(129, 1, 40_000), fp32(160, 1, 40_000)
+    assert (p2 - r2) - (p1 - r1) == 32_768 * 31 * 4 + 16 * (160 ** 2 - 129 ** 2)
+    # the factors (the slots are the same for both)
+    assert fp32(8 * 132, 8, 4000)[0] - fp32(8 * 129, 8, 4000)[0] == 4 * 8 * (132 ** 2 - 129 ** 2)
+
+
 def train(rff, data, limit=0, iters=6, state=None):
     s = rff.Solver(**CASE)
     if limit:
