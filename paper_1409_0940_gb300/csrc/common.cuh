@@ -80,34 +80,6 @@ __device__ __forceinline__ float cos_rr(float x) {
   return (static_cast<int>(k) & 1) ? -p : p;
 }
 
-// 2^E cos(x), bit for bit 2^E cos_rr(x), with fewer instructions for the tensor-core
-// epilogues (where the cosine's instruction count, not the tensor pipe, bounds the small-d
-// workloads): k = rint(x / pi) by adding and subtracting 1.5 2^23 to the rounded quotient
-// (exact for |x / pi| < 2^22) instead of a rounding and a float-to-integer conversion on the
-// transcendental unit, the parity of k read from the low mantissa bit of the biased sum, the
-// sign applied by flipping the sign bit, and 2^E folded into the polynomial's coefficients
-// (scaling by a power of two commutes with every rounding of the evaluation).
-template <int E>
-__device__ __forceinline__ float cos_rr_pow2(float x) {
-  constexpr float S = (float)(1u << E);
-  const float inv_pi = 0.318309886183790672f;
-  const float pi_hi = 3.14159274101257324f;
-  const float pi_lo = -8.74227765734758577e-08f;
-  const float magic = 12582912.f;   // 1.5 2^23
-  const float biased = __fadd_rn(__fmul_rn(x, inv_pi), magic);   // not contracted: rint of the rounded quotient
-  const float k = __fsub_rn(biased, magic);
-  float r = fmaf(-k, pi_hi, x);
-  r = fmaf(-k, pi_lo, r);
-  const float s = r * r;
-  float p = -2.605149518331018e-07f * S;
-  p = fmaf(p, s, 2.476016197761055e-05f * S);
-  p = fmaf(p, s, -0.0013888361863791943f * S);
-  p = fmaf(p, s, 0.04166663810610771f * S);
-  p = fmaf(p, s, -0.5f * S);
-  p = fmaf(p, s, 1.0f * S);
-  return __int_as_float(__float_as_int(p) ^ (__float_as_int(biased) << 31));
-}
-
 // ------------------------------------------------------------------ packed FP32
 // Two FP32 operations in one instruction, each rounded as its scalar form (and not contracted).  A
 // pair is the two words of a 64-bit register.
@@ -137,9 +109,14 @@ __device__ __forceinline__ void unpair2(f32x2 v, float& lo, float& hi) {
 }
 __device__ __forceinline__ f32x2 both2(float v) { return pair2(v, v); }
 
-// 2^E cos of both words, bit for bit cos_rr_pow2<E> of each: half the issue slots of the two scalar
-// evaluations.  The sign of odd k is added as k's low bit times 2^31 (modulo 2^32 the same as
-// flipping the sign bit, in one instruction).
+// 2^E cos of both words, bit for bit 2^E cos_rr of each, with fewer instructions for the tensor-core
+// epilogues (where the cosine's instruction count, not the tensor pipe, bounds the small-d
+// workloads): k = rint(x / pi) by adding and subtracting 1.5 2^23 to the rounded quotient
+// (exact for |x / pi| < 2^22) instead of a rounding and a float-to-integer conversion on the
+// transcendental unit, the parity of k read from the low mantissa bit of the biased sum and added as
+// that bit times 2^31 (modulo 2^32 the same as flipping the sign bit, in one instruction), and 2^E
+// folded into the polynomial's coefficients (scaling by a power of two commutes with every rounding
+// of the evaluation).
 template <int E>
 __device__ __forceinline__ f32x2 cos2_pow2(f32x2 x) {
   constexpr float S = (float)(1u << E);

@@ -492,12 +492,7 @@ __global__ void __launch_bounds__(256, row_loss(LOSS) && PL > 5 ? 3 : 4) k_excha
       else y[q] = 0.f;
     }
     float o[PL];
-    if (row_loss(LOSS)) {
-      prox_row(LOSS, w_in, y, a.m, a.t_loss, a.newton, o);
-    } else {
-#pragma unroll
-      for (int q = 0; q < PL; ++q) o[q] = prox_scalar(LOSS, w_in[q], y[q], a.t_loss, a.newton);
-    }
+    prox_row(LOSS, w_in, y, a.m, a.t_loss, a.newton, o);
 #pragma unroll
     for (int q = 0; q < PL; ++q) {
       const int k = lane + 32 * q;

@@ -60,7 +60,7 @@ constexpr int NTHREADS = 64 + 32 * NEPI;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t ACC2_COL = 256;         // acc2 with a single acc1 (ZT 0, 1)
 constexpr int MAXG = 64;                    // groups (column blocks) per CTA
-static_assert(COS_SCALE == 128.f, "the epilogues form COS_SCALE cos(.) as cos_rr_pow2<7>");
+static_assert(COS_SCALE == 128.f, "the epilogues form COS_SCALE cos(.) as cos2_pow2<7>");
 constexpr int PRED_GT = 8;                  // scoring: feature tiles per group, at least
 constexpr size_t PRED_PART_BYTES = size_t(64) << 20;   // the most a split batch may take for its groups' sums
 
