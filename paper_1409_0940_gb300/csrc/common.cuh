@@ -80,6 +80,20 @@ __device__ __forceinline__ float cos_rr(float x) {
   return (static_cast<int>(k) & 1) ? -p : p;
 }
 
+// SMs of the device (asked once; 148 where there is none to ask)
+inline int device_sms() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      v = 0;
+    }
+    return v > 0 ? v : 148;
+  }();
+  return n;
+}
+
 // ------------------------------------------------------------------ packed FP32
 // Two FP32 operations in one instruction, each rounded as its scalar form (and not contracted).  A
 // pair is the two words of a 64-bit register.

@@ -637,18 +637,6 @@ __global__ void k_zero_strict_upper(double* A, int64_t s) {
 }  // namespace
 
 namespace {
-int dense_sms() {
-  static int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      v = 0;
-    cudaGetLastError();
-    return v > 0 ? v : 148;
-  }();
-  return n;
-}
-
 template <int MQ>
 cudaError_t launch_gemm_mq(const GemmDesc* descs, const GemmDesc& one, int nbatch, int maxM, int maxK, float alpha,
                            float beta, const uint8_t* bmask, cudaStream_t st) {
@@ -658,7 +646,7 @@ cudaError_t launch_gemm_mq(const GemmDesc* descs, const GemmDesc& one, int nbatc
   // One CTA per 128 rows, or a cluster sharing its K chunks where that ends sooner: waves times
   // chunks per CTA, four chunks for filling the ring and, in a cluster, the exchange (clusters of
   // eight leave about an eighth of the SMs unused)
-  const int64_t ctas = ceil_div(maxM, GEMM_M) * nbatch, nch = ceil_div(maxK, GEMM_K), nsm = dense_sms();
+  const int64_t ctas = ceil_div(maxM, GEMM_M) * nbatch, nch = ceil_div(maxK, GEMM_K), nsm = device_sms();
   const int64_t whole = ceil_div(ctas, nsm) * (nch + 2);
   const int64_t shared = ceil_div(ctas * GEMM_CL, nsm * 7 / 8) * (ceil_div(nch, GEMM_CL) + 4);
   const int cl = 16 * MQ <= GEMM_CL_MAX_N && shared < whole ? GEMM_CL : 1;

@@ -470,17 +470,6 @@ OzShape oz_shape(int ph, int k, int s) {
   }
 }
 
-int sm_count() {
-  static int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess)
-      v = 0;
-    return v > 0 ? v : 1;
-  }();
-  return n;
-}
-
 // work items of one product: per 128-row block, its columns (those on or left of the block
 // diagonal when lower) in pieces of `cols`
 template <typename F>
@@ -502,7 +491,7 @@ int oz_item_cols(const OzShape& sh, int nj) {
     return n * nj;
   };
   int w = OZ_ITEM_COLS;
-  while (w > OZ_BN && count(w) < sm_count()) w /= 2;
+  while (w > OZ_BN && count(w) < device_sms()) w /= 2;
   return w;
 }
 
@@ -717,7 +706,7 @@ cudaError_t factor_and_invert_sliced(const std::vector<MatJob>& jobs, bool inver
   a.err = tc_error_ptr();
   if (!a.err) return cudaErrorMemoryAllocation;
   a.timeout_cycles = 4000000000LL;   // about two seconds at the boost clock
-  const int nsm = sm_count();
+  const int nsm = device_sms();
 
   // slices of both operands of phase ph (rows up to rowsA / rowsB, zero to the tile edge), then
   // the product over its work items

@@ -425,17 +425,6 @@ __global__ void k_split3_q(const double* __restrict__ Q, int s, int64_t ldq, int
   q3[o] = l;
 }
 
-int qsm_count() {
-  static int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess)
-      v = 0;
-    return v > 0 ? v : 1;
-  }();
-  return n;
-}
-
 template <int NA, int NB, int F16, int KC>
 cudaError_t set_smem_attr() {
   static std::once_flag once;
@@ -524,7 +513,7 @@ cudaError_t split_gemm(const SgView& v) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern(), QNT, smem);
   if (e != cudaSuccess) return e;
   per_sm = std::min(std::max(per_sm, 1), std::max(1, 512 / (int)a.tmem_cols));
-  const int64_t slots = (int64_t)qsm_count() * per_sm;
+  const int64_t slots = (int64_t)device_sms() * per_sm;
   auto run = [&](int64_t grid, int cl) -> cudaError_t {
     a.cl = cl;
     cudaLaunchConfig_t cfg{};

@@ -578,18 +578,6 @@ __global__ void __launch_bounds__(NT, 1) k_write_z_simt(const __grid_constant__ 
   if (wd == 2) write_z_half<1>(p, b, acc, a0, b0 + BN);
 }
 
-int simt_sms() {
-  static int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      v = 0;
-    cudaGetLastError();
-    return v > 0 ? v : 148;
-  }();
-  return n;
-}
-
 template <int MQ>
 cudaError_t launch_pass2_mq(const PassArgs& p, int64_t items, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_pass2_simt<MQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
@@ -597,7 +585,7 @@ cudaError_t launch_pass2_mq(const PassArgs& p, int64_t items, cudaStream_t st) {
   // Whole waves of items go one to a CTA; the rest, which would leave SMs idle for a whole item's
   // time, goes to clusters of PARTS CTAs where those end sooner (an eighth of the tiles per
   // CTA; clusters of eight leave about an eighth of the SMs unused)
-  const int64_t nsm = simt_sms(), units = p.per_block ? p.C : 1;
+  const int64_t nsm = device_sms(), units = p.per_block ? p.C : 1;
   const int64_t nt = ceil_div(p.g_rows / BN, units);   // feature tiles of an item
   int64_t full = items / nsm * nsm, rest = items - full;
   const int cl = nt > 4 ? PARTS : nt > 2 ? 4 : 2;

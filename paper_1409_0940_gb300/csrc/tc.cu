@@ -1303,19 +1303,6 @@ int* err_word() {
   return p;
 }
 
-int sm_count() {
-  static int n = 0;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      n = 148;
-    }
-  });
-  return n;
-}
-
 int view_kc(const TcView& v) { return (v.kc == 32 || v.kc == 64) ? v.kc : ring_kc(); }
 int view_cg(const TcView& v) { return (v.cg == 2 && v.zt != 3) ? 2 : 1; }
 int view_zt(const TcView& v) {
@@ -1426,7 +1413,7 @@ cudaError_t write_z(const TcView& view, int64_t r0, int64_t nr, int64_t f0, int6
   const int64_t rt = ceil_div(nr, 128), nt = ceil_div(nf, 128);
   int64_t best = 1, cost = INT64_MAX;
   for (int64_t ny = 1; ny <= std::min<int64_t>(nt, 1024); ++ny) {
-    const int64_t c = ceil_div(rt * ny, sm_count()) * (2 * ceil_div(nt, ny) + 1);
+    const int64_t c = ceil_div(rt * ny, device_sms()) * (2 * ceil_div(nt, ny) + 1);
     if (c < cost) {
       cost = c;
       best = ny;
@@ -1536,7 +1523,7 @@ cudaError_t tc_pass2(const TcView& v, const __half* Mhi, const __half* Mlo, int6
   // none takes more than MAXG work items
   const int cg = view_cg(v);
   const int maxg = view_zt(v) == 3 ? W_MAXG : MAXG;
-  const int64_t grid = std::min<int64_t>(nitems, std::max<int64_t>(sm_count() / cg, ceil_div(nitems, maxg)));
+  const int64_t grid = std::min<int64_t>(nitems, std::max<int64_t>(device_sms() / cg, ceil_div(nitems, maxg)));
   return launch(a, dim3((unsigned)(grid * cg)), v.st, view_kc(v), view_zt(v), cg);
 }
 
@@ -1596,13 +1583,13 @@ cudaError_t tc_multi_create(const TcView* views, int n, int which, float* const*
     }
     int64_t used = 0;
     for (int g = 0; g < n; ++g) {
-      const int64_t share = std::max<int64_t>(1, (int64_t)(sm_count() * work[g] / std::max(total, 1.0)));
+      const int64_t share = std::max<int64_t>(1, (int64_t)(device_sms() * work[g] / std::max(total, 1.0)));
       t->m.gx[g] = std::min<int64_t>(std::max<int64_t>(items[g], 1),
                                      std::max<int64_t>(share, ceil_div(items[g], MAXG)));
       t->m.gy[g] = 1;
       used += t->m.gx[g];
     }
-    for (; used < sm_count(); ++used) {
+    for (; used < device_sms(); ++used) {
       int best = -1;
       for (int g = 0; g < n; ++g)
         if (t->m.gx[g] < items[g] && (best < 0 || work[g] / t->m.gx[g] > work[best] / t->m.gx[best])) best = g;
@@ -1712,7 +1699,7 @@ cudaError_t tc_predict(const TcView& v, const __half* Xh, const __half* Xl, int6
                        size_t part_bytes) {
   if (nrows <= 0) return cudaSuccess;
   if (nrows % 128) return cudaErrorInvalidValue;
-  const int64_t tiles = nrows / 128, nsm = sm_count();
+  const int64_t tiles = nrows / 128, nsm = device_sms();
   const int gt = pred_group(v);
   const int64_t ngr = ceil_div(v.fslots / 128, gt);
   const int64_t full = tiles / nsm * nsm, rest = tiles - full;
@@ -1737,7 +1724,7 @@ cudaError_t tc_predict(const TcView& v, const __half* Xh, const __half* Xl, int6
 }
 
 size_t tc_predict_part_bytes(const TcView& v, int64_t nrows) {
-  const int64_t rest = nrows / 128 % sm_count(), ngr = ceil_div(v.fslots / 128, pred_group(v));
+  const int64_t rest = nrows / 128 % device_sms(), ngr = ceil_div(v.fslots / 128, pred_group(v));
   const size_t need = (size_t)ngr * rest * 128 * v.mpad * sizeof(float);
   return ngr > 1 && view_cg(v) == 1 && need <= PRED_PART_BYTES ? need : 0;
 }
