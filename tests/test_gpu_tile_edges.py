@@ -68,13 +68,14 @@ def test_ragged_solves_match_the_oracle(rff, prec, tol, n, d, m, D, R, C):
     s.close()
 
 
-# With a memory limit the forward sweep runs after the factorisation instead of beside it, the outer
-# form takes fewer row blocks at once, and TensorSketch features are formed in row chunks
+# With a memory limit the forward sweep runs after the factorisation instead of beside it, and a
+# TensorSketch solve forms its features in row chunks (9,000 rows of 8,192 features: 256 MB take 8,192
+# rows) instead of whole
 @pytest.mark.parametrize("kw,d,n", [
     (dict(D=900, R=2, C=3, prec="split_bf16"), 10, 2000),
     (dict(D=900, R=2, C=1, prec="fp32"), 10, 2000),
     (dict(D=2000, R=6, C=2, prec="fp32"), 10, 1500),
-    (dict(D=600, R=1, C=2, prec="cached_z", feature_map="tensorsketch", degree=3, coef0=1.0), 20, 1500)])
+    (dict(D=8192, R=1, C=2, prec="cached_z", feature_map="tensorsketch", degree=2, coef0=1.0), 20, 9000)])
 def test_a_memory_limit_changes_no_result(rff, kw, d, n):
     X, Y = data(n, d, 4)
     got = []
@@ -87,6 +88,60 @@ def test_a_memory_limit_changes_no_result(rff, kw, d, n):
         got.append(s.weights())
         s.close()
     assert np.array_equal(got[0], got[1])
+
+
+# The outer form's set-up takes Z^T of several row blocks at once and factors blocks in batches.  Of
+# 100 row blocks by 2 column blocks, limits of some MB above the resident set leave room for batches
+# of 1 block, of 31 (that begin and end within a row of the grid) and of 133, whose row blocks are more
+# than the 46 that Z^T is then formed for at once
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("split_bf16", 1e-4)])
+def test_outer_set_up_in_batches(rff, prec, tol):
+    kw = dict(loss="squared", reg="l2", lam=1e-3, sigma=4.0, rho=1.0, D=4201, R=100, C=2, seed=5)
+    X, Y = data(12_737, 6, 2)
+    ref = admm.admm(admm.Problem(X, Y, **kw), 4)["Wbar"]
+    resident = rff.rff_admm_estimate_bytes(rff.make_params(prec=prec, m=2, **kw), *X.shape)[0]
+    got = []
+    for extra in (0, 290, 310, 370):
+        s = rff.Solver(prec=prec, m=2, **kw)
+        if extra:
+            rff.rff_admm_set_memory_limit(s.h, resident + (extra << 20))
+        s.set_data(X, Y)
+        s.solve(4, stats=False)
+        got.append(s.weights())
+        s.close()
+    assert rel(got[0], ref) <= tol
+    assert all(np.array_equal(g, got[0]) for g in got)
+
+
+# ... and, without a limit, more row blocks than 256 MB of Z^T hold (36 of 40)
+def test_outer_set_up_of_more_row_blocks_than_fit_at_once(rff):
+    kw = dict(loss="squared", reg="l2", lam=1e-3, sigma=4.0, rho=1.0, D=2100, R=40, C=1, seed=5)
+    X, Y = data(33_501, 6, 2)
+    ref = admm.admm(admm.Problem(X, Y, **kw), 3)["Wbar"]
+    s = rff.Solver(prec="fp32", m=2, **kw)
+    s.set_data(X, Y)
+    s.solve(3, stats=False)
+    assert rel(s.weights(), ref) <= 1e-5
+    s.close()
+
+
+# the row losses by outputs per lane: 2, 3, 5 (of 4) and 8 (of 7), with ragged lanes; their step tests
+# go through another kernel
+@pytest.mark.parametrize("loss", ["multinomial", "crammer_singer"])
+@pytest.mark.parametrize("m", [40, 70, 115, 200])
+def test_row_losses_by_outputs_per_lane(rff, loss, m):
+    rng = np.random.default_rng(m)
+    X = rng.standard_normal((700, 9)).astype(np.float32)
+    Y = np.full((700, m), -1.0, np.float32)
+    Y[np.arange(700), rng.integers(0, m, 700)] = 1.0
+    kw = dict(loss=loss, reg="l2", lam=1e-3, sigma=3.0, rho=1.0, D=300, R=2, C=2, seed=5)
+    ref = admm.admm(admm.Problem(X, Y, **kw), 8)["Wbar"]
+    for prec, tol in (("fp32", 1e-5), ("split_bf16", 1e-4)):
+        s = rff.Solver(prec=prec, m=m, **kw)
+        s.set_data(X, Y)
+        s.solve(8, stats=False)
+        assert rel(s.weights(), ref) <= tol, prec
+        s.close()
 
 
 # the diagonal blocks multiply by 1 / pivot: pivots whose reciprocal or square is out of range factor
