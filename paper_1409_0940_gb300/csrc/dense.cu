@@ -518,6 +518,31 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
 }
 
 // ------------------------------------------------------------------ diagonal potrf
+// Blocks whose diagonal lies far from 1 (a subnormal pivot's reciprocal would be infinite, though its
+// square root is an ordinary number) are factored as S A S, S = diag(2^sexp) bringing the diagonal into
+// [1, 4); L of S A S is S L, and its inverse L^-1 S^-1.  Called, not inlined: they are rare, and the
+// kernel's code is fetched anew for every one of its short launches.
+__device__ __noinline__ void scale_block(double (*M)[65], int* sexp) {
+  const int tid = threadIdx.x;
+  if (tid < 64) {
+    int e = 1;
+    const double d = M[tid][tid];
+    if (d > 0.0 && isfinite(d)) frexp(d, &e);   // in [2^(e-1), 2^e)
+    sexp[tid] = -((e - 1) >> 1);
+  }
+  __syncthreads();
+  for (int t = tid; t < 64 * 64; t += 256)
+    M[t / 64][t % 64] = ldexp(ldexp(M[t / 64][t % 64], sexp[t / 64]), sexp[t % 64]);
+  __syncthreads();
+}
+__device__ __noinline__ void unscale_block(double* A, int64_t ld, double* inv, int bs, const int* sexp) {
+  for (int t = threadIdx.x; t < 64 * 64; t += 256) {   // (the elements this thread wrote)
+    const int r = t / 64, c = t % 64;
+    if (r < bs && c < bs) A[r * ld + c] = ldexp(A[r * ld + c], -sexp[r]);
+    inv[t] = ldexp(inv[t], sexp[c]);
+  }
+}
+
 // One CTA per matrix: factor the bs x bs diagonal block starting at column kcol
 // (bs = min(64, s - kcol)) in shared memory, write L back (upper part zeroed) and
 // the inverse of L into inv (64 x 64, zero padded).  info = column+1 of the first
@@ -542,9 +567,9 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
   __shared__ double col[64];    // t of the current step
   __shared__ double u[64];
   __shared__ double piv[64];    // the pivots d_c, then their square roots
-  __shared__ double rinv[64];   // 1 / d_c (or -1 / (2^shift d_c)), then 1 / sqrt(d_c)
+  __shared__ double rinv[64];   // 1 / d_c, then 1 / sqrt(d_c)
   __shared__ uint16_t elem[64 * 65 / 2];   // (r << 8) | q, r = 63 first
-  __shared__ int bad, shift;    // shift: of the last pivot that needed one
+  __shared__ int bad, sexp[64];   // S = diag(2^sexp)
   const int tid = threadIdx.x;
   for (int t = tid; t < 64 * 64; t += 256) {
     const int r = t / 64, c = t % 64;
@@ -563,27 +588,27 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
     piv[c] = d;
     // 1 / d by Newton's iteration from the FP32 reciprocal, shorter than a division: everything
     // waits for it.  The second step's error is 2^-92 before its rounding (0.5000 ulp at most in
-    // 20,000 random pivots).  Pivots out of FP32's range are moved into it by 2^shift first: 1 / d
-    // of a subnormal pivot would be infinite, though its square root is an ordinary number
+    // 20,000 random pivots)
     const float f = (float)d;
     double r;
-    int sh = 0;
     if (f > 1e-30f && f < 1e30f) {
       r = (double)(1.f / f);
       r = fma(r, fma(-d, r, 1.0), r);
       r = fma(r, fma(-d, r, 1.0), r);
     } else {
-      sh = d < 1.0 ? 512 : -512;
-      r = 1.0 / (d * (sh > 0 ? 0x1p+512 : 0x1p-512));
+      r = 1.0 / d;
     }
-    rinv[c] = sh ? -r : r;
-    if (sh) shift = sh;
+    rinv[c] = r;
   };
+  int far = 0;
   for (int t = tid; t < 64 * 64; t += 256) {
     const int r = t / 64, c = t % 64;
-    M[r][c] = (r < bs && c < bs) ? jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] : (r == c ? 1.0 : 0.0);
+    const double v = (r < bs && c < bs) ? jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] : (r == c ? 1.0 : 0.0);
+    M[r][c] = v;
+    if (r == c) far |= (unsigned)((__double2hiint(v) >> 20) - (1023 - 96)) > 2u * 96u;   // sign and exponent
   }
-  __syncthreads();
+  const bool scaled = __syncthreads_or(far) != 0;
+  if (scaled) scale_block(M, sexp);
   if (tid == 0) pivot(0, M[0][0]);
   __syncthreads();
   for (int c = 0; c < bs; ++c) {
@@ -591,8 +616,7 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
       double v;
       if (tid > c) {
         v = M[tid][c];
-        const double ri = rinv[c];
-        col[tid] = __double2hiint(ri) >= 0 ? v * ri : v * (shift > 0 ? -0x1p+512 : -0x1p-512) * ri;
+        col[tid] = v * rinv[c];
         L[tid][c] = v;
         M[tid][c] = 0.0;   // X_rc starts from the identity's zero
       } else {
@@ -625,6 +649,7 @@ __global__ void __launch_bounds__(256) k_potrf_diag(const DiagJob* __restrict__ 
     if (in) jb.A[(int64_t)(kcol + r) * jb.ld + kcol + c] = c < r ? L[r][c] * rinv[c] : c == r ? piv[r] : 0.0;
     jb.inv[t] = in && c <= r ? (c < r ? M[r][c] : 1.0) * rinv[r] : 0.0;
   }
+  if (scaled) unscale_block(jb.A + (int64_t)kcol * jb.ld + kcol, jb.ld, jb.inv, bs, sexp);
   if (tid == 0 && bad && jb.info && *jb.info == 0) *jb.info = bad;
 }
 
