@@ -883,7 +883,11 @@ cudaError_t launch_prox_reg(int reg, const float* V, const float* mu, int64_t n,
 }
 
 namespace {
-// the row losses by outputs per lane: at m = 147 five instead of eight (multinomial, 40,000 rows: 409 -> 340 us)
+// The row losses by outputs per lane: at m = 147 five instead of eight (multinomial, 40,000 rows: 409 ->
+// 340 us).  Four, six and seven outputs per lane have no instance and run as five and eight, which costs
+// them, on 40,000 rows with 2 column blocks, 237 us instead of 225 (m = 112 and 128), 369 instead of 340
+// (m = 176 and 192) and 410 instead of 399 (m = 208 and 224) for the multinomial loss, and 49 / 45, 73 /
+// 64 and 77 / 73 us for Crammer-Singer
 template <int LOSS>
 cudaError_t launch_exchange(const RowEpiArgs& a, unsigned grid, size_t smem, cudaStream_t st) {
   const int pl = row_loss(LOSS) ? (int)ceil_div(a.mpad, 32) : 1;

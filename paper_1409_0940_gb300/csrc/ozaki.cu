@@ -593,7 +593,10 @@ cudaError_t factor_and_invert_sliced(const std::vector<MatJob>& jobs, bool inver
   // most SMs idle for half of its time, and step k of the forward sweep L Y = I needs only panel k:
   // with buffers for the factorisation's slices of its own, the two run side by side, the chain on a
   // stream of higher priority.  Four blocks of order 4096, set-up and first iteration: 52.3 -> 46.1
-  // ms; six of order 1000: 5.86 -> 5.44 ms.
+  // ms; six of order 1000: 5.86 -> 5.44 ms.  Measured down to the smallest order it applies to (65, one
+  // to 16 blocks, both precisions), the whole set-up with the stream, the event and the buffers opened
+  // for it: never slower (order 65: 0.572 -> 0.558 ms one block, 1.424 -> 1.405 sixteen; order 512: 1.67
+  // -> 1.45 and 3.26 -> 3.05).
   OzSide side;
   const size_t slice_bytes = round_up((int64_t)nj * S * rpad * 64 * 2, 1024), exp_bytes = round_up((int64_t)nj * rpad * 4, 1024);
   const bool beside = overlap && invert && nb > 1 && side.open(2 * (slice_bytes + exp_bytes), st);

@@ -544,7 +544,11 @@ cudaError_t split_gemm(const SgView& v) {
   // the pace of the copies: clusters share those jobs' stages, as many CTAs as fit side by side
   // (where a partial result fits the ring's memory).  A sweep of four solves (16 to 64 jobs of K =
   // 1024 or 2048, m = 8): 47 -> 24 us a product, 12.4 -> 11.5 ms over 10 iterations; 48 jobs of K =
-  // 1000: 50 iterations 17.7 -> 17.0 ms; the streamed passes of 40,000 rows at D = 8192, 2 x 2 (pass 2:
+  // 1000: 50 iterations 17.7 -> 17.0 ms.  A product's chains of round-toward-zero accumulations get as
+  // much shorter (K = 1024 over eight CTAs: emulated error 1.6e-6 -> 2.3e-7), so the solvers' errors
+  // against float64 fall (sweeps of four solves 6.0e-6 -> 4.4e-6, all outputs, eight inputs) except
+  // where the longer chain's bias happened to cancel another: the sweep's largest data set, D = 1024,
+  // 1.16e-6 -> 1.47e-6.  The streamed passes of 40,000 rows at D = 8192, 2 x 2 (pass 2:
   // 626 jobs on 304 slots): 10 iterations 14.2 -> 13.7 ms.
   const int64_t rest = v.njobs % slots, full = v.njobs - rest;
   int cl = 1;

@@ -15,7 +15,8 @@
 // holders give them back.  CTAs of two kernels that both held columns while they waited for the rest
 // of their clusters could wait for one another on two SMs without end.  So a CTA of a cluster gives
 // its columns back (tmem_return) before the first barrier of the cluster: whoever holds columns
-// finishes on its own, whatever else shares the SM.
+// finishes on its own, whatever else shares the SM.  (The tensor-core passes' CTA pairs hold theirs to
+// the end: no two of them fit an SM's shared memory.)
 #pragma once
 #include "common.cuh"
 #include "tcgen05.cuh"

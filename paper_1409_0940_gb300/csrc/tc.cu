@@ -155,8 +155,9 @@ __device__ __forceinline__ void red_add_v4(float4* p, float4 v) {
 // The epilogues' arithmetic, two elements per instruction: about 10 issue slots per cosine and split
 // instead of 17.  Eight warps leave little to hide behind, so every pass gains: a sweep of four
 // solves at d = 128, 553 -> 445 us per launch; 20,011 rows at d = 33, D = 3000, 96 -> 83 us; 200,000
-// rows at d = 440, D = 16,384, 147 classes, 7.8 -> 7.2 ms (1.68 PFLOP/s of products executed, at the
-// power cap: 0.96 of the sustained cuBLAS rate).  Sixteen warps of 32 columns gained
+// rows at d = 440, D = 16,384, 147 classes, 7.8 -> 7.2 ms at first (two iterations after a pause: 1.65 to
+// 1.72 PFLOP/s of products executed), 7.3 to 7.5 ms over 8 iterations and 7.6 to 7.7 over 30, once the
+// power cap holds: 1.56 PFLOP/s, 0.89 of the sustained cuBLAS rate.  Sixteen warps of 32 columns gained
 // at d = 33 only (17.5 against 17.9 ms a fit) and lost at d = 440 (142 against 139 ms, 8 iterations).
 // The phases added to an epilogue thread's accumulator columns: none (b is part of the product),
 // one (the feature index is the A row: pass 1), or one per column, from global memory.
@@ -234,6 +235,10 @@ static_assert(smem_bytes<64, 0, 1>() <= 232448 && smem_bytes<64, 1, 1>() <= 2324
                   smem_bytes<64, 1, 2>() <= 232448 && smem_bytes<32, 1, 2>() <= 232448 &&
                   smem_bytes<64, 2, 2>() <= 232448 && smem_bytes<32, 2, 2>() <= 232448,
               "every ring geometry fits the 227 KB of shared memory a CTA may use");
+// (a pair's CTAs hold their tensor memory while they wait for each other: see simt.cuh)
+static_assert(2 * smem_bytes<64, 1, 2>() > 233472 && 2 * smem_bytes<32, 1, 2>() > 233472 &&
+                  2 * smem_bytes<64, 2, 2>() > 233472 && 2 * smem_bytes<32, 2, 2>() > 233472,
+              "CTAs of two pairs never share an SM");
 
 // one poll of an mbarrier (acquire at cluster scope when the CTA pair shares it)
 template <int CG>
