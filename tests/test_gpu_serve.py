@@ -150,3 +150,32 @@ def test_cancel_queued_request(rff):
     with pytest.raises(rff.RffError):
         rff.rff_server_get_weights(srv, b, np.empty((256, 1), np.float32))
     rff.rff_server_destroy(srv)
+
+
+def test_cluster_kernels_of_several_solves_side_by_side(rff):
+    """Solves whose kernels run as clusters that take most of an SM's tensor memory (factor products
+    of 129 to 144 outputs, FP32 passes, split products of 17 to 32): at the same time, each gives
+    what it gives alone."""
+    specs = [("fp32", 700, 9, 140, 600, 1, 1), ("cached_z", 900, 20, 20, 700, 1, 2), ("fp32", 651, 40, 130, 1200, 5, 3),
+             ("cached_z", 2000, 12, 30, 900, 2, 2), ("split_bf16", 1200, 30, 100, 900, 1, 1)]
+    reqs = []
+    for k, (prec, n, d, m, D, R, C) in enumerate(specs):
+        X, Y = synth.multiclass(n=n, d=d, m=m, seed=k)
+        reqs.append((dict(loss="squared", reg="l2", prec=prec, lam=1e-3, sigma=3.0, D=D, R=R, C=C, seed=k, m=m), X, Y))
+    alone = []
+    for kw, X, Y in reqs:
+        s = rff.Solver(**kw)
+        s.set_data(X, Y)
+        s.solve(40, stats=False)
+        alone.append(s.weights())
+        s.close()
+    srv = rff.rff_server_create(0, len(reqs))
+    ids = [rff.rff_server_submit_solve(srv, rff.make_params(**kw), X, Y, 40) for kw, X, Y in reqs * 2]
+    got = _wait_all(rff, srv, ids)
+    assert all(c["status"] == rff.RFF_OK for c in got.values()), got
+    for k, rid in enumerate(ids):
+        kw = reqs[k % len(reqs)][0]
+        W = np.empty((kw["D"], kw["m"]), dtype=np.float32)
+        rff.rff_server_get_weights(srv, rid, W)
+        assert np.array_equal(W, alone[k % len(reqs)]), k
+    rff.rff_server_destroy(srv)
