@@ -1441,6 +1441,7 @@ SgView qgemm_view(const rff_admm_s& s) {
   v.two_acc = 1;
   v.bmask = s.act();
   v.accumulate = 1;   // W'_ij += Q_ij rhs_ij (the incremental projection)
+  v.centre = 1;
   v.kc = 64;          // the split inverses are zero past s_j columns
   v.st = s.st;        // one job per CTA: the hardware hands the 3.4 waves of jobs to whichever SM is free
   return v;

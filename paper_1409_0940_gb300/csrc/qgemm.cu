@@ -59,6 +59,8 @@ struct QArgs {
   const uint8_t* bmask;      // active blocks of a stochastic iteration, or null
   int accumulate;            // 1: out += result (amax of the sum)
   int cl;                    // CTAs (a cluster) that share a job's K stages
+  const __nv_bfloat16 *c_a, *c_b;   // leading terms of A and B where the chains are centred, or null
+  int64_t c_lda, c_ldb;
   int* err;
   long long timeout_cycles;
 };
@@ -92,6 +94,35 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
                : "memory");
   return v;
 }
+
+// Where a chain of accumulations starts.  The tensor cores' accumulator rounds toward zero, a bias in
+// proportion to the running sum.  A factor's product Q r is mostly cancellation (Q = (I + Z^T Z)^-1 takes
+// r's part along Z's large singular vectors down by their squares): row k's sum runs from 0 down to some
+// -Q_kk r_k times k's place, jumps by Q_kk r_k at k and falls back to about 0, and over the rows, whose
+// jumps lie anywhere, the bias cancels.  Cut into chains that start at 0, the one with the jump stays at
+// Q_kk r_k and the others run from 0 to a fraction of -Q_kk r_k: these biases differ by a tenth, a share of
+// r that Q should have taken out and that Z brings back enlarged.  So each chain starts at minus half of
+// what it will add (its share of -Q_kk r_k, and Q_kk r_k where it holds the jump), and over the rows
+// it lies on one side of 0 as much as on the other; what it started from is subtracted at the end.
+// Scores after two iterations (TensorSketch, degree 3, n = 2002, D = 4096, l1 loss, largest eigenvalue
+// 6e4), error against float64: one chain 2.6e-4, eight from 0 9.7e-4, eight from here 3.2e-4; where
+// little cancels the error is that of the short chains (binary fit of 20k rows 4.5e-6, 3.8e-6, 3.8e-6).
+struct ChainStart {   // of one output row
+  const __nv_bfloat16* r;   // B's leading term at the row's own feature, column 0 (null: start at 0)
+  int64_t ldr;
+  float w;                  // A's there, times the weight
+  __device__ __forceinline__ ChainStart(const SgJob& job, const QArgs& a, int row, int k0, int k1, int k_all)
+      : r(nullptr), ldr(a.c_ldb), w(0.f) {
+    if (!a.c_a) return;
+    // the A column, and K element, of the row's own feature
+    const int k = (int)(job.out / a.mpad - (int64_t)(job.b_row / a.mpad) * a.c_ldb - job.b_k0) + row;
+    if (k >= a.c_lda) return;   // a padding row
+    w = __bfloat162float(a.c_a[(job.a_row + row) * a.c_lda + job.a_k0 + k]) *
+        (0.5f * (float)(k1 - k0) / (float)k_all - (k >= k0 && k < k1 ? 0.5f : 0.f));
+    r = a.c_b + job.b_row * a.c_ldb + job.b_k0 + k;
+  }
+  __device__ __forceinline__ float operator()(int c) const { return r ? w * __bfloat162float(r[c * ldr]) : 0.f; }
+};
 
 // split-product order (A term, B term): exponents summing to at most 2^-16
 __host__ __device__ constexpr int prod_a(int p) { return p == 2 || p == 4 ? 1 : p == 5 ? 2 : 0; }
@@ -205,6 +236,11 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
           ok = false;
           break;
         }
+        // (one accumulator set: the second's barrier says that the chains' starts are in place)
+        if (NA == 3 && a.c_a && !qwait(bar_acce + 8, 0, sh, a)) {
+          ok = false;
+          break;
+        }
         fence_after();
         const uint32_t acc = tmem + buf * a.buf_cols;
         int s0, s1;
@@ -227,7 +263,7 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
               if (a.acc_b) {
                 // hi.hi alone in the first accumulator, the smaller products in the second
                 const uint32_t d = p == 0 ? acc : acc + a.acc_b;
-                mma_bf16(d, da, db, idesc, (kc > s0 || kk > 0 || p > 1) ? 1u : 0u);
+                mma_bf16(d, da, db, idesc, (kc > s0 || kk > 0 || p > 1 || (NA == 3 && p == 0 && a.c_a)) ? 1u : 0u);
               } else {
                 mma_bf16(acc, da, db, idesc, (kc > s0 || kk > 0 || p > 0) ? 1u : 0u);
               }
@@ -250,6 +286,24 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
     const int row = quarter * 32 + lane;
     uint32_t done_jobs = 0;
     float mx = 0.f;
+    if (NA == 3 && a.c_a) {
+      const SgJob job = a.jobs[job0];
+      if (!q_skip(job, a)) {
+        int s0, s1;
+        stages_of(job.nk, s0, s1);
+        const ChainStart start(job, a, row, s0 * KC, s1 * KC, job.nk * QKC);
+        for (int c = c_begin; c < c_end; c += 8) {
+          float o[8];
+#pragma unroll
+          for (int t = 0; t < 8; ++t) o[t] = start(c + t);
+          tmem_st8(tmem + ((uint32_t)(quarter * 32) << 16) + c, o);
+        }
+        tmem_wait_st();
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_acce + 8);
+      }
+    }
     for (int jx = job0; jx < a.njobs; jx += job_step) {
       const SgJob job = a.jobs[jx];
       if (q_skip(job, a)) continue;
@@ -268,6 +322,13 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
         if (a.acc_b) tmem_ld8(taddr + a.acc_b + c, s8);
         tmem_wait_ld();
         float x[8];
+        if (NA == 3 && a.c_a) {
+          int s0, s1;
+          stages_of(job.nk, s0, s1);
+          const ChainStart start(job, a, row, s0 * KC, s1 * KC, job.nk * QKC);
+#pragma unroll
+          for (int t = 0; t < 8; ++t) r8[t] = __float_as_uint(__uint_as_float(r8[t]) - start(c + t));
+        }
 #pragma unroll
         for (int t = 0; t < 8; ++t) x[t] = sc * (__uint_as_float(r8[t]) + __uint_as_float(s8[t]));
         if (a.cl > 1) {   // the ring is free: this job is the CTA's only one
@@ -546,9 +607,10 @@ cudaError_t split_gemm(const SgView& v) {
   // 1024 or 2048, m = 8): 47 -> 24 us a product, 12.4 -> 11.5 ms over 10 iterations; 48 jobs of K =
   // 1000: 50 iterations 17.7 -> 17.0 ms.  A product's chains of round-toward-zero accumulations get as
   // much shorter (K = 1024 over eight CTAs: emulated error 1.6e-6 -> 2.3e-7), so the solvers' errors
-  // against float64 fall (sweeps of four solves 6.0e-6 -> 4.4e-6, all outputs, eight inputs) except
-  // where the longer chain's bias happened to cancel another: the sweep's largest data set, D = 1024,
-  // 1.16e-6 -> 1.47e-6.  The streamed passes of 40,000 rows at D = 8192, 2 x 2 (pass 2:
+  // against float64 fall (60 drawn scoring cases 6.2e-6 -> 4.2e-6 in the geometric mean, sweeps of four
+  // solves 6.2e-6 -> 4.5e-6 over all outputs), with the starts above also where a projection cancels;
+  // some single outputs rise where the longer chain's bias cancelled another one (the sweep's largest
+  // data set, D = 1024: 1.16e-6 -> 1.47e-6).  The streamed passes of 40,000 rows at D = 8192, 2 x 2 (pass 2:
   // 626 jobs on 304 slots): 10 iterations 14.2 -> 13.7 ms.
   const int64_t rest = v.njobs % slots, full = v.njobs - rest;
   int cl = 1;
@@ -561,6 +623,12 @@ cudaError_t split_gemm(const SgView& v) {
   }
   a.jobs = v.jobs + full;
   a.njobs = (int)rest;
+  if (v.centre && v.two_acc && v.na == 3) {
+    a.c_a = static_cast<const __nv_bfloat16*>(v.A[0]);
+    a.c_b = static_cast<const __nv_bfloat16*>(v.B[0]);
+    a.c_lda = v.a_cols;
+    a.c_ldb = v.b_cols;
+  }
   return run(rest, cl);
 }
 

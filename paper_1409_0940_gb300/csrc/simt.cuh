@@ -60,11 +60,7 @@ __device__ __forceinline__ uint32_t park_base(uint32_t tmem, uint32_t cols) {
   const uint32_t w = threadIdx.x / 32;
   return tmem + ((w & 3) << 21) + (w >> 2) * (cols / 2);
 }
-__device__ __forceinline__ void park8(uint32_t taddr, const float (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "f"(v[0]),
-               "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
-               : "memory");
-}
+__device__ __forceinline__ void park8(uint32_t taddr, const float (&v)[8]) { tc5::tmem_st8(taddr, v); }
 __device__ __forceinline__ void unpark8(uint32_t taddr, float (&v)[8]) {   // complete after tmem_wait_ld
   uint32_t r[8];
   tc5::tmem_ld8(taddr, r);
