@@ -411,19 +411,25 @@ __global__ void k_to_pairs(const GemmDesc* __restrict__ descs) {
 // wait in tensor memory between folds.  Against 128 x 64 tiles of 8 x 4 outputs with the
 // accumulator in registers (238 of them, one CTA of eight warps): the 256 blocks of
 // 625 rows x 4096 features of a 32 x 8 grid 86 ms in 512 launches -> 15.3 ms in 16 (34 TFLOP/s).
-constexpr int GR_T = 128, GR_K = 32, GR_NS = 4;
+// cl = GR_CL: the rows are shared by a cluster of GR_CL CTAs, whole runs of 64 each, whose float-float
+// sums are added in order through distributed shared memory.  Few tiles leave most SMs idle for as
+// long as a CTA takes for all rows: the set-up of 60,000 rows in 2 blocks at D = 300 (6 tiles) 7.3 ->
+// 1.7 ms (5.8 with 128 x 64 tiles), at D = 1000 9.2 -> 5.2 (8.5), four blocks of 1024 30.0 -> 14.0 (24.4)
+constexpr int GR_T = 128, GR_K = 32, GR_NS = 4, GR_CL = 8;
 constexpr size_t GR_SMEM = (size_t)GR_NS * 2 * GR_K * GR_T * 4;
+static_assert((size_t)2 * GR_T * GR_T * 4 <= GR_SMEM, "a tile's float-float sums fit the ring's memory");
 
 __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ Zall, int64_t ldz, int64_t n,
                                                       const int64_t* __restrict__ slot,
                                                       const int64_t* __restrict__ size, int64_t s_one,
-                                                      double* __restrict__ Hall, int64_t h_stride) {
+                                                      double* __restrict__ Hall, int64_t h_stride, int cl) {
   using namespace simt;
+  const int rank = cl > 1 ? (int)tc5::cluster_rank() : 0, tile = (int)blockIdx.x / cl;
   // tile (ta, tb), tb <= ta, of the lower triangle
-  int ta = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
-  while (ta * (ta + 1) / 2 > (int)blockIdx.x) --ta;
-  while ((ta + 1) * (ta + 2) / 2 <= (int)blockIdx.x) ++ta;
-  const int64_t a0 = (int64_t)ta * GR_T, b0 = ((int64_t)blockIdx.x - (int64_t)ta * (ta + 1) / 2) * GR_T;
+  int ta = (int)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);
+  while (ta * (ta + 1) / 2 > tile) --ta;
+  while ((ta + 1) * (ta + 2) / 2 <= tile) ++ta;
+  const int64_t a0 = (int64_t)ta * GR_T, b0 = ((int64_t)tile - (int64_t)ta * (ta + 1) / 2) * GR_T;
   const int64_t s = size ? size[blockIdx.y] : s_one;
   if (a0 >= s) return;   // past this matrix
   const float* Z = Zall + (slot ? slot[blockIdx.y] - slot[0] : 0);
@@ -432,13 +438,15 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
   __shared__ uint32_t tmem_word;
   const int tid = threadIdx.x, tx = thread_tx(), ty = thread_ty();
   if (tid < 32) tc5::tmem_alloc<1>(tc5::smem_u32(&tmem_word), 512);
-  const int64_t nst = ceil_div(n, GR_K);
+  // stages st0 .. st1 of 32 rows, st0 even (sums are folded after every second one)
+  const int64_t runs = ceil_div(n, 2 * GR_K);
+  const int64_t st0 = 2 * (rank * runs / cl), st1 = min(ceil_div(n, GR_K), 2 * ((rank + 1) * runs / cl));
   // this thread's four columns of either operand: zeros past the matrix (rows are padded to 16 bytes)
   const int c4 = 4 * (tid % 32);
   const bool a_in = a0 + c4 < s, b_in = b0 + c4 < s;
   const int64_t a_col = a_in ? a0 + c4 : 0, b_col = b_in ? b0 + c4 : 0;
   auto issue = [&](int64_t st) {
-    if (st < nst) {
+    if (st < st1) {
       float* As = gr_smem + (st % GR_NS) * (2 * GR_K * GR_T);
       float* Bs = As + GR_K * GR_T;
 #pragma unroll
@@ -453,7 +461,7 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
     cp_commit();
   };
 #pragma unroll
-  for (int st = 0; st < GR_NS - 1; ++st) issue(st);
+  for (int st = 0; st < GR_NS - 1; ++st) issue(st0 + st);
   tc5::fence_before();
   __syncthreads();
   tc5::fence_after();
@@ -466,7 +474,7 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
 #pragma unroll
   for (int i = 0; i < 16; ++i) park8(park + 8 * i, acc[0]);
   tc5::tmem_wait_st();
-  for (int64_t st = 0; st < nst; ++st) {
+  for (int64_t st = st0; st < st1; ++st) {
     cp_wait<GR_NS - 2>();
     __syncthreads();   // stage st has landed; everyone is done with stage st - 1
     issue(st + GR_NS - 1);
@@ -485,7 +493,7 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
-    if ((st & 1) || st + 1 == nst) {   // every 64 rows: fold the partial sums into hi + lo
+    if ((st & 1) || st + 1 == st1) {   // every 64 rows: fold the partial sums into hi + lo
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         float hi[8], lo[8];
@@ -502,19 +510,50 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
       tc5::tmem_wait_st();
     }
   }
+  if (cl == 1) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float hi[8], lo[8];
-    unpark8(park + 16 * i, hi);
-    unpark8(park + 16 * i + 8, lo);
-    const int64_t gm = a0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
+    for (int i = 0; i < 8; ++i) {
+      float hi[8], lo[8];
+      unpark8(park + 16 * i, hi);
+      unpark8(park + 16 * i + 8, lo);
+      const int64_t gm = a0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t gn = b0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
-      if (gm < s && gn < s) H[gm * s + gn] += (double)hi[j] + (double)lo[j];
+      for (int j = 0; j < 8; ++j) {
+        const int64_t gn = b0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
+        if (gm < s && gn < s) H[gm * s + gn] += (double)hi[j] + (double)lo[j];
+      }
     }
+    tmem_return(tmem_word, 512);
+  } else {
+    cp_wait<0>();      // (only empty groups are left)
+    __syncthreads();   // everyone is done reading the ring
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float v[8];
+      float* row = gr_smem + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4) * GR_T;
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {   // the sums, then their low parts
+        unpark8(park + 16 * i + 8 * part, v);
+        *reinterpret_cast<float4*>(row + part * GR_T * GR_T + tx * 4) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(row + part * GR_T * GR_T + 64 + tx * 4) = make_float4(v[4], v[5], v[6], v[7]);
+      }
+    }
+    tmem_return(tmem_word, 512);   // before the cluster is waited for
+    tc5::cluster_sync_all();
+    constexpr int SHARE = GR_T * GR_T / GR_CL;
+    const uint32_t base = tc5::smem_u32(gr_smem);
+    for (int e = rank * SHARE + tid; e < (rank + 1) * SHARE; e += 256) {
+      float th = ld_cluster(base + 4 * e, 0), tl = ld_cluster(base + 4 * (GR_T * GR_T + e), 0);
+#pragma unroll
+      for (int r = 1; r < GR_CL; ++r) {
+        two_sum_into(th, tl, ld_cluster(base + 4 * e, r));
+        tl = __fadd_rn(tl, ld_cluster(base + 4 * (GR_T * GR_T + e), r));
+      }
+      const int64_t gm = a0 + e / GR_T, gn = b0 + e % GR_T;
+      if (gm < s && gn < s) H[gm * s + gn] += (double)th + (double)tl;
+    }
+    tc5::cluster_sync_all();   // nobody leaves while others read its shared memory
   }
-  tmem_return(tmem_word, 512);
 }
 
 // ------------------------------------------------------------------ diagonal potrf
@@ -750,9 +789,26 @@ cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, const
   const int64_t nt = ceil_div(s_max, GR_T);
   const cudaError_t e = cudaFuncSetAttribute(k_gram_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GR_SMEM);
   if (e != cudaSuccess) return e;
-  k_gram_tile<<<dim3((unsigned)(nt * (nt + 1) / 2), (unsigned)nb), 256, GR_SMEM, st>>>(Z, ldz, n, slot, size, s_max, H,
-                                                                                       h_stride);
-  return cudaGetLastError();
+  // One CTA per tile, or a cluster sharing its rows where that ends sooner (waves times stages per CTA, four
+  // for filling the ring and, in a cluster, six more for the exchange; clusters of eight leave about an
+  // eighth of the SMs unused).  One matrix only: how many are launched together may depend on the
+  // memory there is, which must not show in the sums.
+  const int64_t tiles = nt * (nt + 1) / 2, nst = ceil_div(n, GR_K), nsm = device_sms();
+  const int64_t whole = ceil_div(tiles, nsm) * (nst + 4);
+  const int64_t shared = ceil_div(tiles * GR_CL, nsm * 7 / 8) * (ceil_div(nst, GR_CL) + 10);
+  const int cl = !size && nb == 1 && shared < whole ? GR_CL : 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(tiles * cl), (unsigned)nb);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = GR_SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_gram_tile, Z, ldz, n, slot, size, s_max, H, h_stride, cl);
 }
 
 cudaError_t launch_zero_strict_upper(double* A, int64_t s, int nbatch, cudaStream_t st) {

@@ -157,7 +157,7 @@ cudaError_t launch_to_pairs(const GemmDesc* descs_dev, int nbatch, int maxM, int
 // Gram: H_b (FP64, s_b x s_b, ld s_b; 128 x 128 tiles on or below the diagonal) += A_b^T A_b for the
 // nb matrices A_b = Z[0..n) x [slot[b] - slot[0], + size[b]) (FP32, row-major, ld ldz), H_b h_stride
 // apart; slot and size on the device (slots are multiples of 128), s_max the largest size; or
-// one matrix with slot = size = null, s = s_max.  FP32 products, float-float sums.  ldz % 4 == 0
+// one matrix with slot = size = null, s = s_max (its rows may be shared by clusters).  FP32 products, float-float sums.  ldz % 4 == 0
 // and Z holds round_up(s, 4) columns per matrix (those past s_b are read, not used)
 cudaError_t launch_gram_f32_to_f64(const float* Z, int64_t ldz, int64_t n, const int64_t* slot, const int64_t* size,
                                    int64_t s_max, int nb, double* H, int64_t h_stride, cudaStream_t st);

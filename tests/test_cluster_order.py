@@ -33,4 +33,4 @@ def test_tensor_memory_is_given_back_before_a_cluster_is_waited_for():
         before = [m.start() for m in RELEASE.finditer(body) if m.start() < barrier.start()]
         after = [m.start() for m in RELEASE.finditer(body) if m.start() > barrier.start()]
         assert before and not after, (path, name)
-    assert sorted(seen) == ["k_gemm_f32_nn", "k_pass2_simt", "k_split_gemm"]
+    assert sorted(seen) == ["k_gemm_f32_nn", "k_gram_tile", "k_pass2_simt", "k_split_gemm"]
