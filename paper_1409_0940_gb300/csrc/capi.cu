@@ -2397,7 +2397,6 @@ rff_status rff_admm_predict(rff_admm_t h, const float* Xq, int64_t q, float* sco
   float* sc = reinterpret_cast<float*>(xl + chunk * s.dld);
   float* part = partb ? sc + chunk * s.mpad : nullptr;
   const cudaMemcpyKind kin = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  const cudaMemcpyKind kout = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   for (int64_t q0 = 0; q0 < q; q0 += chunk) {
     const int64_t nq = std::min(chunk, q - q0), nqp = round_up(nq, SLOT);
     CK(cudaMemcpyAsync(stage, Xq + q0 * s.d, nq * s.d * 4, kin, s.st));
@@ -2411,16 +2410,22 @@ rff_status rff_admm_predict(rff_admm_t h, const float* Xq, int64_t q, float* sco
     if (s.tc_scores()) CK(launch_split_f16(xq32, nqp * s.dld, s.xscale, xh, xl, s.st));
     if ((r = scores_pass(h, xq32, xh, xl, nqp, nullptr, sc, part, partb)) != RFF_OK) return r;
     // The check's outcome is read with the scores formed, not before: waiting for it in front of a
-    // dozen launches left the GPU idle while they were made.  Refused queries leave `scores` alone.
+    // dozen launches left the GPU idle while they were made.  Refused queries leave `scores` alone: on
+    // the device the copy looks at the outcome itself, so that one wait is enough; to the host it waits
+    // for it.
+    if (is_device_ptr)
+      CK(launch_copy_scores(sc, (int)s.mpad, nq, (int)s.m, scores + q0 * s.m, s.flag,
+                            s.tc_scores() ? 32768.f / s.xscale : INFINITY, s.st));
     int fl[3] = {0, 0, 0};
     CK(cudaMemcpyAsync(fl, s.flag, 12, cudaMemcpyDeviceToHost, s.st));
     CK(cudaStreamSynchronize(s.st));
     if (fl[0] & 1) return h->fail(RFF_EINVAL, "queries contain NaN or Inf");
     if (fl[0] & 4) return h->fail(RFF_EINVAL, "the random Laplace map takes nonnegative queries");
     if ((r = check_query_range(h, fl[2])) != RFF_OK) return r;
-    CK(cudaMemcpy2DAsync(scores + q0 * s.m, s.m * 4, sc, s.mpad * 4, s.m * 4, nq, kout, s.st));
+    if (!is_device_ptr)
+      CK(cudaMemcpy2DAsync(scores + q0 * s.m, s.m * 4, sc, s.mpad * 4, s.m * 4, nq, cudaMemcpyDeviceToHost, s.st));
   }
-  CK(cudaStreamSynchronize(s.st));
+  if (!is_device_ptr) CK(cudaStreamSynchronize(s.st));
   return RFF_OK;
 }
 

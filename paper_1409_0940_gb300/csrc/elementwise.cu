@@ -821,6 +821,15 @@ __global__ void __launch_bounds__(256) k_finite(const float* __restrict__ x, int
   }
 }
 
+// dst (rows x m) = src (ld mpad), unless the check of the queries refused them: flag[0] has a bit set,
+// or max |x| (float bits in flag[2]) is not below limit
+__global__ void k_copy_scores(const float* __restrict__ src, int mpad, int64_t rows, int m, float* __restrict__ dst,
+                              const int* __restrict__ flag, float limit) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= rows * m || flag[0] != 0 || !(__int_as_float(flag[2]) < limit)) return;
+  dst[t] = src[t / m * mpad + t % m];
+}
+
 inline unsigned nblk(int64_t n, int bs = 256) { return (unsigned)ceil_div(n, bs); }
 
 }  // namespace
@@ -1081,6 +1090,13 @@ __global__ void k_argmax_rows(const float* __restrict__ S, int64_t q, int m, int
 cudaError_t launch_argmax_rows(const float* scores, int64_t q, int m, int64_t ld, int32_t* labels, cudaStream_t st) {
   if (q <= 0) return cudaSuccess;
   k_argmax_rows<<<nblk(q * 32), 256, 0, st>>>(scores, q, m, ld, labels);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_copy_scores(const float* src, int mpad, int64_t rows, int m, float* dst, const int* flag,
+                               float limit, cudaStream_t st) {
+  if (rows <= 0) return cudaSuccess;
+  k_copy_scores<<<nblk(rows * m), 256, 0, st>>>(src, mpad, rows, m, dst, flag, limit);
   return cudaGetLastError();
 }
 

@@ -281,6 +281,10 @@ cudaError_t launch_loss_partials(int loss, const float* Y, const float* S, const
                                  int m, int mpad, double* partials, int nblocks, cudaStream_t st);
 cudaError_t launch_reg_partials(int reg, const float* W, int64_t n, double* partials, int nblocks, cudaStream_t st,
                                 const float* w = nullptr, int ncol = 1);
+// dst (rows x m) = the first m columns of src (ld mpad) if flag[0] == 0 and the maximum in flag[2] (float
+// bits) is below limit
+cudaError_t launch_copy_scores(const float* src, int mpad, int64_t rows, int m, float* dst, const int* flag,
+                               float limit, cudaStream_t st);
 // flag |= 1 for NaN/Inf; pm1 = 1: |= 2 for a value other than +-1; pm1 = 2: |= 4 for a negative value
 cudaError_t launch_finite_check(const float* x, int64_t n, int pm1, int* flag, cudaStream_t st,
                                 unsigned* maxbits = nullptr);

@@ -63,3 +63,44 @@ def test_tiny_scores_do_not_depend_on_the_batch(rff, prec, scale):
     split = 4 * np.sqrt(ref.size / 3.0) * 2.0 ** -133
     assert np.linalg.norm(full[:50].astype(np.float64) - ref) <= 1e-4 * np.linalg.norm(ref) + split
     s.close()
+
+
+# refused queries leave the caller's scores alone, on the device (where the copy out looks at the
+# check's outcome itself) and on the host
+@pytest.mark.parametrize("prec,fmap", [("split_bf16", "fourier"), ("fp32", "laplace"), ("cached_z", "tensorsketch")])
+@pytest.mark.parametrize("where", ["device", "host"])
+def test_refused_queries_leave_the_scores_alone(rff, prec, fmap, where):
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(3)
+    X = rng.random((300, 7)).astype(np.float32)
+    Y = np.sign(rng.standard_normal((300, 2))).astype(np.float32)
+    s = rff.Solver(loss="squared", lam=1e-3, sigma=2.0, D=200, R=1, C=2, seed=9, m=2, prec=prec, feature_map=fmap)
+    s.set_data(X, Y)
+    s.solve(2)
+    good = rng.random((200, 7)).astype(np.float32)
+    want = s.predict(good)
+    bad = {"nan": np.nan}
+    if prec == "split_bf16":
+        bad["range"] = 1e30      # beyond the FP16 split's range
+    if fmap == "laplace":
+        bad["negative"] = -1.0
+
+    def call(Q):
+        out = np.full((200, 2), 7.0, np.float32)
+        if where == "host":
+            return out, lambda: s.predict(Q, out), lambda: out
+        q, o = torch.from_numpy(Q).cuda(), torch.from_numpy(out).cuda()
+        return out, lambda: s.predict(q, o), lambda: o.cpu().numpy()
+
+    for value in bad.values():
+        Q = good.copy()
+        Q[150, 3] = value
+        before, run, after = call(Q)
+        with pytest.raises(rff.RffError) as e:
+            run()
+        assert e.value.status == rff.RFF_EINVAL
+        assert np.array_equal(after(), np.full((200, 2), 7.0, np.float32))
+    _, run, after = call(good)
+    run()
+    assert np.array_equal(after(), want)
+    s.close()
