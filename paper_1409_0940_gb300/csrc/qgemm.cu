@@ -107,21 +107,44 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
 // Scores after two iterations (TensorSketch, degree 3, n = 2002, D = 4096, l1 loss, largest eigenvalue
 // 6e4), error against float64: one chain 2.6e-4, eight from 0 9.7e-4, eight from here 3.2e-4; where
 // little cancels the error is that of the short chains (binary fit of 20k rows 4.5e-6, 3.8e-6, 3.8e-6).
-struct ChainStart {   // of one output row
-  const __nv_bfloat16* r;   // B's leading term at the row's own feature, column 0 (null: start at 0)
+struct ChainStart {   // of the 32 output rows of a writing warp, a row per lane
+  const __nv_bfloat16* r;   // B's leading term at the first row's own feature, column 0
   int64_t ldr;
-  float w;                  // A's there, times the weight
-  __device__ __forceinline__ ChainStart(const SgJob& job, const QArgs& a, int row, int k0, int k1, int k_all)
-      : r(nullptr), ldr(a.c_ldb), w(0.f) {
-    if (!a.c_a) return;
-    // the A column, and K element, of the row's own feature
-    const int k = (int)(job.out / a.mpad - (int64_t)(job.b_row / a.mpad) * a.c_ldb - job.b_k0) + row;
-    if (k >= a.c_lda) return;   // a padding row
-    w = __bfloat162float(a.c_a[(job.a_row + row) * a.c_lda + job.a_k0 + k]) *
-        (0.5f * (float)(k1 - k0) / (float)k_all - (k >= k0 && k < k1 ? 0.5f : 0.f));
-    r = a.c_b + job.b_row * a.c_ldb + job.b_k0 + k;
+  float w;                  // A's leading term at this lane's own feature, times the weight
+  __device__ __forceinline__ ChainStart() : r(nullptr), ldr(0), w(0.f) {}
+  // row0: the warp's first row; the chain takes K elements k0 .. k1 of k_all
+  __device__ __forceinline__ ChainStart(const SgJob& job, const QArgs& a, int row0, int k0, int k1, int k_all)
+      : ldr(a.c_ldb), w(0.f) {
+    // the A column, and K element, of a row's own feature: out's row, counted from the job's first feature
+    // (m_pad is a multiple of 16, and a 16th of out's elements a 32-bit number)
+    const uint32_t out_row = (uint32_t)(job.out >> 4) / (uint32_t)(a.mpad >> 4);
+    const int first = (int)(out_row - (uint32_t)(job.b_row / a.mpad) * (uint32_t)a.c_ldb - (uint32_t)job.b_k0) + row0;
+    const int row = row0 + (int)(threadIdx.x & 31), k = first + (int)(threadIdx.x & 31);
+    r = a.c_b + job.b_row * a.c_ldb + job.b_k0 + first;
+    if (k < a.c_lda)   // (past it a padding row)
+      w = __bfloat162float(a.c_a[(job.a_row + row) * a.c_lda + job.a_k0 + k]) *
+          (0.5f * (float)(k1 - k0) / (float)k_all - (k >= k0 && k < k1 ? 0.5f : 0.f));
   }
-  __device__ __forceinline__ float operator()(int c) const { return r ? w * __bfloat162float(r[c * ldr]) : 0.f; }
+  // columns c .. c + 31, those below c_end (a multiple of 8): 8 columns of 32 rows at a time as one
+  // 16-byte load per lane, all in flight together, turned through the warp's 512 bytes of buf (a
+  // 2-byte load per row and column took 9 us of a product of 128 columns, these 4)
+  __device__ __forceinline__ void load(int c, int c_end, uint4* buf, float (&o)[32]) const {
+    const int lane = threadIdx.x & 31;
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      v[u] = c + 8 * u < c_end ? *reinterpret_cast<const uint4*>(r + (c + 8 * u + lane / 4) * ldr + 8 * (lane % 4))
+                               : make_uint4(0, 0, 0, 0);
+    const __nv_bfloat16* mine = reinterpret_cast<const __nv_bfloat16*>(buf) + lane;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      __syncwarp();
+      buf[lane] = v[u];
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < 8; ++t) o[8 * u + t] = w * __bfloat162float(mine[32 * t]);
+    }
+  }
 };
 
 // split-product order (A term, B term): exponents summing to at most 2^-16
@@ -286,22 +309,28 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
     const int row = quarter * 32 + lane;
     uint32_t done_jobs = 0;
     float mx = 0.f;
+    __shared__ uint4 turn[QEPI][32];   // (see ChainStart::load)
+    ChainStart start;
+    float o[32];   // the chains' starts of 32 columns
     if (NA == 3 && a.c_a) {
       const SgJob job = a.jobs[job0];
       if (!q_skip(job, a)) {
         int s0, s1;
         stages_of(job.nk, s0, s1);
-        const ChainStart start(job, a, row, s0 * KC, s1 * KC, job.nk * QKC);
-        for (int c = c_begin; c < c_end; c += 8) {
-          float o[8];
+        start = ChainStart(job, a, quarter * 32, s0 * KC, s1 * KC, job.nk * QKC);
+        for (int c = c_begin; c < c_end; c += 32) {
+          start.load(c, c_end, turn[warp - 2], o);
 #pragma unroll
-          for (int t = 0; t < 8; ++t) o[t] = start(c + t);
-          tmem_st8(tmem + ((uint32_t)(quarter * 32) << 16) + c, o);
+          for (int u = 0; u < 4; ++u) {
+            const float v[8] = {o[8 * u], o[8 * u + 1], o[8 * u + 2], o[8 * u + 3], o[8 * u + 4], o[8 * u + 5], o[8 * u + 6], o[8 * u + 7]};
+            if (c + 8 * u < c_end) tmem_st8(tmem + ((uint32_t)(quarter * 32) << 16) + c + 8 * u, v);
+          }
         }
         tmem_wait_st();
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_acce + 8);
+        if (c_end - c_begin > 32) start.load(c_begin, c_end, turn[warp - 2], o);   // again the first 32, before the products end
       }
     }
     for (int jx = job0; jx < a.njobs; jx += job_step) {
@@ -323,11 +352,13 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
         tmem_wait_ld();
         float x[8];
         if (NA == 3 && a.c_a) {
-          int s0, s1;
-          stages_of(job.nk, s0, s1);
-          const ChainStart start(job, a, row, s0 * KC, s1 * KC, job.nk * QKC);
+          const int at = c - c_begin;
+          if (at % 32 == 0 && at > 0) start.load(c, c_end, turn[warp - 2], o);
 #pragma unroll
-          for (int t = 0; t < 8; ++t) r8[t] = __float_as_uint(__uint_as_float(r8[t]) - start(c + t));
+          for (int t = 0; t < 8; ++t) {
+            const float v = (at & 16) ? ((at & 8) ? o[24 + t] : o[16 + t]) : ((at & 8) ? o[8 + t] : o[t]);
+            r8[t] = __float_as_uint(__uint_as_float(r8[t]) - v);
+          }
         }
 #pragma unroll
         for (int t = 0; t < 8; ++t) x[t] = sc * (__uint_as_float(r8[t]) + __uint_as_float(s8[t]));
