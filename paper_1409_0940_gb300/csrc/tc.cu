@@ -152,6 +152,18 @@ __device__ __forceinline__ void red_add_v4(float4* p, float4 v) {
                : "memory");
 }
 
+// row[0 .. half) += sc times the accumulator columns at taddr, by loads, additions and stores
+__device__ __noinline__ void add_rows_plain(uint32_t taddr, float* row, int half, float sc, const TcArgs& a) {
+  for (int c = 0; c < half; c += 8) {
+    uint32_t r8[8];
+    tmem_ld8(taddr + c, r8);
+    tmem_wait_ld();
+    if (!RFF_SPAN(row + c - a.out, 8, a.out_elems)) continue;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) row[c + t] = __fadd_rn(row[c + t], __fmul_rn(sc, __uint_as_float(r8[t])));
+  }
+}
+
 // The epilogues' arithmetic, two elements per instruction: about 10 issue slots per cosine and split
 // instead of 17.  Eight warps leave little to hide behind, so every pass gains: a sweep of four
 // solves at d = 128, 553 -> 445 us per launch; 20,011 rows at d = 33, D = 3000, 96 -> 83 us; 200,000
@@ -765,6 +777,9 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
             const float sc = a.scale / COS_SCALE * (a.m_amax ? f16_inv_scale(__uint_as_float(*a.m_amax)) : 1.f);
             float omx = 0.f;
             const bool add_rows = a.mode == MODE_PREDICT && !a.pred_part && g > 0;
+            if (add_rows && sc < RED_MIN_SC) {   // rare, and in a loop of its own
+              add_rows_plain(tmem + lane_addr + A2 + c0, orow + c0, half, sc, a);
+            } else
             for (int c = 0; c < half; c += 8) {
               uint32_t r8[8];
               tmem_ld8(tmem + lane_addr + A2 + c0 + c, r8);
@@ -775,15 +790,10 @@ __device__ __forceinline__ void regen_body(const TcArgs& a, const CtaPos& pos) {
               float4 v1 = make_float4(sc * __uint_as_float(r8[4]), sc * __uint_as_float(r8[5]),
                                       sc * __uint_as_float(r8[6]), sc * __uint_as_float(r8[7]));
               const bool in = RFF_SPAN(orow + c0 + c - a.out, 8, a.out_elems);
-              if (in && add_rows && sc >= RED_MIN_SC) {   // this thread wrote these values for the groups before
+              if (in && add_rows) {   // this thread wrote these values for the groups before
                 red_add_v4(dst, v0);
                 red_add_v4(dst + 1, v1);
               } else if (in) {
-                if (add_rows) {
-                  const float4 p0 = dst[0], p1 = dst[1];
-                  v0 = make_float4(p0.x + v0.x, p0.y + v0.y, p0.z + v0.z, p0.w + v0.w);
-                  v1 = make_float4(p1.x + v1.x, p1.y + v1.y, p1.z + v1.z, p1.w + v1.w);
-                }
                 dst[0] = v0;
                 dst[1] = v1;
               }
@@ -1144,6 +1154,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
             const float sc = a.scale / COS_SCALE * (a.m_amax ? f16_inv_scale(__uint_as_float(*a.m_amax)) : 1.f);
             float omx = 0.f;
             const bool add_rows = a.mode == MODE_PREDICT && !a.pred_part && g > 0;
+            if (add_rows && sc < RED_MIN_SC) {   // rare, and in a loop of its own
+              add_rows_plain(tmem + lane_addr + W_A2 + c0, orow + c0, half, sc, a);
+            } else
             for (int c = 0; c < half; c += 8) {
               uint32_t r8[8];
               tmem_ld8(tmem + lane_addr + W_A2 + c0 + c, r8);
@@ -1154,15 +1167,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_regen_wide(const __grid_constan
               float4 v1 = make_float4(sc * __uint_as_float(r8[4]), sc * __uint_as_float(r8[5]),
                                       sc * __uint_as_float(r8[6]), sc * __uint_as_float(r8[7]));
               const bool in = RFF_SPAN(orow + c0 + c - a.out, 8, a.out_elems);
-              if (in && add_rows && sc >= RED_MIN_SC) {
+              if (in && add_rows) {
                 red_add_v4(dst, v0);
                 red_add_v4(dst + 1, v1);
               } else if (in) {
-                if (add_rows) {
-                  const float4 p0 = dst[0], p1 = dst[1];
-                  v0 = make_float4(p0.x + v0.x, p0.y + v0.y, p0.z + v0.z, p0.w + v0.w);
-                  v1 = make_float4(p1.x + v1.x, p1.y + v1.y, p1.z + v1.z, p1.w + v1.w);
-                }
                 dst[0] = v0;
                 dst[1] = v1;
               }
