@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(256) k_gemm_f32_nn(const GemmDesc* __restrict_
         gm_smem[(GEMM_M + ty + 16 * i) * N + tx + 16 * q] = PARK ? l[i] : lo[PARK ? 0 : q][i];
       }
     }
-    if (PARK) tmem_return(tmem_word, gemm_tmem_cols(MQ));   // before the cluster is waited for
-    tc5::cluster_sync_all();
+    if (PARK) tmem_return_and_meet(tmem_word, gemm_tmem_cols(MQ));
+    else tc5::cluster_sync_all();
     constexpr int SHARE = GEMM_M * N / GEMM_CL;
     const uint32_t base = tc5::smem_u32(gm_smem);
     for (int e = rank * SHARE + tid; e < (rank + 1) * SHARE; e += 256) {
@@ -538,8 +538,7 @@ __global__ void __launch_bounds__(256, 1) k_gram_tile(const float* __restrict__ 
         *reinterpret_cast<float4*>(row + part * GR_T * GR_T + 64 + tx * 4) = make_float4(v[4], v[5], v[6], v[7]);
       }
     }
-    tmem_return(tmem_word, 512);   // before the cluster is waited for
-    tc5::cluster_sync_all();
+    tmem_return_and_meet(tmem_word, 512);
     constexpr int SHARE = GR_T * GR_T / GR_CL;
     const uint32_t base = tc5::smem_u32(gr_smem);
     for (int e = rank * SHARE + tid; e < (rank + 1) * SHARE; e += 256) {

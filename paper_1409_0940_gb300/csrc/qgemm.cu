@@ -396,16 +396,18 @@ __global__ void __launch_bounds__(QNT) k_split_gemm(const __grid_constant__ QArg
       if (lane == 0 && mx > 0.f) atomicMax(a.amax, __float_as_uint(mx));
     }
   }
-  // (the roles' single threads rejoin their warps; a cluster is waited for only afterwards, see simt.cuh)
+  // (the roles' single threads rejoin their warps; the columns go back before a cluster is waited for, see
+  // simt.cuh)
   __syncwarp();
   fence_before();
   __syncthreads();
   fence_after();
+  if (a.cl > 1) cluster_arrive();
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
   }
   if (a.cl > 1) {
-    cluster_sync_all();
+    cluster_wait();
     const SgJob job = a.jobs[job0];
     if (!q_skip(job, a)) {
       const int rows = 128 / a.cl, n4 = rows * a.mpad / 4;

@@ -465,8 +465,7 @@ __global__ void __launch_bounds__(NT, 1) k_pass2_simt(const __grid_constant__ Pa
         for (int i = 0; i < 8; ++i) smem[elems + chain_row(b.ty, i) * p.mpad + b.tx + 16 * q] = v[i];
       }
     }
-    tmem_return(tmem_word, 512);   // before the cluster is waited for
-    tc5::cluster_sync_all();
+    tmem_return_and_meet(tmem_word, 512);
     const int share = elems / cl;
     const uint32_t base = tc5::smem_u32(smem);
     for (int e = (int)rank * share + threadIdx.x; e < ((int)rank + 1) * share; e += NT) {

@@ -14,7 +14,7 @@
 // Clusters and tensor memory: a CTA whose columns are taken waits in tcgen05.alloc until their
 // holders give them back.  CTAs of two kernels that both held columns while they waited for the rest
 // of their clusters could wait for one another on two SMs without end.  So a CTA of a cluster gives
-// its columns back (tmem_return) before the first barrier of the cluster: whoever holds columns
+// its columns back before it first waits for the cluster (tmem_return_and_meet): whoever holds columns
 // finishes on its own, whatever else shares the SM.  (The tensor-core passes' CTA pairs hold theirs to
 // the end: no two of them fit an SM's shared memory.)
 #pragma once
@@ -75,6 +75,16 @@ __device__ __forceinline__ void tmem_return(uint32_t tmem, uint32_t cols) {
   __syncthreads();
   tc5::fence_after();
   if (threadIdx.x < 32) tc5::tmem_dealloc<1>(tmem, cols);
+}
+
+// the same, and the cluster is met: the columns go back while the others arrive
+__device__ __forceinline__ void tmem_return_and_meet(uint32_t tmem, uint32_t cols) {
+  tc5::fence_before();
+  __syncthreads();
+  tc5::fence_after();
+  tc5::cluster_arrive();
+  if (threadIdx.x < 32) tc5::tmem_dealloc<1>(tmem, cols);
+  tc5::cluster_wait();
 }
 
 __device__ __forceinline__ float ld_cluster(uint32_t addr, uint32_t rank) {   // a CTA's shared memory in the cluster
