@@ -127,7 +127,7 @@ struct ChainStart {   // of the 32 output rows of a writing warp, a row per lane
   }
   // columns c .. c + 31, those below c_end (a multiple of 8): 8 columns of 32 rows at a time as one
   // 16-byte load per lane, all in flight together, turned through the warp's 512 bytes of buf (a
-  // 2-byte load per row and column took 9 us of a product of 128 columns, these 4)
+  // 2-byte load per row and column took 14 us of a product of 128 columns, these 4)
   __device__ __forceinline__ void load(int c, int c_end, uint4* buf, float (&o)[32]) const {
     const int lane = threadIdx.x & 31;
     uint4 v[4];
