@@ -563,11 +563,11 @@ __device__ __forceinline__ void write_z_half(const ZArgs& p, Body<0>& b, const f
 }
 
 // Materialise Z (or Z^T) for rows [r0, r0 + nr) and feature slots [f0, f0 + nf) into
-// out (leading dimension ldo); one CTA per 128 rows x 256 features.
-__global__ void __launch_bounds__(NT, 1) k_write_z_simt(const __grid_constant__ ZArgs p) {
+// out (leading dimension ldo); one CTA per 128 rows x 128 `tiles` features (tiles = 1 or 2).
+__global__ void __launch_bounds__(NT, 1) k_write_z_simt(const __grid_constant__ ZArgs p, int tiles) {
   extern __shared__ __align__(16) float smem[];
-  const int64_t a0 = p.r0 + (int64_t)blockIdx.x * BM, b0 = p.f0 + (int64_t)blockIdx.y * 2 * BN;
-  const int wd = b0 - p.f0 + BN < p.nf ? 2 : 1;
+  const int64_t a0 = p.r0 + (int64_t)blockIdx.x * BM, b0 = p.f0 + (int64_t)blockIdx.y * tiles * BN;
+  const int wd = tiles == 2 && b0 - p.f0 + BN < p.nf ? 2 : 1;
   Body<0> b(smem, Operands{p.X + a0 * p.ldx, p.Gt, nullptr, p.bias, p.feat_ok, p.ldx, p.ldg, p.K, 0}, b0, make_walk(wd, 1, 0, 1));
   float acc[16][8];
   if (wd == 2) b.form_t<16>(acc);
@@ -659,7 +659,13 @@ cudaError_t launch_write_z_simt(const ZArgs& p, cudaStream_t st) {
   if (p.K % 4 || p.K < 1) return cudaErrorInvalidValue;
   const cudaError_t e = cudaFuncSetAttribute(k_write_z_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
   if (e != cudaSuccess) return e;
-  k_write_z_simt<<<dim3((unsigned)ceil_div(p.nr, BM), (unsigned)ceil_div(p.nf, 2 * BN)), NT, SMEM, st>>>(p);
+  // Two tiles of features to a CTA (the panel of X is read once for both: 20,000 rows at d = 200, 2048
+  // features 480 us), unless one each ends within a wave, where a pair is only the longer chain: 500 rows
+  // at d = 33, 1000 features 23.8 -> 13.5 us, 1000 rows at d = 200, 2048 features 54 -> 32.  At two
+  // waves of single tiles both are alike (5000 rows at d = 64, 512 features: 29 us as pairs).
+  const int64_t rows = ceil_div(p.nr, BM), cols = ceil_div(p.nf, BN);
+  const int tiles = rows * cols <= device_sms() ? 1 : 2;
+  k_write_z_simt<<<dim3((unsigned)rows, (unsigned)ceil_div(cols, tiles)), NT, SMEM, st>>>(p, tiles);
   return cudaGetLastError();
 }
 

@@ -158,3 +158,21 @@ def test_cholesky_of_tiny_and_huge_pivots(rff, e):
     rff.rff_cholesky_f64(At, info)
     assert info.item() == 0
     assert np.array_equal(At[0].cpu().numpy(), L)
+
+
+@pytest.mark.parametrize("nf", [1, 127, 129, 1000])
+@pytest.mark.parametrize("d", [1, 33, 70])
+def test_features_do_not_depend_on_the_number_of_rows(rff, d, nf):
+    """Few tiles go one to a block of threads, many two to one: every row has the same bits either way."""
+    import torch
+    n, few = 20100, 130   # 158 row tiles: pairs on any GPU of up to 157 SMs; 2 x 8 tiles: singles
+    g = torch.Generator(device="cuda").manual_seed(d)
+    X = torch.randn(n, d, device="cuda", generator=g)
+    full, part = torch.empty(n, nf, device="cuda"), torch.empty(few, nf, device="cuda")
+    rff.rff_features(X, 7, 1.5, nf, 0, nf, "fp32", full)
+    for lo in (0, n - few):
+        rff.rff_features(X[lo:lo + few].contiguous(), 7, 1.5, nf, 0, nf, "fp32", part)
+        assert torch.equal(part, full[lo:lo + few])
+    want = orff.features_block(X[n - few:].cpu().numpy(), 7, 1.5, nf, 0, nf)
+    # float32 dot products of length d and the float32 cosine (as the features against the oracle elsewhere)
+    assert np.abs(part.cpu().numpy() - want).max() < 1e-5 * max(1.0, np.sqrt(d / 16)) * np.sqrt(2.0 / nf)
